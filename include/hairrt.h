@@ -169,7 +169,8 @@ typedef struct hr_light {
  * overlapped hr_asset_update (the call before it) uses the fixed order and
  * leaves the schedule as it is, and so does HR_FLAG_FIXED_TILE_ORDER, which
  * traces every tile whole, in raster order.  Counting renders (HR_FLAG_COUNT,
- * hr_render_profile) always use the fixed order. */
+ * hr_render_profile) and frames with HR_FLAG_SHADOWS always use the fixed
+ * order. */
 #define HR_FLAG_FIXED_TILE_ORDER 8192u
 
 typedef struct hr_render_desc {

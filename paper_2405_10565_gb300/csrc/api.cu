@@ -757,7 +757,8 @@ static hr_status render_impl(hr_ctx* ctx, hr_asset* a, const hr_render_desc* des
   // far slower (animated frames through the C ABI: the frame kernel 1.3-2.0
   // instead of 0.82 ms), so such a frame keeps the fixed order and leaves the
   // schedule as it is.
-  if (!count && !(desc->flags & HR_FLAG_FIXED_TILE_ORDER) && ctx->prev_kind != kUpdateCall)
+  if (!count && !(desc->flags & (HR_FLAG_FIXED_TILE_ORDER | HR_FLAG_SHADOWS)) &&
+      ctx->prev_kind != kUpdateCall)
     HR_TRY(tile_schedule(ctx, a, fa, st));
   if (stats) HR_CUDA(ctx, cudaEventRecord(ctx->ev0, st));
   if (t_begin) HR_CUDA(ctx, cudaEventRecord(t_begin, st));

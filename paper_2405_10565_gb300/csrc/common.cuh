@@ -355,6 +355,10 @@ hr_status launch_frame(hr_ctx* ctx, const FrameArgs& fa, int precision, bool cou
                        float* rgb_dev, cudaStream_t st);
 hr_status launch_frame_shadow(hr_ctx* ctx, const FrameArgs& fa, int precision, bool count,
                        float* rgb_dev, cudaStream_t st);
+// Tiles of a frame with shadow rays by separate hit, light-path and shading
+// kernels; *left: tiles from *work on may be left for the one-kernel form.
+hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, const float4* rect,
+                               uint32_t* work, float* rgb, cudaStream_t st, bool* left);
 hr_status launch_samples(hr_ctx* ctx, const FrameArgs& fa, int precision, const uint32_t* sids,
                          uint32_t m, float* rad_dev, int32_t* hit_dev, cudaStream_t st);
 // IM(theta, beta) lookups at m device points (test export of the shading code)

@@ -39,6 +39,8 @@ __device__ __forceinline__ float3 operator*(float3 a, float s) { return f3(a.x *
 __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ float clampf(float x, float lo, float hi) { return fminf(fmaxf(x, lo), hi); }
 
+__device__ __forceinline__ float3 hit_point(const float3 o, const float3 d, float t) { return o + d * t; }
+
 // ------------------------------------------------------------------ geometry
 
 // ------------------------------------------------------------------ precision
@@ -830,15 +832,36 @@ __device__ __forceinline__ void shadow_path(const FrameArgs& fa, const float3 x,
   }
 }
 
+// Direction from x toward a light and its falloff E; the length of the light
+// path.
+__device__ __forceinline__ void light_dir(const float4 L, const float3 x, float3& wi, float& E) {
+  E = 1.f;
+  if (L.w == 0.f) {
+    wi = f3(L.x, L.y, L.z);
+  } else {
+    const float3 to = f3(L.x, L.y, L.z) - x;
+    const float dd = dot3(to, to);
+    const float id = rsqrtf(dd);
+    wi = to * id;
+    E = id * id;
+  }
+}
+__device__ __forceinline__ float path_length(const float4 L, float E) {
+  return L.w == 0.f ? kInf : sqrtf(1.f / E);
+}
+
 // Radiance of one hit toward -d (sum over lights of T f E cos(theta_i), T and
 // the spread of f from shadow_path when SHADOW (HR_FLAG_SHADOWS), else T = 1)
 // and its opacity (strand 1; thick hair 1 - exp(-2 r l n_tot / (pi a b))).
 // SHADOW is a template parameter so kernels without shadow rays carry none
-// of their registers.
-template <int PREC, bool COUNT, bool SHADOW = false>
+// of their registers.  With PATHS the light paths were walked before: light
+// l's (T, spread variance) is paths[l * path_stride].
+template <int PREC, bool COUNT, bool SHADOW = false, bool PATHS = false>
 __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, float t,
                                           const float3 o, const float3 d, float rgb[3],
-                                          float& alpha, Counts& cn) {
+                                          float& alpha, Counts& cn,
+                                          const float4* __restrict__ paths = nullptr,
+                                          size_t path_stride = 0) {
   const float4 aux = __ldg(fa.prim_aux + id);
   const float4 r2 = __ldg(fa.prim_xf + 3 * (size_t)id + 2);
   const float3 T = f3(r2.x, r2.y, r2.z) * rsqrtf(r2.x * r2.x + r2.y * r2.y + r2.z * r2.z);
@@ -849,7 +872,7 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
   const float th_o = asinf(so);
   const float3 wop = wo - T * so;
   const float nop = sqrtf(dot3(wop, wop));
-  const float3 x = o + d * t;
+  const float3 x = hit_point(o, d, t);
   const bool eth = aux.y > 0.f && !(fa.flags & HR_FLAG_SINGLE_ON_ETH);
   EthHit eh{0.f, 1.f, 0.f, 0.f};
   alpha = 1.f;
@@ -871,16 +894,8 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
   for (int l = 0; l < fa.lights.n; ++l) {
     const float4 L = fa.lights.xyzw[l];
     float3 wi;
-    float E = 1.f;
-    if (L.w == 0.f) {
-      wi = f3(L.x, L.y, L.z);
-    } else {
-      const float3 to = f3(L.x, L.y, L.z) - x;
-      const float dd = dot3(to, to);
-      const float id = rsqrtf(dd);
-      wi = to * id;
-      E = id * id;
-    }
+    float E;
+    light_dir(L, x, wi, E);
     const float si = clampf(dot3(wi, T), -1.f, 1.f);
     const float th_i = asinf(si);
     const float3 wip = wi - T * si;
@@ -890,9 +905,16 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
     float Tl[3] = {1.f, 1.f, 1.f}, sg2 = 0.f;
     if (SHADOW) {
       bool sok = true;
-      shadow_path<PREC, COUNT>(fa, x, wi, L.w == 0.f ? kInf : sqrtf(1.f / E),
-                               __float_as_uint(aux.x), Tl, sg2, sok, cn);
+      shadow_path<PREC, COUNT>(fa, x, wi, path_length(L, E), __float_as_uint(aux.x), Tl, sg2, sok,
+                               cn);
       if (!sok) atomicAdd(fa.overflow, 1u);
+    }
+    if (PATHS) {
+      const float4 path = __ldg(paths + l * path_stride);
+      Tl[0] = path.x;
+      Tl[1] = path.y;
+      Tl[2] = path.z;
+      sg2 = path.w;
     }
     float f[3];
     if (eth) {

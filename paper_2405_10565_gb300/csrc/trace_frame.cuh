@@ -257,9 +257,10 @@ hr_status launch_k(hr_ctx* ctx, const FrameArgs& fa, bool count, float* rgb, cud
   HR_TRY(scratch(ctx, 47, 2 * sizeof(float4), (void**)&rect));
   uint32_t* work = reinterpret_cast<uint32_t*>(rect + 1);
   HR_CUDA(ctx, cudaMemsetAsync(rgb, 0, (size_t)fa.cam.W * fa.cam.H * 3 * sizeof(float), st));
-  // the counting kernel keeps the plain hand-out order (its tile log is indexed by it)
+  // the counting kernel keeps the plain hand-out order (its tile log is indexed
+  // by it), and so do frames with shadow rays
   FrameArgs f = fa;
-  if (count) f.sched = nullptr;
+  if (count || SHADOW) f.sched = nullptr;
   f.frame_warps = (uint32_t)frame_grid<KMAX, PREC, false, SHADOW>() * (kBlock / 32);
   k_scene_rect<<<1, kRectThreads, 0, st>>>(f, rect, work);
   HR_LAUNCHED(ctx);
@@ -267,8 +268,13 @@ hr_status launch_k(hr_ctx* ctx, const FrameArgs& fa, bool count, float* rgb, cud
     const int g = (int)std::min<uint32_t>(tiles, frame_grid<KMAX, PREC, true, SHADOW>());
     k_frame<KMAX, PREC, true, SHADOW><<<g, kBlock, 0, st>>>(f, rect, work, rgb);
   } else {
+    if (SHADOW) {  // the one-kernel form takes what the rounds leave over
+      bool left = true;
+      HR_TRY(launch_shadow_rounds(ctx, f, PREC, rect, work, rgb, st, &left));
+      if (!left) return HR_OK;
+    }
     const int g = (int)std::min<uint32_t>(tiles, frame_grid<KMAX, PREC, false, SHADOW>());
-    k_frame<KMAX, PREC, false, SHADOW><<<g, kBlock, 0, st>>>(fa, rect, work, rgb);
+    k_frame<KMAX, PREC, false, SHADOW><<<g, kBlock, 0, st>>>(f, rect, work, rgb);
   }
   HR_LAUNCHED(ctx);
   return HR_OK;

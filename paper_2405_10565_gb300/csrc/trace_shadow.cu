@@ -1,0 +1,275 @@
+// Frames with dual-scattering light paths (HR_FLAG_SHADOWS) in three kernels
+// a round: the primary rays and their hits, one light path per (hit, light),
+// and the shading of the hits with the paths' transmittances.
+//
+// A light path is a whole BVH walk (the full-head frame makes 840 node visits
+// a traced sample for its eight lights, 46 for the primary ray).  Walked
+// inside the shading loop they run one after the other per sample, so a frame
+// lasts as long as the tile whose lanes walk the most, at the few warps that a
+// kernel holding the primary ray's and the shading's state can keep resident:
+// 14.2 ms for 100k strands at 1920 x 1080, 8 spp, 8 lights, at a tenth of the
+// close view's visits per second.  As independent walks of a lean kernel, 32
+// neighbouring hits toward one light per warp, they fill the GPU.
+//
+// The hits of a round go to a buffer of at most kPathBudget light paths; the
+// primary kernel stops taking tiles once it is full and the next round goes on
+// from there.  The host does not know how many rounds a frame needs without
+// waiting for it, so it launches up to kMaxRounds and, when the worst case
+// would need more, the one-kernel form for whatever tiles are left.
+#include <algorithm>
+
+#include "trace_frame.cuh"
+
+namespace hr {
+namespace {
+
+constexpr uint64_t kPathBudget = 1ull << 24;  // 256 MB of path records
+constexpr uint32_t kMaxRounds = 3;
+
+struct ShadowTile {
+  uint32_t tile;      // index in the frame's warp grid
+  uint32_t base;      // first hit of the tile
+  uint32_t cnt[8];    // hits of each lane, eight bits each
+};
+
+struct ShadowWork {
+  uint32_t* ctr;      // [0] hits, [1] tiles with hits (of the round)
+  float4* hit;        // [cap] hit position and entry word (id, flags)
+  float* depth;       // [cap] depth past the re-based origin
+  ShadowTile* tiles;  // [cap]
+  float4* path;       // [lights][cap] (T rgb, spread variance)
+  uint32_t stop;      // no further tile is taken at this many hits
+  uint32_t cap;       // stop plus what the warps at work can still add
+};
+
+// Primary rays of the tiles handed out; every hit that shading can reach (up
+// to the first opaque one) is listed, a tile's hits together and in lane
+// order.
+template <int KMAX>
+__global__ void __launch_bounds__(kBlock, 4)
+    k_shadow_hits(const FrameArgs fa, const float4* __restrict__ rect_p, uint32_t* work,
+                  const ShadowWork sw) {
+  const float4 rect = *rect_p;
+  const WarpGrid g = warp_grid(rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
+  const uint32_t lane = threadIdx.x & 31, G = fa.grp;
+  bool overflow = false;
+  for (;;) {
+    uint32_t t = 0xffffffffu;
+    if (lane == 0 && __ldcg(sw.ctr) < sw.stop) t = atomicAdd(work, 1u);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    if (t >= g.n) break;
+    const uint32_t p = lane / G;
+    const uint32_t x = g.x0 + (t % g.nx) * g.wtw + p % g.wtw;
+    const uint32_t y = g.y0 + (t / g.nx) * g.wth + p / g.wtw;
+    const bool inside = x < (uint32_t)fa.cam.W && y < (uint32_t)fa.cam.H &&
+                        (float)x + 1.f >= rect.x && (float)x <= rect.z &&
+                        (float)y + 1.f >= rect.y && (float)y <= rect.w;
+    const uint64_t pixel = (uint64_t)y * (uint32_t)fa.cam.W + x;
+    const uint32_t s = lane & (G - 1);
+    tr::KBuf<KMAX> kb;
+    float3 o, d;
+    uint32_t cnt = 0;
+    if (inside && s < fa.spp) {
+      tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
+      tr::RayKey rk;
+      tr::primary_ray(fa, pixel * fa.spp + s, o, d, rk);
+      overflow |= !tr::traverse<KMAX, false>(fa, rk, o, d, kb, cn);
+      bool past = false;
+#pragma unroll
+      for (int j = 0; j < KMAX; ++j)
+        if (j < (int)fa.k && kb.t[j] < kInf && !past) {
+          ++cnt;
+          past = (kb.id[j] & tr::kOpaque) != 0u;
+        }
+    }
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, q);
+      if (lane >= (uint32_t)q) incl += v;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (!total) continue;  // background: the image is cleared
+    uint32_t base = 0, rec = 0;
+    if (lane == 0) {
+      base = atomicAdd(sw.ctr, total);
+      rec = atomicAdd(sw.ctr + 1, 1u);
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    rec = __shfl_sync(0xffffffffu, rec, 0);
+    if (lane == 0) {
+      sw.tiles[rec].tile = t;
+      sw.tiles[rec].base = base;
+    }
+    reinterpret_cast<uint8_t*>(sw.tiles[rec].cnt)[lane] = (uint8_t)cnt;
+    const uint32_t h0 = base + incl - cnt;
+#pragma unroll
+    for (int j = 0; j < KMAX; ++j)
+      if (j < (int)cnt) {
+        const float3 x3 = tr::hit_point(o, d, kb.t[j]);
+        sw.hit[h0 + j] = make_float4(x3.x, x3.y, x3.z, __uint_as_float(kb.id[j]));
+        sw.depth[h0 + j] = kb.t[j];
+      }
+  }
+  if (overflow) atomicAdd(fa.overflow, 1u);
+}
+
+// The light paths: a warp takes 32 consecutive hits and one light.
+template <int PREC>
+__global__ void __launch_bounds__(kBlock) k_shadow_paths(const FrameArgs fa, const ShadowWork sw) {
+  const uint32_t n = *sw.ctr, L = (uint32_t)fa.lights.n;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t tasks = (uint64_t)((n + 31) / 32) * L;
+  const uint64_t warps = (uint64_t)gridDim.x * (kBlock / 32);
+  for (uint64_t w = ((uint64_t)blockIdx.x * kBlock + threadIdx.x) >> 5; w < tasks; w += warps) {
+    const uint32_t l = (uint32_t)(w % L), h = (uint32_t)(w / L) * 32 + lane;
+    if (h >= n) continue;
+    const float4 hit = __ldg(sw.hit + h);
+    const uint32_t id = __float_as_uint(hit.w) & tr::kIdMask;
+    const float3 x = tr::f3(hit.x, hit.y, hit.z);
+    const float4 light = fa.lights.xyzw[l];
+    float3 wi;
+    float E;
+    tr::light_dir(light, x, wi, E);
+    float T[3], sg2;
+    bool ok = true;
+    tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
+    tr::shadow_path<PREC, false>(fa, x, wi, tr::path_length(light, E),
+                                 __float_as_uint(__ldg(&fa.prim_aux[id].x)), T, sg2, ok, cn);
+    if (!ok) atomicAdd(fa.overflow, 1u);
+    sw.path[(size_t)l * sw.cap + h] = make_float4(T[0], T[1], T[2], sg2);
+  }
+}
+
+// Shading and compositing of the listed tiles, one warp each, with the same
+// sums as the one-kernel form.
+template <int PREC>
+__global__ void __launch_bounds__(kBlock)
+    k_shadow_shade(const FrameArgs fa, const float4* __restrict__ rect_p, const ShadowWork sw,
+                   float* __restrict__ rgb) {
+  const float4 rect = *rect_p;
+  const WarpGrid g = warp_grid(rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
+  const uint32_t lane = threadIdx.x & 31, G = fa.grp;
+  const uint32_t n = sw.ctr[1], warps = gridDim.x * (kBlock / 32);
+  for (uint32_t i = (blockIdx.x * kBlock + threadIdx.x) >> 5; i < n; i += warps) {
+    const ShadowTile& st = sw.tiles[i];
+    const uint32_t t = st.tile, cnt = reinterpret_cast<const uint8_t*>(st.cnt)[lane];
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, q);
+      if (lane >= (uint32_t)q) incl += v;
+    }
+    const uint32_t h0 = st.base + incl - cnt;
+    const uint32_t x0 = g.x0 + (t % g.nx) * g.wtw, y0 = g.y0 + (t / g.nx) * g.wth, p = lane / G;
+    float acc[3] = {0.f, 0.f, 0.f};
+    if (cnt) {
+      const uint64_t pixel = (uint64_t)(y0 + p / g.wtw) * (uint32_t)fa.cam.W + x0 + p % g.wtw;
+      tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
+      tr::RayKey rk;
+      float3 o, d;
+      tr::primary_ray(fa, pixel * fa.spp + (lane & (G - 1)), o, d, rk);
+      float T = 1.f;
+      for (uint32_t j = 0; j < cnt && T > 0.f; ++j) {
+        float c[3], a;
+        tr::shade_hit<PREC, false, false, true>(
+            fa, __float_as_uint(__ldg(&sw.hit[h0 + j].w)) & tr::kIdMask, __ldg(sw.depth + h0 + j), o, d,
+            c, a, cn, sw.path + h0 + j, sw.cap);
+        const float ta = T * a;
+        acc[0] = fmaf(ta, c[0], acc[0]);
+        acc[1] = fmaf(ta, c[1], acc[1]);
+        acc[2] = fmaf(ta, c[2], acc[2]);
+        T *= 1.f - a;
+      }
+    }
+    tr::tile_write(fa, x0, y0, g.wtw, rect, acc, rgb);
+  }
+}
+
+int sm_count() {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+template <typename K>
+int resident_grid(K kernel) {
+  const int sms = sm_count();
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kBlock, 0) != cudaSuccess || per < 1) {
+    cudaGetLastError();
+    per = 1;
+  }
+  return sms * per;
+}
+
+template <int KMAX, int PREC>
+hr_status launch_rounds(hr_ctx* ctx, const FrameArgs& fa, const float4* rect, uint32_t* work,
+                        ShadowWork sw, uint32_t rounds, int g_hits, float* rgb, cudaStream_t st) {
+  static const int g_paths = resident_grid(k_shadow_paths<PREC>);
+  static const int g_shade = resident_grid(k_shadow_shade<PREC>);
+  for (uint32_t r = 0; r < rounds; ++r) {
+    HR_CUDA(ctx, cudaMemsetAsync(sw.ctr, 0, 8, st));
+    k_shadow_hits<KMAX><<<g_hits, kBlock, 0, st>>>(fa, rect, work, sw);
+    HR_LAUNCHED(ctx);
+    k_shadow_paths<PREC><<<8 * g_paths, kBlock, 0, st>>>(fa, sw);
+    HR_LAUNCHED(ctx);
+    k_shadow_shade<PREC><<<g_shade, kBlock, 0, st>>>(fa, rect, sw, rgb);
+    HR_LAUNCHED(ctx);
+  }
+  return HR_OK;
+}
+
+template <int PREC>
+hr_status launch_rounds_k(hr_ctx* ctx, const FrameArgs& fa, const float4* rect, uint32_t* work,
+                          const ShadowWork& sw, uint32_t rounds, int g_hits, float* rgb,
+                          cudaStream_t st) {
+  switch (kmax_for(fa.k)) {
+    case 1: return launch_rounds<1, PREC>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st);
+    case 2: return launch_rounds<2, PREC>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st);
+    case 4: return launch_rounds<4, PREC>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st);
+    default: return launch_rounds<8, PREC>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st);
+  }
+}
+
+}  // namespace
+
+// The tiles that the rounds take; *left says whether tiles can be left over
+// (from *work on, for the one-kernel form).  Nothing is launched (and *left is
+// set) where the buffers do not fit the context's budget or a lane traces
+// more than one sample of a pixel (more than 32 spp: its hits would need
+// an order of their own).
+hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, const float4* rect,
+                               uint32_t* work, float* rgb, cudaStream_t st, bool* left) {
+  *left = true;
+  if (fa.spp > fa.grp) return HR_OK;
+  const uint64_t L = (uint64_t)fa.lights.n;
+  const uint64_t worst = (uint64_t)fa.cam.W * fa.cam.H * fa.spp * fa.k;
+  const uint64_t stop = std::min<uint64_t>(worst, kPathBudget / L);
+  // every launched warp can be at a tile of 32 lanes and k hits when the round
+  // fills up; nothing is added past the worst case
+  const int g_hits = 4 * sm_count();
+  const uint64_t cap = std::min<uint64_t>(worst, stop + (uint64_t)g_hits * kBlock * fa.k);
+  const size_t bytes = 64 + cap * (sizeof(float4) + sizeof(ShadowTile) + sizeof(float) + L * sizeof(float4));
+  char* p = nullptr;
+  if (scratch(ctx, 17, bytes, (void**)&p) != HR_OK) {
+    set_error(ctx, HR_OK, "");
+    return HR_OK;
+  }
+  ShadowWork sw{};
+  sw.path = reinterpret_cast<float4*>(p);
+  sw.hit = sw.path + L * cap;
+  sw.tiles = reinterpret_cast<ShadowTile*>(sw.hit + cap);
+  sw.depth = reinterpret_cast<float*>(sw.tiles + cap);
+  sw.ctr = reinterpret_cast<uint32_t*>(sw.depth + cap);
+  sw.stop = (uint32_t)stop;
+  sw.cap = (uint32_t)cap;
+  const uint32_t rounds = (uint32_t)std::min<uint64_t>((worst + stop - 1) / stop, kMaxRounds);
+  *left = (uint64_t)rounds * stop < worst;
+  return precision == HR_PREC_FP16
+             ? launch_rounds_k<HR_PREC_FP16>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st)
+             : launch_rounds_k<HR_PREC_FP32>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st);
+}
+
+}  // namespace hr
