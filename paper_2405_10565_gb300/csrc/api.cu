@@ -81,12 +81,33 @@ uint64_t ctx_budget(hr_ctx* ctx) { return ctx->budget; }
 
 uint32_t* ctx_overflow(hr_ctx* ctx) { return ctx->d_overflow; }
 
+// Gives back the scratch that frames can do without (the rays put aside, the
+// light paths of a shadow frame), so that it never stands in the way of
+// another allocation; false when there was none.
+static bool drop_optional_scratch(hr_ctx* ctx) {
+  bool any = false;
+  for (int slot : {kScratchPaths, kScratchLong}) {
+    Scratch& s = ctx->scratch[slot];
+    if (!s.p) continue;
+    if (!any) cudaStreamSynchronize(ctx->stream);
+    dfree(ctx, s.p, s.bytes);
+    s = Scratch();
+    any = true;
+  }
+  return any;
+}
+
 hr_status dalloc(hr_ctx* ctx, void** p, size_t bytes, const char* what) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
-  if (ctx->budget && ctx->used.load() + bytes > ctx->budget)
+  if (ctx->budget && ctx->used.load() + bytes > ctx->budget &&
+      (!drop_optional_scratch(ctx) || ctx->used.load() + bytes > ctx->budget))
     return set_error(ctx, HR_ENOMEM, std::string("HBM budget exceeded allocating ") + what);
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess && drop_optional_scratch(ctx)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -157,8 +178,9 @@ hr_status to_device(hr_ctx* ctx, void* dst, const void* src, size_t bytes, cudaS
 FrameArgs frame_args(hr_ctx* ctx, hr_asset* a, const Bvh& bv, const hr_render_desc& d) {
   FrameArgs fa{};
   fa.nodes = bv.nodes;
-  fa.prim_xf = a->prim_xf;
-  fa.prim_aux = a->prim_aux;
+  fa.frame = bv.frame;
+  fa.prim_uv = a->prim_uv;
+  fa.prim_wa = a->prim_wa;
   fa.leaf_id = bv.leaf_id;
   fa.verts = a->verts;
   fa.xsec = a->xsec;
@@ -374,30 +396,30 @@ hr_status hr_asset_update(hr_ctx* ctx, hr_asset* a, const float* vertices) {
     const size_t nv = (size_t)a->N * (a->S + 1);
     if (a->other_total != P) {  // (re)size the other set to the current records
       if (a->verts_other) dfree(ctx, a->verts_other, nv * sizeof(float4)), a->verts_other = nullptr;
-      if (a->xf_other) dfree(ctx, a->xf_other, (size_t)a->other_total * 3 * sizeof(float4)), a->xf_other = nullptr;
+      if (a->uv_other) dfree(ctx, a->uv_other, (size_t)a->other_total * 2 * sizeof(float4)), a->uv_other = nullptr;
       if (a->box_other) dfree(ctx, a->box_other, (size_t)a->other_total * 2 * sizeof(float4)), a->box_other = nullptr;
-      if (a->aux_other) dfree(ctx, a->aux_other, (size_t)a->other_total * sizeof(float4)), a->aux_other = nullptr;
+      if (a->wa_other) dfree(ctx, a->wa_other, (size_t)a->other_total * 2 * sizeof(float4)), a->wa_other = nullptr;
       a->other_total = 0;
       HR_TRY(dalloc(ctx, (void**)&a->verts_other, nv * sizeof(float4), "vertices (second set)"));
-      HR_TRY(dalloc(ctx, (void**)&a->xf_other, P * 3 * sizeof(float4), "records (second set)"));
+      HR_TRY(dalloc(ctx, (void**)&a->uv_other, P * 2 * sizeof(float4), "records (second set)"));
       HR_TRY(dalloc(ctx, (void**)&a->box_other, P * 2 * sizeof(float4), "boxes (second set)"));
-      HR_TRY(dalloc(ctx, (void**)&a->aux_other, P * sizeof(float4), "aux (second set)"));
+      HR_TRY(dalloc(ctx, (void**)&a->wa_other, P * 2 * sizeof(float4), "aux (second set)"));
       a->other_total = (uint32_t)P;
     }
     cudaStream_t sd = ctx->side;
     HR_CUDA(ctx, cudaStreamWaitEvent(sd, ctx->ev_built, 0));
     if (P > ns) {  // the thick-hair records too, so the new set is whole whatever comes next
-      HR_CUDA(ctx, cudaMemcpyAsync(a->xf_other + 3 * ns, a->prim_xf + 3 * ns, (P - ns) * 3 * sizeof(float4),
+      HR_CUDA(ctx, cudaMemcpyAsync(a->uv_other + 2 * ns, a->prim_uv + 2 * ns, (P - ns) * 2 * sizeof(float4),
                                    cudaMemcpyDeviceToDevice, sd));
       HR_CUDA(ctx, cudaMemcpyAsync(a->box_other + 2 * ns, a->prim_box + 2 * ns, (P - ns) * 2 * sizeof(float4),
                                    cudaMemcpyDeviceToDevice, sd));
-      HR_CUDA(ctx, cudaMemcpyAsync(a->aux_other + ns, a->prim_aux + ns, (P - ns) * sizeof(float4),
+      HR_CUDA(ctx, cudaMemcpyAsync(a->wa_other + 2 * ns, a->prim_wa + 2 * ns, (P - ns) * 2 * sizeof(float4),
                                    cudaMemcpyDeviceToDevice, sd));
     }
     std::swap(a->verts, a->verts_other);
-    std::swap(a->prim_xf, a->xf_other);
+    std::swap(a->prim_uv, a->uv_other);
     std::swap(a->prim_box, a->box_other);
-    std::swap(a->prim_aux, a->aux_other);
+    std::swap(a->prim_wa, a->wa_other);
     HR_TRY(update_strands(ctx, a, view, sd));
     // everything enqueued on the main stream from here on sees the new set
     HR_CUDA(ctx, cudaEventRecord(ctx->ev_update, sd));
@@ -432,17 +454,17 @@ hr_status hr_asset_destroy(hr_ctx* ctx, hr_asset* a) {
   if (a->xsec) dfree(ctx, a->xsec, (size_t)a->E * S1 * 3 * sizeof(float4));
   if (a->xsec_other) dfree(ctx, a->xsec_other, (size_t)a->E * S1 * 3 * sizeof(float4));
   if (a->verts_other) dfree(ctx, a->verts_other, (size_t)a->N * S1 * sizeof(float4));
-  if (a->xf_other) dfree(ctx, a->xf_other, (size_t)a->other_total * 3 * sizeof(float4));
+  if (a->uv_other) dfree(ctx, a->uv_other, (size_t)a->other_total * 2 * sizeof(float4));
   if (a->box_other) dfree(ctx, a->box_other, (size_t)a->other_total * 2 * sizeof(float4));
-  if (a->aux_other) dfree(ctx, a->aux_other, (size_t)a->other_total * sizeof(float4));
+  if (a->wa_other) dfree(ctx, a->wa_other, (size_t)a->other_total * 2 * sizeof(float4));
   if (a->lod) dfree(ctx, a->lod, a->C);
   if (a->sched) dfree(ctx, a->sched, sizeof(TileSched));
   drop_guides(ctx, a);
   const uint64_t P = a->n_prims_total;
-  if (a->prim_xf) dfree(ctx, a->prim_xf, P * 3 * sizeof(float4));
+  if (a->prim_uv) dfree(ctx, a->prim_uv, P * 2 * sizeof(float4));
   if (a->prim_box) dfree(ctx, a->prim_box, P * 2 * sizeof(float4));
-  if (a->prim_aux) dfree(ctx, a->prim_aux, P * sizeof(float4));
-  if (a->d_bounds) dfree(ctx, a->d_bounds, 8 * sizeof(uint32_t));
+  if (a->prim_wa) dfree(ctx, a->prim_wa, P * 2 * sizeof(float4));
+  if (a->d_bounds) dfree(ctx, a->d_bounds, kBoundWords * sizeof(uint32_t));
   free_bvh(ctx, a->bvh);
   delete a;
   return HR_OK;

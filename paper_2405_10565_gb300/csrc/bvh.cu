@@ -17,10 +17,14 @@
 // them) in barrier-separated rounds in shared memory; k_climb finishes the few
 // nodes that span blocks by float atomic min / max from each climb start.
 //
-// Node layout (4 x float4 = 64 bytes), children's boxes stored in the parent:
-//   n0 = (lo0.x, hi0.x, lo0.y, hi0.y)  n1 = (lo1.x, hi1.x, lo1.y, hi1.y)
-//   n2 = (lo0.z, hi0.z, lo1.z, hi1.z)  n3 = (child0, child1, -, -) as int bits
-// A child index >= 0 is an internal node, < 0 is leaf ~index.
+// Node layout (2 x uint4 = 32 bytes, one sector), children's boxes stored in
+// the parent: per child the x, y and z intervals and the child index.  An
+// interval is lo | hi << 16 on the BVH's grid (Bvh::frame: 65,520 steps over
+// the bounds of every strand and thick-hair box), rounded outward and widened
+// by one step more, which covers the half step that the traversal's decoding
+// can be off.  A child index >= 0 is an internal node, < 0 is primitive
+// ~index.  FP32 boxes took two sectors: a far larger part of the traversal's
+// loads missed L1 (the 4K frame of 500k strands: 25% of the sectors).
 #include <algorithm>
 #include <vector>
 
@@ -87,6 +91,37 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
   return v;
 }
 
+constexpr size_t kFrameWords = 5;
+
+// The grid of the node boxes, from the bounds of the strands' and the thick
+// hairs' boxes: low corner (two steps below the bounds), step, 1 / step; and
+// the leaves' bounds and the climb's counts cleared for k_gather_refit.
+__device__ __forceinline__ void begin_refit(const uint32_t* __restrict__ bounds, float4* frame,
+                                            unsigned* counts) {
+  float lo[3], hi[3], st[3];
+  for (int i = 0; i < 3; ++i) {
+    lo[i] = from_ordered(bounds[i]);
+    hi[i] = from_ordered(bounds[3 + i]);
+    const uint32_t el = bounds[kEthBounds + i], eh = bounds[kEthBounds + 3 + i];
+    if (el <= eh) {  // there are thick hairs
+      lo[i] = fminf(lo[i], from_ordered(el));
+      hi[i] = fmaxf(hi[i], from_ordered(eh));
+    }
+    st[i] = fmaxf((hi[i] - lo[i]) * (1.0f / 65520.0f), 1e-30f);
+    lo[i] = fmaf(-2.0f, st[i], lo[i]);
+  }
+  frame[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
+  frame[1] = make_float4(st[0], st[1], st[2], 0.f);
+  frame[2] = make_float4(1.0f / st[0], 1.0f / st[1], 1.0f / st[2], 0.f);
+  uint32_t* leaf_bounds = reinterpret_cast<uint32_t*>(frame + 3);
+  for (int i = 0; i < 6; ++i) leaf_bounds[i] = i < 3 ? 0xffffffffu : 0u;
+  counts[0] = counts[1] = 0u;
+}
+
+__global__ void k_begin_refit(const uint32_t* __restrict__ bounds, float4* frame, unsigned* counts) {
+  begin_refit(bounds, frame, counts);
+}
+
 // Primitive centroid codes keep the top 7 bits of each axis (21 bits, three
 // radix passes).  Primitives in one cell keep the order of the active list
 // (clusters in root Morton order, each strand's segments in order along the
@@ -97,8 +132,10 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
 constexpr int kMortonBits = 21;
 
 __global__ void k_prim_morton(const float4* __restrict__ box, const uint32_t* __restrict__ ids,
-                              uint32_t n, const uint32_t* __restrict__ bounds, uint32_t* keys) {
+                              uint32_t n, const uint32_t* __restrict__ bounds, uint32_t* keys,
+                              float4* frame, unsigned* counts) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) begin_refit(bounds, frame, counts);
   if (i >= n) return;
   float3 lo, hi, inv_ext;
   lo.x = from_ordered(__ldg(bounds)), lo.y = from_ordered(__ldg(bounds + 1));
@@ -172,56 +209,46 @@ __global__ void k_gather(const uint32_t* __restrict__ sorted_ids, uint32_t n, ui
   if (i < n) leaf_id[i] = sorted_ids[i];
 }
 
-__device__ __forceinline__ void node_union(const float4* nodes, int c, float* b) {
-  // union of an internal node's two child boxes (read through L2: written by
-  // other blocks during this kernel)
-  const float4 n0 = __ldcg(nodes + 4 * c), n1 = __ldcg(nodes + 4 * c + 1),
-               n2 = __ldcg(nodes + 4 * c + 2);
-  b[0] = fminf(n0.x, n1.x);
-  b[1] = fmaxf(n0.y, n1.y);
-  b[2] = fminf(n0.z, n1.z);
-  b[3] = fmaxf(n0.w, n1.w);
-  b[4] = fminf(n2.x, n2.z);
-  b[5] = fmaxf(n2.y, n2.w);
+// A box on the grid: per axis lo | (65535 - hi) << 16, so that the union of
+// two boxes is the smaller of each half.
+struct QBox {
+  uint32_t x, y, z;
+};
+__device__ __forceinline__ uint32_t q_axis(float l, float h, float lo, float inv_step) {
+  const float a = floorf((l - lo) * inv_step) - 1.f, b = ceilf((h - lo) * inv_step) + 1.f;
+  const uint32_t qa = (uint32_t)fminf(fmaxf(a, 0.f), 65535.f);
+  const uint32_t qb = (uint32_t)fminf(fmaxf(b, 0.f), 65535.f);
+  return qa | ((65535u - qb) << 16);
+}
+__device__ __forceinline__ QBox q_box(const float4 l, const float4 h, const float4* __restrict__ frame) {
+  const float4 lo = __ldg(frame), is = __ldg(frame + 2);
+  return QBox{q_axis(l.x, h.x, lo.x, is.x), q_axis(l.y, h.y, lo.y, is.y), q_axis(l.z, h.z, lo.z, is.z)};
+}
+__device__ __forceinline__ QBox q_union(const QBox a, const QBox b) {
+  return QBox{__vminu2(a.x, b.x), __vminu2(a.y, b.y), __vminu2(a.z, b.z)};
+}
+constexpr uint32_t kFlipHi = 0xffff0000u;  // 65535 - hi <-> hi
+
+__device__ __forceinline__ QBox q_of(const uint4 child) {  // a node record's child box
+  return QBox{child.x ^ kFlipHi, child.y ^ kFlipHi, child.z ^ kFlipHi};
 }
 
-__device__ __forceinline__ void lbox_read(const float4* lbox, int leaf, float* b) {
-  const float4 l = __ldcg(lbox + 2 * leaf), h = __ldcg(lbox + 2 * leaf + 1);
-  b[0] = l.x; b[1] = h.x; b[2] = l.y; b[3] = h.y; b[4] = l.z; b[5] = h.z;
-}
-
-// Bounds of an internal node, from two child boxes (lo.x, hi.x, lo.y, hi.y,
-// lo.z, hi.z), as the node record.  The records are stored with an L2
-// evict-last policy: the frame kernel that follows the build reads them, and
-// keeping them in L2 over the leaf records written beside them took the
-// full-head frame from 0.63 to 0.60 ms (evict-last on the leaf records as
-// well was slower).
-__device__ __forceinline__ void store_node(float4* nodes, int node, int4 ch, const float* c0,
-                                           const float* c1) {
-  float4* o = nodes + 4 * node;
+// The record of a node from its children's boxes and indices.  The records are
+// stored with an L2 evict-last policy: the frame kernel that follows the build
+// reads them (with 64-byte records the full-head frame took 0.60 instead of
+// 0.63 ms).
+__device__ __forceinline__ void store_node(uint4* nodes, int node, const QBox c0, int i0, const QBox c1,
+                                           int i1) {
+  uint4* o = nodes + 2 * (size_t)node;
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-  const float4 v[4] = {make_float4(c0[0], c0[1], c0[2], c0[3]), make_float4(c1[0], c1[1], c1[2], c1[3]),
-                       make_float4(c0[4], c0[5], c1[4], c1[5]),
-                       make_float4(__int_as_float(ch.x), __int_as_float(ch.y), 0.f, 0.f)};
+  const uint4 v[2] = {make_uint4(c0.x ^ kFlipHi, c0.y ^ kFlipHi, c0.z ^ kFlipHi, (uint32_t)i0),
+                      make_uint4(c1.x ^ kFlipHi, c1.y ^ kFlipHi, c1.z ^ kFlipHi, (uint32_t)i1)};
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;"
-                 :: "l"(o + q), "f"(v[q].x), "f"(v[q].y), "f"(v[q].z), "f"(v[q].w), "l"(pol)
+  for (int q = 0; q < 2; ++q)
+    asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;"
+                 :: "l"(o + q), "r"(v[q].x), "r"(v[q].y), "r"(v[q].z), "r"(v[q].w), "l"(pol)
                  : "memory");
-}
-
-// Float min / max as one integer atomic on the float's bits (non-negative
-// floats order like signed ints; negative ones order like unsigned ints in
-// reverse).  -0 must not reach them: callers pass +0.  Returns whether the
-// stored value changed.
-__device__ __forceinline__ bool atomic_min_f(float* a, float v) {
-  if (v >= 0.f) return atomicMin(reinterpret_cast<int*>(a), __float_as_int(v)) > __float_as_int(v);
-  return atomicMax(reinterpret_cast<unsigned*>(a), __float_as_uint(v)) < __float_as_uint(v);
-}
-__device__ __forceinline__ bool atomic_max_f(float* a, float v) {
-  if (v >= 0.f) return atomicMax(reinterpret_cast<int*>(a), __float_as_int(v)) < __float_as_int(v);
-  return atomicMin(reinterpret_cast<unsigned*>(a), __float_as_uint(v)) > __float_as_uint(v);
 }
 
 // Warp-aggregated append of one child (node index, or ~leaf) per lane that
@@ -240,28 +267,31 @@ __device__ __forceinline__ void append_start(bool has, int v, unsigned* count, i
 // leaf b0 + j and internal node b0 + j (b0 = b * B).  A node record names a
 // leaf child by ~(its global primitive id), so the frame kernel reads the
 // primitive's records where they are (no copy into leaf order).
-//  1. Gather: each thread reads its leaf's box (and id) into shared memory.
+//  1. Gather: each thread reads its leaf's box (and id) into shared memory, on
+//     the grid: three words, united by three 16-bit pair minima.
 //  2. Local subtrees: node i's leaf range starts or ends at leaf i, so a node
 //     whose range lies inside the block's leaves ("local") is owned by a
 //     thread of the block and so are its children.  These are finished in
 //     rounds separated by barriers: a node whose children are done takes
 //     their boxes from shared memory, writes its record and its union.  The
 //     rounds number the local subtrees' height; no fences, no atomics.
-//  3. The few nodes that span blocks are left to k_climb: their owners set
-//     their child boxes empty, and the owner of each local node (or leaf)
-//     whose parent spans blocks publishes its box and lists it as a climb
-//     start, so that no block stays resident behind a climb.
+//  3. The few nodes that span blocks are left to k_climb: their owners give
+//     them a slot of twelve words (their children's coordinates, all taken as
+//     minima), noted in the record, and the owner of each local node (or
+//     leaf) whose parent spans blocks lists it as a climb start, so that no
+//     block stays resident behind a climb.
 template <int B>
 __global__ void __launch_bounds__(B) k_gather_refit(
     const int4* __restrict__ child, const int* __restrict__ parent_int,
     const int* __restrict__ parent_leaf, const float4* __restrict__ box,
-    const uint32_t* sorted_ids, int n, float4* nodes, float4* lbox, uint32_t* leaf_id,
-    unsigned* n_starts, int* starts) {
+    float4* frame, const uint32_t* sorted_ids, int n, uint4* nodes,
+    uint32_t* leaf_id, unsigned* counts, int* starts, int* span_node, uint32_t* span) {
   __shared__ int4 s_child[B];
   __shared__ uint32_t s_id[B];  // global primitive id of each of the block's leaves
-  __shared__ float s_lbox[B][6];  // leaf boxes (lo.x, hi.x, lo.y, hi.y, lo.z, hi.z)
-  __shared__ float s_nbox[B][6];  // unions of the block's local nodes
+  __shared__ QBox s_lbox[B];    // leaf boxes
+  __shared__ QBox s_nbox[B];    // unions of the block's local nodes
   __shared__ unsigned char s_done[B];
+  __shared__ uint32_t s_bound[6];
   const int b0 = blockIdx.x * B;
   const int j = threadIdx.x;
   const int leaf = b0 + j, node = b0 + j;
@@ -272,19 +302,46 @@ __global__ void __launch_bounds__(B) k_gather_refit(
   s_done[j] = 0;
   const bool node_local = has_node && ch.z >= b0 && ch.w < b0 + B;
   // 1. gather
-  float4 bl = make_float4(0.f, 0.f, 0.f, 0.f), bh = bl;
   int lparent = -1;
+  float4 bl = make_float4(0.f, 0.f, 0.f, 0.f), bh = bl;
   if (leaf < n) {
     const uint32_t id = sorted_ids[leaf];
-    bl = box[2 * (size_t)id];
-    bh = box[2 * (size_t)id + 1];
     lparent = parent_leaf[leaf];
     leaf_id[leaf] = id;
     s_id[j] = id;
-    s_lbox[j][0] = bl.x; s_lbox[j][1] = bh.x; s_lbox[j][2] = bl.y;
-    s_lbox[j][3] = bh.y; s_lbox[j][4] = bl.z; s_lbox[j][5] = bh.z;
+    bl = box[2 * (size_t)id];
+    bh = box[2 * (size_t)id + 1];
+    s_lbox[j] = q_box(bl, bh, frame);
+  }
+  if (j < 6) s_bound[j] = j < 3 ? 0xffffffffu : 0u;
+  __syncthreads();
+  // the leaves' exact bounds (the camera rays are re-based at their entry into
+  // them): the block's, and of those the few that reach further than any so
+  // far (one read a block: a read a warp queued up at the one line, 0.17 ms
+  // for 4.6M leaves)
+  {
+    const uint32_t lo[3] = {ordered_bits(bl.x + 0.f), ordered_bits(bl.y + 0.f), ordered_bits(bl.z + 0.f)};
+    const uint32_t hi[3] = {ordered_bits(bh.x + 0.f), ordered_bits(bh.y + 0.f), ordered_bits(bh.z + 0.f)};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const uint32_t l = __reduce_min_sync(0xffffffffu, leaf < n ? lo[i] : 0xffffffffu);
+      const uint32_t h = __reduce_max_sync(0xffffffffu, leaf < n ? hi[i] : 0u);
+      if ((j & 31) == 0) {
+        atomicMin(&s_bound[i], l);
+        atomicMax(&s_bound[3 + i], h);
+      }
+    }
   }
   __syncthreads();
+  if (j < 6) {
+    uint32_t* g = reinterpret_cast<uint32_t*>(frame + 3) + j;
+    const uint32_t v = s_bound[j], far = __ldcg(g);
+    if (j < 3) {
+      if (v < far) atomicMin(g, v);
+    } else if (v > far) {
+      atomicMax(g, v);
+    }
+  }
   // 2. local subtrees, one level of readiness per round
   bool pending = node_local;
   for (;;) {
@@ -292,24 +349,12 @@ __global__ void __launch_bounds__(B) k_gather_refit(
     if (pending)
       ready = (ch.x < 0 || s_done[ch.x - b0]) && (ch.y < 0 || s_done[ch.y - b0]);
     if (ready) {
-      const float* p0 = ch.x < 0 ? s_lbox[~ch.x - b0] : s_nbox[ch.x - b0];
-      const float* p1 = ch.y < 0 ? s_lbox[~ch.y - b0] : s_nbox[ch.y - b0];
-      float c0[6], c1[6];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        c0[q] = p0[q];
-        c1[q] = p1[q];
-      }
+      const QBox c0 = ch.x < 0 ? s_lbox[~ch.x - b0] : s_nbox[ch.x - b0];
+      const QBox c1 = ch.y < 0 ? s_lbox[~ch.y - b0] : s_nbox[ch.y - b0];
       // a leaf child is named by its primitive id (the leaf lies in this block)
-      const int4 chp = make_int4(ch.x < 0 ? ~(int)s_id[~ch.x - b0] : ch.x,
-                                 ch.y < 0 ? ~(int)s_id[~ch.y - b0] : ch.y, ch.z, ch.w);
-      store_node(nodes, node, chp, c0, c1);
-      s_nbox[j][0] = fminf(c0[0], c1[0]);
-      s_nbox[j][1] = fmaxf(c0[1], c1[1]);
-      s_nbox[j][2] = fminf(c0[2], c1[2]);
-      s_nbox[j][3] = fmaxf(c0[3], c1[3]);
-      s_nbox[j][4] = fminf(c0[4], c1[4]);
-      s_nbox[j][5] = fmaxf(c0[5], c1[5]);
+      store_node(nodes, node, c0, ch.x < 0 ? ~(int)s_id[~ch.x - b0] : ch.x, c1,
+                 ch.y < 0 ? ~(int)s_id[~ch.y - b0] : ch.y);
+      s_nbox[j] = q_union(c0, c1);
     }
     const int any = __syncthreads_or(ready);  // this round's reads of s_done are over
     if (ready) {
@@ -320,77 +365,87 @@ __global__ void __launch_bounds__(B) k_gather_refit(
     __syncthreads();  // this round's flags are visible
   }
   // 3. nodes that span blocks: empty child boxes, widened by k_climb
-  if (has_node && !node_local) {
-    float4* o = nodes + 4 * (size_t)node;
-    const float inf = __int_as_float(0x7f800000);
-    const float4 e = make_float4(inf, -inf, inf, -inf);
-    __stcg(o, e);
-    __stcg(o + 1, e);
-    __stcg(o + 2, e);
-    const int c0 = ch.x < 0 ? ~(int)sorted_ids[~ch.x] : ch.x;
-    const int c1 = ch.y < 0 ? ~(int)sorted_ids[~ch.y] : ch.y;
-    __stcg(o + 3, make_float4(__int_as_float(c0), __int_as_float(c1), 0.f, 0.f));
-  }
-  bool start_leaf = false, start_node = false;
-  if (leaf < n && lparent >= 0) {
-    const bool parent_local = lparent >= b0 && lparent < b0 + B && s_child[lparent - b0].z >= b0 &&
-                              s_child[lparent - b0].w < b0 + B;
-    if (!parent_local) {
-      __stcg(lbox + 2 * leaf, bl);
-      __stcg(lbox + 2 * leaf + 1, bh);
-      start_leaf = true;
+  const bool spans = has_node && !node_local;
+  const unsigned m = __ballot_sync(0xffffffffu, spans);
+  if (m) {
+    const int lane = j & 31, lead = __ffs(m) - 1;
+    unsigned base = 0;
+    if (lane == lead) base = atomicAdd(counts + 1, (unsigned)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, lead);
+    if (spans) {
+      const unsigned slot = base + __popc(m & ((1u << lane) - 1u));
+      span_node[slot] = node;
+      for (int q = 0; q < 12; ++q) span[12 * (size_t)slot + q] = 0xffffffffu;
+      const int c0 = ch.x < 0 ? ~(int)sorted_ids[~ch.x] : ch.x;
+      const int c1 = ch.y < 0 ? ~(int)sorted_ids[~ch.y] : ch.y;
+      nodes[2 * (size_t)node] = make_uint4(slot, 0u, 0u, (uint32_t)c0);
+      nodes[2 * (size_t)node + 1] = make_uint4(0u, 0u, 0u, (uint32_t)c1);
     }
   }
+  bool start_leaf = false, start_node = false;
+  if (leaf < n && lparent >= 0)
+    start_leaf = !(lparent >= b0 && lparent < b0 + B && s_child[lparent - b0].z >= b0 &&
+                   s_child[lparent - b0].w < b0 + B);
   if (node_local && node != 0) {
     const int p = __ldg(parent_int + node);
     start_node = !(p >= b0 && p < b0 + B && s_child[p - b0].z >= b0 && s_child[p - b0].w < b0 + B);
   }
-  append_start(start_leaf, ~leaf, n_starts, starts);
-  append_start(start_node, node, n_starts, starts);
+  append_start(start_leaf, ~leaf, counts, starts);
+  append_start(start_node, node, counts, starts);
 }
 
 // Bounds of the nodes that span blocks.  Each climb start (a leaf or local
-// node whose parent spans blocks; its record is complete) widens, with float
-// atomics, its own slot in its parent, then its parent's slot in the
-// grandparent, and so on to the root.  Each of the six coordinates stops at
-// the first ancestor slot that it does not change: that slot already holds a
-// value at least as wide from another start below it, which carries it on
-// up.  No ordering between starts is needed.
-__global__ void k_climb(const unsigned* __restrict__ n_starts, const int* __restrict__ starts,
+// node whose parent spans blocks; its record is complete) lowers, with integer
+// atomics, its own words in its parent's slot, then its parent's in the
+// grandparent's, and so on to the root.  Each of the six coordinates stops at
+// the first ancestor that it does not change: that one already holds a value
+// at least as wide from another start below it, which carries it on up.  No
+// ordering between starts is needed.
+__global__ void k_climb(const unsigned* __restrict__ counts, const int* __restrict__ starts,
                         const int4* __restrict__ child, const int* __restrict__ parent_int,
-                        const int* __restrict__ parent_leaf, float4* nodes, const float4* lbox) {
-  const unsigned m = *n_starts;
+                        const int* __restrict__ parent_leaf, const float4* __restrict__ box,
+                        const float4* __restrict__ frame, const uint32_t* __restrict__ leaf_id,
+                        const uint4* __restrict__ nodes, uint32_t* span) {
+  const unsigned m = *counts;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
     int cur = __ldg(starts + i);
-    float b[6];
+    QBox u;
     int p;
     if (cur < 0) {
-      lbox_read(lbox, ~cur, b);
+      const size_t id = __ldg(leaf_id + ~cur);
+      u = q_box(__ldg(box + 2 * id), __ldg(box + 2 * id + 1), frame);
       p = __ldg(parent_leaf + ~cur);
     } else {
-      node_union(nodes, cur, b);
+      u = q_union(q_of(__ldg(nodes + 2 * (size_t)cur)), q_of(__ldg(nodes + 2 * (size_t)cur + 1)));
       p = __ldg(parent_int + cur);
     }
-#pragma unroll
-    for (int q = 0; q < 6; ++q) b[q] = b[q] + 0.f;  // -0 -> +0
+    const uint32_t b[6] = {u.x & 0xffffu, u.x >> 16, u.y & 0xffffu, u.y >> 16, u.z & 0xffffu, u.z >> 16};
     unsigned live = 0x3fu;
     while (p >= 0) {
-      const int4 ch = __ldg(child + p);
+      const int first = __ldg(&child[p].x);
       const int up = p == 0 ? -1 : __ldg(parent_int + p);
-      float* r = reinterpret_cast<float*>(nodes + 4 * (size_t)p);
-      // record slots of (lo.x, hi.x, lo.y, hi.y, lo.z, hi.z) for child 0 / child 1
-      const int o = ch.x == cur ? 0 : 4, oz = ch.x == cur ? 8 : 10;
-      const int off[6] = {o, o + 1, o + 2, o + 3, oz, oz + 1};
+      uint32_t* r = span + 12 * (size_t)__ldg(&nodes[2 * (size_t)p].x) + (first == cur ? 0 : 6);
 #pragma unroll
       for (int q = 0; q < 6; ++q)
-        if ((live >> q) & 1u) {
-          const bool changed = (q & 1) ? atomic_max_f(r + off[q], b[q]) : atomic_min_f(r + off[q], b[q]);
-          if (!changed) live &= ~(1u << q);
-        }
+        if ((live >> q) & 1u)
+          if (atomicMin(r + q, b[q]) <= b[q]) live &= ~(1u << q);
       if (!live) break;
       cur = p;
       p = up;
     }
+  }
+}
+
+// The records of the nodes that span blocks, from their slots.
+__global__ void k_span_records(const unsigned* __restrict__ counts, const int* __restrict__ span_node,
+                               const uint32_t* __restrict__ span, uint4* nodes) {
+  const unsigned m = counts[1];
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+    const uint32_t* r = span + 12 * (size_t)i;
+    const int node = span_node[i];
+    const int c0 = (int)nodes[2 * (size_t)node].w, c1 = (int)nodes[2 * (size_t)node + 1].w;
+    store_node(nodes, node, QBox{r[0] | r[1] << 16, r[2] | r[3] << 16, r[4] | r[5] << 16}, c0,
+               QBox{r[6] | r[7] << 16, r[8] | r[9] << 16, r[10] | r[11] << 16}, c1);
   }
 }
 
@@ -400,21 +455,22 @@ __global__ void k_bytes_differ(const uint8_t* __restrict__ x, const uint8_t* __r
   if (i < n && x[i] != y[i]) *diff = 1u;
 }
 
-// Leaf records of the primitives `ids` (in leaf order) and every node's
-// bounds, over the topology in bv.
+// Every node's record over the topology in bv and the primitives `ids` in leaf
+// order, after begin_refit on the same stream.
 hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, cudaStream_t st) {
   const uint32_t n = bv.n;
-  unsigned* n_starts = nullptr;
-  float4* lbox = nullptr;
-  int* starts = nullptr;  // at most one per leaf and one per internal node
-  HR_TRY(scratch(ctx, 39, 16, (void**)&n_starts));
-  HR_TRY(scratch(ctx, 46, (size_t)n * 2 * sizeof(float4), (void**)&lbox));
-  HR_TRY(scratch(ctx, 48, (size_t)n * 2 * 4, (void**)&starts));
-  HR_CUDA(ctx, cudaMemsetAsync(n_starts, 0, 4, st));
+  unsigned* counts = nullptr;  // climb starts, nodes that span blocks
+  int *starts = nullptr, *span_node = nullptr;
+  uint32_t* span = nullptr;
+  HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
+  HR_TRY(scratch(ctx, 46, (size_t)n * 13 * 4, (void**)&span));
+  HR_TRY(scratch(ctx, 48, (size_t)n * 2 * 4, (void**)&starts));  // one per leaf and per node at most
+  span_node = reinterpret_cast<int*>(span + 12 * (size_t)n);
   k_gather_refit<256><<<(n + 255) / 256, 256, 0, st>>>(bv.child, bv.par_int, bv.par_leaf,
-                                                       a->prim_box, ids, (int)n, bv.nodes, lbox,
-                                                       bv.leaf_id, n_starts, starts);
+                                                       a->prim_box, bv.frame, ids, (int)n, bv.nodes,
+                                                       bv.leaf_id, counts, starts, span_node, span);
   HR_LAUNCHED(ctx);
+  if (n <= 256) return HR_OK;  // one block: every node is local
   static int climb_grid = 0;
   if (!climb_grid) {
     int dev = 0, sms = 1, per = 0;
@@ -427,7 +483,10 @@ hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, c
     climb_grid = sms * per;
   }
   const unsigned grid = (unsigned)std::min<size_t>((size_t)climb_grid, ((size_t)n * 2 + 255) / 256);
-  k_climb<<<grid, 256, 0, st>>>(n_starts, starts, bv.child, bv.par_int, bv.par_leaf, bv.nodes, lbox);
+  k_climb<<<grid, 256, 0, st>>>(counts, starts, bv.child, bv.par_int, bv.par_leaf, a->prim_box,
+                                bv.frame, bv.leaf_id, bv.nodes, span);
+  HR_LAUNCHED(ctx);
+  k_span_records<<<grid, 256, 0, st>>>(counts, span_node, span, bv.nodes);
   HR_LAUNCHED(ctx);
   return HR_OK;
 }
@@ -436,7 +495,8 @@ hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, c
 
 void free_bvh(hr_ctx* ctx, Bvh& bv) {
   if (bv.cap) {
-    dfree(ctx, bv.nodes, (size_t)std::max(bv.cap, 2u) * 4 * sizeof(float4));
+    dfree(ctx, bv.nodes, (size_t)std::max(bv.cap, 2u) * 2 * sizeof(uint4));
+    dfree(ctx, bv.frame, kFrameWords * sizeof(float4));
     dfree(ctx, bv.leaf_id, (size_t)bv.cap * 4);
     dfree(ctx, bv.child, (size_t)bv.cap * sizeof(int4));
     dfree(ctx, bv.par_int, (size_t)bv.cap * 4);
@@ -483,7 +543,8 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
       HR_CUDA(ctx, cudaStreamSynchronize(st));
       free_bvh(ctx, bv);
     }
-    HR_TRY(dalloc(ctx, (void**)&bv.nodes, (size_t)std::max(n, 2u) * 4 * sizeof(float4), "BVH nodes"));
+    HR_TRY(dalloc(ctx, (void**)&bv.nodes, (size_t)std::max(n, 2u) * 2 * sizeof(uint4), "BVH nodes"));
+    HR_TRY(dalloc(ctx, (void**)&bv.frame, kFrameWords * sizeof(float4), "BVH grid"));
     HR_TRY(dalloc(ctx, (void**)&bv.leaf_id, (size_t)n * 4, "BVH leaf ids"));
     HR_TRY(dalloc(ctx, (void**)&bv.child, (size_t)n * sizeof(int4), "BVH children"));
     HR_TRY(dalloc(ctx, (void**)&bv.par_int, (size_t)n * 4, "BVH parents"));
@@ -520,7 +581,10 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
   HR_TRY(scratch(ctx, 33, (size_t)n * 4, (void**)&keys));
   HR_TRY(scratch(ctx, 34, (size_t)n * 4, (void**)&k2));
   HR_TRY(scratch(ctx, 35, (size_t)n * 4, (void**)&v2));
-  k_prim_morton<<<(n + 255) / 256, 256, 0, st>>>(a->prim_box, ids, n, a->d_bounds, keys);
+  unsigned* counts = nullptr;
+  HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
+  k_prim_morton<<<(n + 255) / 256, 256, 0, st>>>(a->prim_box, ids, n, a->d_bounds, keys, bv.frame,
+                                                 counts);
   HR_LAUNCHED(ctx);
   HR_TRY(radix_sort_pairs(ctx, keys, ids, k2, v2, n, kMortonBits, st, kLookbackPolls, &keys, &ids));
   if (n == 1) {
@@ -563,7 +627,13 @@ hr_status refit_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
   bv.valid = 0;
   const uint32_t n = bv.n;
   // a single leaf has no node; its records are the primitive's own
-  if (n > 1) HR_TRY(gather_refit(ctx, a, bv, bv.leaf_id, st));
+  if (n > 1) {
+    unsigned* counts = nullptr;
+    HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
+    k_begin_refit<<<1, 1, 0, st>>>(a->d_bounds, bv.frame, counts);
+    HR_LAUNCHED(ctx);
+    HR_TRY(gather_refit(ctx, a, bv, bv.leaf_id, st));
+  }
   bv.valid = 1;
   return HR_OK;
 }

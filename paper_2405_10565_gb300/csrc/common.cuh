@@ -34,7 +34,9 @@ struct TileSched;
 struct Bvh {
   uint32_t n = 0;           // active primitives (leaves)
   uint32_t cap = 0;         // allocated leaves
-  float4* nodes = nullptr;  // [(n-1) * 4]; a leaf child is ~(global primitive id)
+  uint4* nodes = nullptr;   // [(n-1) * 2] quantised boxes (see bvh.cu); a leaf child is ~(global primitive id)
+  float4* frame = nullptr;  // [5] the boxes' grid: low corner, step, 1 / step; then, as ordered float
+                            // bits, the leaves' exact bounds lo xyz, hi xyz
   uint32_t* leaf_id = nullptr; // [n] global primitive id of every leaf, Morton order
   uint32_t n_eth = 0;
   int valid = 0;               // bounds and leaf records match the primitives
@@ -77,15 +79,16 @@ struct hr_asset {
   // the other vertex and record buffers of a pipelined hr_asset_update (or
   // null), sized for other_total records
   float4* verts_other = nullptr;
-  float4 *xf_other = nullptr, *box_other = nullptr, *aux_other = nullptr;
+  float4 *uv_other = nullptr, *box_other = nullptr, *wa_other = nullptr;
   uint32_t other_total = 0;
   // all potential primitives: strand segments then thick-hair segments
   uint32_t n_prims_total = 0;
-  float4* prim_xf = nullptr;   // [P_total * 3]
+  float4* prim_uv = nullptr;   // [P_total * 2] world -> unit-cylinder rows u and v
   float4* prim_box = nullptr;  // [P_total * 2]
-  float4* prim_aux = nullptr;  // [P_total]
-  uint32_t* d_bounds = nullptr;  // [8] strand boxes' bounds, ordered float bits (lo xyz, hi xyz);
-                                 // word kHierChanged: the strand order changed since the last BVH build
+  float4* prim_wa = nullptr;   // [P_total * 2] row w, then (material index bits, n_tot, r, a*b)
+  uint32_t* d_bounds = nullptr;  // [16] strand boxes' bounds, ordered float bits (lo xyz, hi xyz);
+                                 // word kHierChanged: the strand order changed since the last BVH build;
+                                 // from word kEthBounds on the thick-hair boxes' bounds
   // LoD
   uint8_t* lod = nullptr;  // [C] current selection on the device
   int lod_valid = 0;
@@ -117,7 +120,9 @@ Tables ctx_tables(hr_ctx* ctx);
 // device allocation charged to the context budget
 hr_status dalloc(hr_ctx* ctx, void** p, size_t bytes, const char* what);
 void dfree(hr_ctx* ctx, void* p, size_t bytes);
-// grow-only scratch slot `slot` of the context
+// grow-only scratch slot `slot` of the context; the two slots below hold what
+// frames can do without and are given back when an allocation needs the room
+constexpr int kScratchPaths = 17, kScratchLong = 18;
 hr_status scratch(hr_ctx* ctx, int slot, size_t bytes, void** p);
 
 #define HR_CUDA(ctx, call)                                                              \
@@ -187,6 +192,8 @@ const void* device_view(const void* p);
 // Word of hr_asset::d_bounds set by a hierarchy build that changed the strand
 // order (or the hierarchy) and cleared by a BVH build: a refit is then invalid.
 constexpr int kHierChanged = 6;
+constexpr int kEthBounds = 8;
+constexpr size_t kBoundWords = 16;
 
 // Float <-> unsigned with the same order (atomic min / max of floats).
 __device__ __forceinline__ uint32_t ordered_bits(float f) {
@@ -259,29 +266,15 @@ struct LaunchLights {
   float4 xyzw[HR_MAX_LIGHTS];
   float4 rgb[HR_MAX_LIGHTS];
 };
-// Warp-tile schedule carried from one frame of an asset to the next.  The
-// warp tiles whose slowest lane took the most traversal steps (node visits
-// plus primitive tests) in the previous frame are traced first, kHeavyRays
-// rays per warp: a ray that shares its warp with 31 other long rays advances
-// at a fraction of the pace it keeps with few (the slowest full-head ray:
-// ~550 us in its 32-ray tile, ~300 us alone), and these few tiles otherwise
-// set the frame's length.  Each traced lane of such a tile stores its partial
-// sums; the warp that finishes the tile's last hand-out composites its pixels
-// with the same shuffle tree as a whole-warp tile, so the image does not
-// depend on the schedule.  Measured on the full-head frame (FP32, 8 spp):
-// 16 tiles of 4-ray hand-outs took the frame from 0.58 to 0.48 ms alone;
-// 64 tiles, 1 or 2 rays per hand-out or a 60-70% threshold were no better,
-// and spent more warp time.
+// Warp-tile schedule carried from one frame of an asset to the next: the warp
+// tiles whose slowest lane took the most traversal steps (node visits plus
+// primitive tests) in the previous frame are handed out first.
 constexpr uint32_t kHeavyMax = 16;         // heavy tiles per frame, at most
 constexpr uint32_t kHeavyRelPct = 50;      // steps of a heavy tile's slowest lane, at least, in
                                            // percent of the frame's slowest tile
 constexpr uint32_t kHeavyMinSteps = 16;    // and more than this
-constexpr uint32_t kHeavyRays = 4;         // rays (lanes) of a heavy tile per hand-out
-constexpr uint32_t kHeavyItems = 32 / kHeavyRays;
-// Only frames of at most this many warp tiles per resident warp trace heavy
-// tiles: with many tiles per warp the hand-out balances the work by itself
-// (the close full-head view, ~160 tiles per warp, was 1.3% slower with them,
-// the middle one, ~24, 1.3% faster, the far one, ~2.4, 19% faster).
+// Only frames of at most this many warp tiles per resident warp have heavy
+// tiles: with many tiles per warp the hand-out balances the work by itself.
 constexpr uint32_t kHeavyTilesPerWarp = 64;
 // The frame kernel lists the tiles whose step count reaches a threshold (half
 // the previous frame's largest) as candidates, kCandMax at most, and keeps
@@ -299,16 +292,29 @@ struct TileSched {
   uint32_t pad[3];
   uint32_t cand_tile[kCandMax];   // grid index of each candidate tile
   uint32_t cand_steps[kCandMax];  // and its slowest lane's steps
-  uint32_t heavy[kHeavyMax];            // tile origins x0 | y0 << 16, heaviest first
-  uint32_t done[kHeavyMax];             // rays finished per heavy tile
-  uint32_t ray_steps[kHeavyMax * 32];   // per ray of a heavy tile
-  float acc[kHeavyMax * 32 * 3];        // per-lane partial sums of a heavy tile
+  uint32_t heavy[kHeavyMax];      // tile origins x0 | y0 << 16, heaviest first
+};
+
+// Rays put aside by the frame kernel (trace_core.cuh, "long walks"); words 0:
+// none are.
+namespace tr {
+struct LongTile;
+}
+struct LongWork {
+  uint32_t* ctr;       // [0] rays, [1] pool words and [2] tiles taken, [3] rays handed out
+  uint32_t* pool;      // the rays' records
+  uint32_t* ray_at;    // [rays_max] where each record starts (0xffffffff: none)
+  tr::LongTile* tiles; // [tiles_max]
+  uint32_t words, rays_max, tiles_max;
 };
 
 struct FrameArgs {
-  const float4* nodes;     // BVH nodes; a leaf child is ~(global primitive id)
-  const float4* prim_xf;   // [P_total * 3] world -> unit-cylinder rows, by global id
-  const float4* prim_aux;  // [P_total] (material index bits, n_tot, r, a*b)
+  const uint4* nodes;      // BVH nodes; a leaf child is ~(global primitive id)
+  const float4* frame;     // the nodes' grid and the leaves' bounds (Bvh::frame)
+  // World -> unit-cylinder records by global id, two 32-byte sectors each: a
+  // test that misses the outline (most of them) reads rows u and v alone.
+  const float4* prim_uv;   // [P_total * 2] rows u, v
+  const float4* prim_wa;   // [P_total * 2] row w, (material index bits, n_tot, r, a*b)
   const uint32_t* leaf_id; // the single leaf's id when the BVH has one leaf
   const float4* verts;     // strand vertices and thick-hair cross-sections: the
   const float4* xsec;      // segments' start points for FP64 decisions
@@ -332,6 +338,7 @@ struct FrameArgs {
   uint32_t* tile_count;      // the frame's number of warp tiles (written when tile_log is set)
   TileSched* sched;          // plain frame kernel: the heavy-tile schedule, or null
   uint32_t frame_warps;      // with sched: resident warps of the frame kernel
+  LongWork lw;               // plain frame kernel: rays put aside
 };
 
 // Tile geometry of the frame and serving kernels for a given spp: each pixel

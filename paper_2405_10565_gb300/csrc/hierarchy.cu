@@ -103,11 +103,12 @@ __device__ __forceinline__ float3 crossf(float3 a, float3 b) {
 // correctly rounded value, and each offset is the compensated dot product of
 // the stored row with c0, so the stored cylinder passes through c0 to within
 // the offset's own rounding.
-__device__ void write_prim(float4* xf, float4* box, float3 c0, float3 c1, float3 e1, float a, float b) {
+__device__ void write_prim(float4* uv, float4* w, float4* box, float3 c0, float3 c1, float3 e1, float a,
+                           float b) {
   const float3 ax = sub3(c1, c0);
   const float L2 = dotf(ax, ax);
   if (!(L2 > 0.f)) {
-    xf[0] = xf[1] = xf[2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    uv[0] = uv[1] = w[0] = make_float4(0.f, 0.f, 0.f, 0.f);
     box[0] = make_float4(c0.x, c0.y, c0.z, 0.f);
     box[1] = box[0];
     return;
@@ -116,9 +117,9 @@ __device__ void write_prim(float4* xf, float4* box, float3 c0, float3 c1, float3
   const float3 e2 = crossf(t, e1);
   const float ia = 1.0f / a, ib = 1.0f / b;
   const float3 r0 = mul3(e1, ia), r1 = mul3(e2, ib), r2 = mul3(ax, 1.0f / L2);
-  xf[0] = make_float4(r0.x, r0.y, r0.z, -dot_comp(r0, c0));
-  xf[1] = make_float4(r1.x, r1.y, r1.z, -dot_comp(r1, c0));
-  xf[2] = make_float4(r2.x, r2.y, r2.z, -dot_comp(r2, c0));
+  uv[0] = make_float4(r0.x, r0.y, r0.z, -dot_comp(r0, c0));
+  uv[1] = make_float4(r1.x, r1.y, r1.z, -dot_comp(r1, c0));
+  w[0] = make_float4(r2.x, r2.y, r2.z, -dot_comp(r2, c0));
   // half extents of the elliptic disc per axis, grown by 2e-6 relative (the
   // FP32 terms carry a few ulps); the corners are rounded outward
   const float ga = 1.000002f;
@@ -164,7 +165,7 @@ __global__ void k_strand_shape(const float4* __restrict__ verts, const float2* _
 }
 
 __global__ void k_strand_prims(const float4* __restrict__ verts, const float4* __restrict__ sh4,
-                               uint32_t N, uint32_t S, float4* xf, float4* box, float4* aux) {
+                               uint32_t N, uint32_t S, float4* uv, float4* box, float4* wa) {
   const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (uint64_t)N * S) return;
   const uint32_t s = (uint32_t)(idx / S), k = (uint32_t)(idx % S);
@@ -182,8 +183,8 @@ __global__ void k_strand_prims(const float4* __restrict__ verts, const float4* _
     e1 = make_float3(fmaf(b1.x, sh.x, b2.x * sh.y), fmaf(b1.y, sh.x, b2.y * sh.y),
                      fmaf(b1.z, sh.x, b2.z * sh.y));
   }
-  write_prim(xf + idx * 3, box + idx * 2, p0, p1, e1, sh.z, sh.w);
-  aux[idx] = make_float4(__uint_as_float(s), 0.f, r, sh.z * sh.w);
+  write_prim(uv + idx * 2, wa + idx * 2, box + idx * 2, p0, p1, e1, sh.z, sh.w);
+  wa[idx * 2 + 1] = make_float4(__uint_as_float(s), 0.f, r, sh.z * sh.w);
 }
 
 // New strand positions in one pass: each block reads the vertices of
@@ -194,7 +195,7 @@ __global__ void k_strand_prims(const float4* __restrict__ verts, const float4* _
 // k_strand_shape and k_strand_prims do.
 __global__ void k_strand_update(const float4* __restrict__ src, float4* __restrict__ verts,
                                 const float2* __restrict__ shape, uint32_t N, uint32_t S,
-                                uint32_t per_block, float4* xf, float4* box, float4* aux) {
+                                uint32_t per_block, float4* uv, float4* box, float4* wa) {
   extern __shared__ float4 sv[];  // per_block * (S + 1) vertices, then per_block shapes
   const uint32_t s0 = blockIdx.x * per_block;
   const uint32_t ns = min(per_block, N - s0);
@@ -233,8 +234,8 @@ __global__ void k_strand_update(const float4* __restrict__ src, float4* __restri
                        fmaf(b1.z, sh.x, b2.z * sh.y));
     }
     const size_t idx = (size_t)(s0 + ls) * S + k;
-    write_prim(xf + idx * 3, box + idx * 2, p0, p1, e1, sh.z, sh.w);
-    aux[idx] = make_float4(__uint_as_float(s0 + ls), 0.f, r, sh.z * sh.w);
+    write_prim(uv + idx * 2, wa + idx * 2, box + idx * 2, p0, p1, e1, sh.z, sh.w);
+    wa[idx * 2 + 1] = make_float4(__uint_as_float(s0 + ls), 0.f, r, sh.z * sh.w);
   }
 }
 
@@ -738,10 +739,11 @@ __global__ void __launch_bounds__(128, 8) k_fit_cross_sections(const float4* __r
 __global__ void k_eth_material(const float4* __restrict__ verts, uint32_t N, uint32_t S,
                                const uint32_t* __restrict__ order,
                                const uint32_t* __restrict__ cl_first, LevelInfo li, uint32_t E,
-                               float* mat, float* eth_r) {
+                               float* mat, float* eth_r, uint32_t* eth_bounds) {
   // one thread per (thick hair, material float); the last float is the radius
   constexpr uint32_t F = HR_MAT_FLOATS + 1;
   const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx < 6) eth_bounds[idx] = idx < 3 ? 0xffffffffu : 0u;  // for k_eth_prims
   if (idx >= (uint64_t)E * F) return;
   const uint32_t e = (uint32_t)(idx / F), j = (uint32_t)(idx % F);
   uint32_t first, cnt, c, lv;
@@ -759,14 +761,11 @@ __global__ void k_eth_material(const float4* __restrict__ verts, uint32_t N, uin
     eth_r[e] = mean;
 }
 
-// Thick-hair segment (e, k): axis c_k -> c_{k+1}, e1 = e1_k made orthogonal to
-// the axis, semi-axes the larger of the two cross-sections'.
-__global__ void k_eth_prims(const float4* __restrict__ xsec, uint32_t N, uint32_t S, uint32_t E,
-                            const uint32_t* __restrict__ cl_first, LevelInfo li,
-                            const float* __restrict__ eth_r, float4* xf, float4* box,
-                            float4* aux) {
-  const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (uint64_t)E * S) return;
+// One thick-hair segment's record; false for an empty thick hair.
+__device__ __forceinline__ bool eth_prim(const float4* __restrict__ xsec, uint32_t N, uint32_t S,
+                                         const uint32_t* __restrict__ cl_first, const LevelInfo& li,
+                                         const float* __restrict__ eth_r, uint64_t idx, float4* uv,
+                                         float4* box, float4* wa) {
   const uint32_t e = (uint32_t)(idx / S), k = (uint32_t)(idx % S);
   const float4* x0 = xsec + ((size_t)e * (S + 1) + k) * 3;
   const float4 q0 = __ldg(x0), q1 = __ldg(x0 + 1), r0 = __ldg(x0 + 3), r1 = __ldg(x0 + 4);
@@ -784,13 +783,53 @@ __global__ void k_eth_prims(const float4* __restrict__ xsec, uint32_t N, uint32_
   uint32_t first, cnt, c, lv;
   eth_members(li, cl_first, e, &first, &cnt, &c, &lv);
   if (cnt == 0) {  // empty thick hair: never active; records left inert
-    xf[p * 3] = xf[p * 3 + 1] = xf[p * 3 + 2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    uv[p * 2] = uv[p * 2 + 1] = wa[p * 2] = make_float4(0.f, 0.f, 0.f, 0.f);
     box[p * 2] = box[p * 2 + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    aux[p] = make_float4(__uint_as_float(N + e), 0.f, 0.f, 0.f);
-    return;
+    wa[p * 2 + 1] = make_float4(__uint_as_float(N + e), 0.f, 0.f, 0.f);
+    return false;
   }
-  write_prim(xf + p * 3, box + p * 2, c0, c1, e1, a, b);
-  aux[p] = make_float4(__uint_as_float(N + e), (float)cnt, eth_r[e], a * b);
+  write_prim(uv + p * 2, wa + p * 2, box + p * 2, c0, c1, e1, a, b);
+  wa[p * 2 + 1] = make_float4(__uint_as_float(N + e), (float)cnt, eth_r[e], a * b);
+  return true;
+}
+
+// Thick-hair segment (e, k): axis c_k -> c_{k+1}, e1 = e1_k made orthogonal to
+// the axis, semi-axes the larger of the two cross-sections'.  Also the bounds
+// of all their boxes (ordered float bits, cleared by k_eth_material).
+__global__ void k_eth_prims(const float4* __restrict__ xsec, uint32_t N, uint32_t S, uint32_t E,
+                            const uint32_t* __restrict__ cl_first, LevelInfo li,
+                            const float* __restrict__ eth_r, float4* uv, float4* box,
+                            float4* wa, uint32_t* bounds) {
+  const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ uint32_t s_b[6];
+  if (threadIdx.x < 6) s_b[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
+  __syncthreads();
+  const bool live = idx < (uint64_t)E * S &&
+                    eth_prim(xsec, N, S, cl_first, li, eth_r, idx, uv, box, wa);
+  uint32_t b[6];
+  const size_t p = (size_t)N * S + idx;
+  if (live) {
+    const float4 l = box[2 * p], h = box[2 * p + 1];
+    b[0] = ordered_bits(l.x), b[1] = ordered_bits(l.y), b[2] = ordered_bits(l.z);
+    b[3] = ordered_bits(h.x), b[4] = ordered_bits(h.y), b[5] = ordered_bits(h.z);
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const uint32_t v = i < 3 ? __reduce_min_sync(0xffffffffu, live ? b[i] : 0xffffffffu)
+                             : __reduce_max_sync(0xffffffffu, live ? b[i] : 0u);
+    if ((threadIdx.x & 31) == 0) {
+      if (i < 3) atomicMin(&s_b[i], v); else atomicMax(&s_b[i], v);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {  // nothing to do once another block has reached as far
+    const uint32_t v = s_b[threadIdx.x], g = __ldcg(bounds + threadIdx.x);
+    if (threadIdx.x < 3) {
+      if (v < g) atomicMin(bounds + threadIdx.x, v);
+    } else if (v > g) {
+      atomicMax(bounds + threadIdx.x, v);
+    }
+  }
 }
 
 // Scene bounds over all primitive boxes (ordered-bit atomics).
@@ -841,11 +880,13 @@ hr_status scene_bounds(hr_ctx* ctx, hr_asset* a, uint64_t n, cudaStream_t st = n
 hr_status build_strand_prims(hr_ctx* ctx, hr_asset* a) {
   const uint64_t n = (uint64_t)a->N * a->S;
   a->n_prims_total = (uint32_t)n;
-  HR_TRY(dalloc(ctx, (void**)&a->prim_xf, n * 3 * sizeof(float4), "strand records"));
+  HR_TRY(dalloc(ctx, (void**)&a->prim_uv, n * 2 * sizeof(float4), "strand records"));
   HR_TRY(dalloc(ctx, (void**)&a->prim_box, n * 2 * sizeof(float4), "strand boxes"));
-  HR_TRY(dalloc(ctx, (void**)&a->prim_aux, n * sizeof(float4), "strand aux"));
-  HR_TRY(dalloc(ctx, (void**)&a->d_bounds, 8 * sizeof(uint32_t), "scene bounds"));
+  HR_TRY(dalloc(ctx, (void**)&a->prim_wa, n * 2 * sizeof(float4), "strand aux"));
+  HR_TRY(dalloc(ctx, (void**)&a->d_bounds, kBoundWords * sizeof(uint32_t), "scene bounds"));
   a->bytes += n * 6 * sizeof(float4);
+  k_init_bounds<<<1, 32, 0, ctx_stream(ctx)>>>(a->d_bounds + kEthBounds);  // no thick hairs yet
+  HR_LAUNCHED(ctx);
   return refresh_strand_prims(ctx, a);
 }
 
@@ -858,7 +899,7 @@ hr_status update_strands(hr_ctx* ctx, hr_asset* a, const float4* src_dev, cudaSt
   const size_t smem = ((size_t)per_block * S1 + per_block) * sizeof(float4);
   const uint32_t blocks = (a->N + per_block - 1) / per_block;
   k_strand_update<<<blocks, 256, smem, st>>>(src_dev, a->verts, a->shape, a->N, a->S, per_block,
-                                             a->prim_xf, a->prim_box, a->prim_aux);
+                                             a->prim_uv, a->prim_box, a->prim_wa);
   HR_LAUNCHED(ctx);
   return scene_bounds(ctx, a, (uint64_t)a->N * a->S, st);
 }
@@ -871,8 +912,8 @@ hr_status refresh_strand_prims(hr_ctx* ctx, hr_asset* a) {
   k_strand_shape<<<(a->N + 255) / 256, 256, 0, st>>>(a->verts, a->shape, a->N, a->S, sh4);
   HR_LAUNCHED(ctx);
   k_strand_prims<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a->verts, sh4, a->N, a->S,
-                                                             a->prim_xf, a->prim_box,
-                                                             a->prim_aux);
+                                                             a->prim_uv, a->prim_box,
+                                                             a->prim_wa);
   HR_LAUNCHED(ctx);
   return scene_bounds(ctx, a, n);
 }
@@ -962,21 +1003,21 @@ hr_status hierarchy_finish(hr_ctx* ctx, hr_asset* a, const LevelInfo& li, uint64
   // grow the primitive arrays to strands + thick hairs (strand part copied)
   const uint64_t ns = (uint64_t)N * S;
   if (a->n_prims_total != total) {
-    float4 *xf = nullptr, *bx = nullptr, *ax = nullptr;
-    HR_TRY(dalloc(ctx, (void**)&xf, total * 3 * sizeof(float4), "records"));
+    float4 *uv = nullptr, *bx = nullptr, *wa = nullptr;
+    HR_TRY(dalloc(ctx, (void**)&uv, total * 2 * sizeof(float4), "records"));
     HR_TRY(dalloc(ctx, (void**)&bx, total * 2 * sizeof(float4), "boxes"));
-    HR_TRY(dalloc(ctx, (void**)&ax, total * sizeof(float4), "aux"));
-    HR_CUDA(ctx, cudaMemcpyAsync(xf, a->prim_xf, ns * 3 * sizeof(float4), cudaMemcpyDeviceToDevice, st));
+    HR_TRY(dalloc(ctx, (void**)&wa, total * 2 * sizeof(float4), "aux"));
+    HR_CUDA(ctx, cudaMemcpyAsync(uv, a->prim_uv, ns * 2 * sizeof(float4), cudaMemcpyDeviceToDevice, st));
     HR_CUDA(ctx, cudaMemcpyAsync(bx, a->prim_box, ns * 2 * sizeof(float4), cudaMemcpyDeviceToDevice, st));
-    HR_CUDA(ctx, cudaMemcpyAsync(ax, a->prim_aux, ns * sizeof(float4), cudaMemcpyDeviceToDevice, st));
+    HR_CUDA(ctx, cudaMemcpyAsync(wa, a->prim_wa, ns * 2 * sizeof(float4), cudaMemcpyDeviceToDevice, st));
     HR_CUDA(ctx, cudaStreamSynchronize(st));
     const uint64_t old = a->n_prims_total;
-    dfree(ctx, a->prim_xf, old * 3 * sizeof(float4));
+    dfree(ctx, a->prim_uv, old * 2 * sizeof(float4));
     dfree(ctx, a->prim_box, old * 2 * sizeof(float4));
-    dfree(ctx, a->prim_aux, old * sizeof(float4));
-    a->prim_xf = xf;
+    dfree(ctx, a->prim_wa, old * 2 * sizeof(float4));
+    a->prim_uv = uv;
     a->prim_box = bx;
-    a->prim_aux = ax;
+    a->prim_wa = wa;
     a->n_prims_total = (uint32_t)total;
   }
   // The scene bounds (for the BVH's Morton codes) are those of the strand
@@ -1009,12 +1050,14 @@ hr_status hierarchy_finish(hr_ctx* ctx, hr_asset* a, const LevelInfo& li, uint64
   }
   k_eth_material<<<(unsigned)((E * (HR_MAT_FLOATS + 1) + 127) / 128), 128, 0, st>>>(a->verts, N, S, a->order,
                                                              a->cl_first, li, (uint32_t)E,
-                                                             a->mat, eth_r);
+                                                             a->mat, eth_r,
+      a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   const uint64_t ne = E * S;
   k_eth_prims<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(a->xsec, N, S, (uint32_t)E,
-                                                           a->cl_first, li, eth_r, a->prim_xf,
-                                                           a->prim_box, a->prim_aux);
+                                                           a->cl_first, li, eth_r, a->prim_uv,
+                                                           a->prim_box, a->prim_wa,
+                                                           a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   return HR_OK;
 }
@@ -1067,10 +1110,12 @@ hr_status rebuild_eth_records(hr_ctx* ctx, hr_asset* a) {
   float* eth_r = nullptr;
   HR_TRY(scratch(ctx, 5, (size_t)E * sizeof(float), (void**)&eth_r));
   k_eth_material<<<(unsigned)(((uint64_t)E * (HR_MAT_FLOATS + 1) + 127) / 128), 128, 0, st>>>(
-      a->verts, N, S, a->order, a->cl_first, li, E, a->mat, eth_r);
+      a->verts, N, S, a->order, a->cl_first, li, E, a->mat, eth_r,
+      a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   k_eth_prims<<<(unsigned)(((uint64_t)E * S + 255) / 256), 256, 0, st>>>(
-      a->xsec, N, S, E, a->cl_first, li, eth_r, a->prim_xf, a->prim_box, a->prim_aux);
+      a->xsec, N, S, E, a->cl_first, li, eth_r, a->prim_uv, a->prim_box, a->prim_wa,
+      a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   return HR_OK;
 }

@@ -24,6 +24,13 @@ namespace tr {
 
 #define kInf __int_as_float(0x7f800000)
 constexpr int kStack = 64;
+// Blocks an SM of the tracing kernels (72 registers; the node visits and leaf
+// tests do not spill, the shading does a little).  With 5, 6, 7 and 8: the far
+// view of the full head 1.31, 1.31, 1.31, 1.45 ms a call, its close view 4.05,
+// 3.85, 3.65, 3.60, the 4K frame of straight hair 10.5, 10.0, 9.6, 9.6, the
+// curled clusters 1.47, 1.44, 1.40, 1.43 (the last blocks cost L1: shared
+// memory, stacks and more rays' records).
+constexpr int kTraceBlocks = 7;
 
 __device__ __forceinline__ uint64_t splitmix_out(uint64_t seed, uint64_t i) {
   uint64_t z = seed + (i + 1) * 0x9E3779B97F4A7C15ull;
@@ -82,11 +89,10 @@ struct RayKey {  // what rebuilds the ray precisely: the sample id and the re-ba
 // than the bound; kBorder when the rounding could change the outcome; else
 // kHit with the nearest root t in (0, tmax] (axial coordinate in [0, 1]),
 // and its error bound terr.
-// M = |o.x| + |o.y| + |o.z| of the ray.
-__device__ __forceinline__ int intersect32(const float4* __restrict__ xf, const float3 o,
-                                           const float3 d, const float M, const float tmax,
-                                           float& t_hit, float& terr) {
-  const float4 r0 = __ldg(xf), r1 = __ldg(xf + 1), r2 = __ldg(xf + 2);
+// r0, r1: the record's rows u and v; M = |o.x| + |o.y| + |o.z| of the ray.
+__device__ __forceinline__ int intersect32(const FrameArgs& fa, const uint32_t id, const float4 r0,
+                                           const float4 r1, const float3 o, const float3 d,
+                                           const float M, const float tmax, float& t_hit, float& terr) {
   const float u0 = fmaf(r0.x, o.x, fmaf(r0.y, o.y, fmaf(r0.z, o.z, r0.w)));
   const float v0 = fmaf(r1.x, o.x, fmaf(r1.y, o.y, fmaf(r1.z, o.z, r1.w)));
   const float du = fmaf(r0.x, d.x, fmaf(r0.y, d.y, r0.z * d.z));
@@ -116,6 +122,7 @@ __device__ __forceinline__ int intersect32(const float4* __restrict__ xf, const 
   const float eroot = border ? sqrtf(dh * inv) : dh * half * (0.5f / g);
   terr = fmaf(e, sqrtf(inv), fmaf(4.f * kEps32, magt, eroot));
   if (tp + terr <= 0.f || tm - terr > tmax) return kMiss;
+  const float4 r2 = __ldg(fa.prim_wa + 2 * (size_t)id);
   const float w0 = fmaf(r2.x, o.x, fmaf(r2.y, o.y, fmaf(r2.z, o.z, r2.w)));
   const float dw = fmaf(r2.x, d.x, fmaf(r2.y, d.y, r2.z * d.z));
   // axial coordinate of each root, and its error bound (the row's rounding
@@ -204,6 +211,13 @@ __device__ __forceinline__ df df_sqrt(df a) {
   return df_fast(r, __fdiv_rn(__fadd_rn(fmaf(-r, r, a.hi), a.lo), 2.f * r));
 }
 
+// Exact bounds of the BVH's leaves.
+__device__ __forceinline__ void root_box(const FrameArgs& fa, float3& lo, float3& hi) {
+  const uint32_t* b = reinterpret_cast<const uint32_t*>(fa.frame + 3);
+  lo = f3(from_ordered(__ldg(b)), from_ordered(__ldg(b + 1)), from_ordered(__ldg(b + 2)));
+  hi = f3(from_ordered(__ldg(b + 3)), from_ordered(__ldg(b + 4)), from_ordered(__ldg(b + 5)));
+}
+
 // The FP32 ray of a sample: the direction normalised in FP32 (correctly
 // rounded steps, so |d| = 1 within a few ulps), and the origin moved to a
 // little before the ray's entry into the scene's bounding box (the root
@@ -219,14 +233,15 @@ __device__ __forceinline__ void primary_ray(const FrameArgs& fa, uint64_t sid, f
   d = f3(__fmul_rn(vx, il), __fmul_rn(vy, il), __fmul_rn(vz, il));
   float s_off = 0.f;
   if (fa.n_prims >= 2) {
-    const float4 n0 = __ldg(fa.nodes), n1 = __ldg(fa.nodes + 1), n2 = __ldg(fa.nodes + 2);
+    float3 blo, bhi;
+    root_box(fa, blo, bhi);
     const float3 oo = f3(ry.o[0].hi, ry.o[1].hi, ry.o[2].hi);
     const float3 inv = f3(1.0f / (fabsf(d.x) > 1e-12f ? d.x : copysignf(1e-12f, d.x)),
                           1.0f / (fabsf(d.y) > 1e-12f ? d.y : copysignf(1e-12f, d.y)),
                           1.0f / (fabsf(d.z) > 1e-12f ? d.z : copysignf(1e-12f, d.z)));
-    const float lx = (fminf(n0.x, n1.x) - oo.x) * inv.x, hx = (fmaxf(n0.y, n1.y) - oo.x) * inv.x;
-    const float ly = (fminf(n0.z, n1.z) - oo.y) * inv.y, hy = (fmaxf(n0.w, n1.w) - oo.y) * inv.y;
-    const float lz = (fminf(n2.x, n2.z) - oo.z) * inv.z, hz = (fmaxf(n2.y, n2.w) - oo.z) * inv.z;
+    const float lx = (blo.x - oo.x) * inv.x, hx = (bhi.x - oo.x) * inv.x;
+    const float ly = (blo.y - oo.y) * inv.y, hy = (bhi.y - oo.y) * inv.y;
+    const float lz = (blo.z - oo.z) * inv.z, hz = (bhi.z - oo.z) * inv.z;
     const float t0 = fmaxf(fmaxf(fminf(lx, hx), fminf(ly, hy)), fminf(lz, hz));
     const float t1 = fminf(fminf(fmaxf(lx, hx), fmaxf(ly, hy)), fmaxf(lz, hz));
     // 2^-10 before the FP32 entry: far more than the slab test's rounding
@@ -253,8 +268,8 @@ static __device__ __noinline__ bool refine(const FrameArgs& fa, const RayKey& rk
                                            float t_est, float& t_hi, float& t_lo) {
   PreciseRay ry;
   camera_ray_dw(fa.cam, fa.seed, fa.spp, rk.sid, ry);
-  const float4* xf = fa.prim_xf + 3 * (size_t)id;
-  const float4 r0 = __ldg(xf), r1 = __ldg(xf + 1), r2 = __ldg(xf + 2);
+  const float4 r0 = __ldg(fa.prim_uv + 2 * (size_t)id), r1 = __ldg(fa.prim_uv + 2 * (size_t)id + 1),
+               r2 = __ldg(fa.prim_wa + 2 * (size_t)id);
   const uint32_t S = fa.S, NS = fa.N * fa.S;
   float4 c0;
   if (id < NS)
@@ -313,21 +328,39 @@ static __device__ __noinline__ bool refine(const FrameArgs& fa, const RayKey& rk
 // Entries order by (t, tr, id).
 constexpr uint32_t kIdMask = 0x3fffffffu, kOpaque = 0x40000000u, kExact = 0x80000000u;
 constexpr uint32_t kNoEntry = kIdMask;  // an empty slot (t = inf)
-template <int KMAX>
-struct KBuf {
-  float t[KMAX];
-  float tr[KMAX];
-  uint32_t id[KMAX];
+// The ray and its hits live in shared memory, a column per thread (no bank
+// conflicts), or one per warp where the warp works on one ray: the node visits
+// need only the slab constants in registers, and the shading loops over the
+// entries instead of being unrolled over them.  With them in registers the
+// frame kernel needed 128 registers (16 warps an SM) and K copies of the
+// shading code.
+template <int KMAX, int COLS>
+struct RayMem {
+  float o[3][COLS], d[3][COLS];  // the FP32 ray
+  float M[COLS];                 // |o.x| + |o.y| + |o.z|
+  float s_off[COLS];             // RayKey
+  uint32_t sid[2][COLS];
+  float t[KMAX][COLS], tr[KMAX][COLS];
+  uint32_t id[KMAX][COLS];
 };
 
-template <int KMAX>
-__device__ __forceinline__ void kbuf_init(KBuf<KMAX>& kb) {
-#pragma unroll
-  for (int j = 0; j < KMAX; ++j) {
-    kb.t[j] = kInf;
-    kb.tr[j] = 0.f;
-    kb.id[j] = kNoEntry;
-  }
+template <int KMAX, int COLS>
+__device__ __forceinline__ void ray_store(RayMem<KMAX, COLS>& rm, uint32_t c, const float3 o,
+                                          const float3 d, const RayKey& rk) {
+  rm.o[0][c] = o.x; rm.o[1][c] = o.y; rm.o[2][c] = o.z;
+  rm.d[0][c] = d.x; rm.d[1][c] = d.y; rm.d[2][c] = d.z;
+  rm.M[c] = fabsf(o.x) + fabsf(o.y) + fabsf(o.z);
+  rm.s_off[c] = rk.s_off;
+  rm.sid[0][c] = (uint32_t)rk.sid;
+  rm.sid[1][c] = (uint32_t)(rk.sid >> 32);
+}
+template <int KMAX, int COLS>
+__device__ __forceinline__ float3 ray_o(const RayMem<KMAX, COLS>& rm, uint32_t c) {
+  return f3(rm.o[0][c], rm.o[1][c], rm.o[2][c]);
+}
+template <int KMAX, int COLS>
+__device__ __forceinline__ float3 ray_d(const RayMem<KMAX, COLS>& rm, uint32_t c) {
+  return f3(rm.d[0][c], rm.d[1][c], rm.d[2][c]);
 }
 
 __device__ __forceinline__ bool key_less(float t, float tr, uint32_t id, float t2, float tr2,
@@ -335,35 +368,33 @@ __device__ __forceinline__ bool key_less(float t, float tr, uint32_t id, float t
   return t < t2 || (t == t2 && (tr < tr2 || (tr == tr2 && (id & kIdMask) < (id2 & kIdMask))));
 }
 
-// Insert keeping the k nearest by (t, tr, id): the candidate bubbles through
-// the sorted slots and whatever falls off the end is dropped.
-template <int KMAX>
-__device__ __forceinline__ void kbuf_insert(KBuf<KMAX>& kb, const uint32_t k, float t, float tr,
-                                            uint32_t id) {
-#pragma unroll
-  for (int j = 0; j < KMAX; ++j) {
-    if (j < (int)k && key_less(t, tr, id, kb.t[j], kb.tr[j], kb.id[j])) {
-      float a = kb.t[j]; kb.t[j] = t; t = a;
-      float r = kb.tr[j]; kb.tr[j] = tr; tr = r;
-      uint32_t b = kb.id[j]; kb.id[j] = id; id = b;
-    }
+// The entry (t, tr, id) into the sorted places 0 .. j, the last one's old
+// entry falling off.
+template <int KMAX, int COLS>
+__device__ __forceinline__ void kbuf_place(RayMem<KMAX, COLS>& rm, uint32_t c, int j, float t, float tr,
+                                           uint32_t id) {
+  for (; j > 0 && key_less(t, tr, id, rm.t[j - 1][c], rm.tr[j - 1][c], rm.id[j - 1][c]); --j) {
+    rm.t[j][c] = rm.t[j - 1][c];
+    rm.tr[j][c] = rm.tr[j - 1][c];
+    rm.id[j][c] = rm.id[j - 1][c];
   }
+  rm.t[j][c] = t;
+  rm.tr[j][c] = tr;
+  rm.id[j][c] = id;
 }
 
 // The search cut: the depth of the k-th entry, or of the first opaque entry
 // when it comes earlier (nothing behind an opaque hit is composited).
-template <int KMAX>
-__device__ __forceinline__ float kbuf_cut(const KBuf<KMAX>& kb, const uint32_t k) {
-  float r = kInf;
-#pragma unroll
-  for (int j = KMAX - 1; j >= 0; --j)
-    if (j < (int)k && (j == (int)k - 1 || (kb.id[j] & kOpaque))) r = kb.t[j];
-  return r;
+template <int KMAX, int COLS>
+__device__ __forceinline__ float kbuf_cut(const RayMem<KMAX, COLS>& rm, uint32_t c, const uint32_t k) {
+  uint32_t j = 0;
+  while (j + 1 < k && !(rm.id[j][c] & kOpaque)) ++j;
+  return rm.t[j][c];
 }
 
 struct Counts {
   uint32_t nodes, tests, sshade, eshade, hits, rays, precise_tests, precise_entries;
-  uint32_t steps;  // node visits plus primitive tests, counted in every kernel (tile schedule)
+  uint32_t steps;  // node visits plus primitive tests, counted by the frame kernel (tile schedule)
 };
 
 // Test primitive `id` (a leaf names its global primitive id) and keep it in
@@ -376,146 +407,205 @@ struct Counts {
 // Otherwise the hit is decided precisely, and so is every FP32 entry within
 // errmax of its precise depth (the only entries whose order against it the
 // FP32 depths leave open).
-template <int KMAX, bool COUNT>
-__device__ __forceinline__ void leaf_test(const FrameArgs& fa, const RayKey& rk, uint32_t id,
-                                          const float3 o, const float3 d, const float M,
-                                          KBuf<KMAX>& kb, float& tcut, float& errmax, Counts& cn) {
-  float th, terr;
-  ++cn.steps;
-  if (COUNT) ++cn.tests;
-  const int r =
-      intersect32(fa.prim_xf + 3 * (size_t)id, o, d, M, tcut + errmax, th, terr);
-  if (r == kMiss) return;
+template <int KMAX, int COLS, bool COUNT>
+__device__ __forceinline__ void keep_hit(const FrameArgs& fa, RayMem<KMAX, COLS>& rm, uint32_t c,
+                                         uint32_t id, int r, float th, float terr, float& tcut,
+                                         float& errmax, Counts& cn) {
+  const uint32_t k = KMAX == 1 ? 1u : fa.k;
   const float slack = terr + errmax;
-  bool need = r == kBorder || terr > kTieRel * (rk.s_off + th) || th >= tcut - slack;
-  if (!need) {
-#pragma unroll
-    for (int j = 0; j < KMAX; ++j)
-      if (j < (int)fa.k && fabsf(th - kb.t[j]) <= slack) need = true;
-  }
-  uint32_t word = id | (__ldg(&fa.prim_aux[id].y) == 0.f ? kOpaque : 0u);
+  const float s_off = rm.s_off[c];
+  bool need = r == kBorder || terr > kTieRel * (s_off + th) || th >= tcut - slack;
+  for (uint32_t j = 0; j < k; ++j) need |= fabsf(th - rm.t[j][c]) <= slack;
+  uint32_t word = id | (id < fa.N * fa.S ? kOpaque : 0u);  // strand ids come first
   float tr = 0.f;
   if (need) {
+    const RayKey rk{rm.sid[0][c] | (uint64_t)rm.sid[1][c] << 32, s_off};
     if (COUNT) ++cn.precise_tests;
     float tl;
     if (!refine(fa, rk, id, th, th, tl)) return;
     tr = tl;
     word |= kExact;
     bool moved = false;
-#pragma unroll
-    for (int j = 0; j < KMAX; ++j) {
-      if (j < (int)fa.k && kb.t[j] < kInf && !(kb.id[j] & kExact) &&
-          fabsf(th - kb.t[j]) <= errmax) {
+#pragma unroll 1
+    for (uint32_t j = 0; j < k; ++j) {
+      const float t = rm.t[j][c];
+      if (t < kInf && !(rm.id[j][c] & kExact) && fabsf(th - t) <= errmax) {
         float h, l;
         if (COUNT) ++cn.precise_entries;
-        if (refine(fa, rk, kb.id[j] & kIdMask, kb.t[j], h, l)) {
-          kb.t[j] = h;
-          kb.tr[j] = l;
-          kb.id[j] |= kExact;
+        if (refine(fa, rk, rm.id[j][c] & kIdMask, t, h, l)) {
+          rm.t[j][c] = h;
+          rm.tr[j][c] = l;
+          rm.id[j][c] |= kExact;
         } else {  // not expected for an FP32 hit inside its bounds; dropped if it happens
-          kb.t[j] = kInf;
-          kb.tr[j] = 0.f;
-          kb.id[j] = kNoEntry;
+          rm.t[j][c] = kInf;
+          rm.tr[j][c] = 0.f;
+          rm.id[j][c] = kNoEntry;
         }
         moved = true;
       }
     }
     if (moved) {  // refined depths moved by at most errmax: restore the order
-#pragma unroll
-      for (int i = 0; i + 1 < KMAX; ++i)
-#pragma unroll
-        for (int j = 0; j + 1 < KMAX - i; ++j)
-          if (key_less(kb.t[j + 1], kb.tr[j + 1], kb.id[j + 1], kb.t[j], kb.tr[j], kb.id[j])) {
-            float a = kb.t[j]; kb.t[j] = kb.t[j + 1]; kb.t[j + 1] = a;
-            float q = kb.tr[j]; kb.tr[j] = kb.tr[j + 1]; kb.tr[j + 1] = q;
-            uint32_t b = kb.id[j]; kb.id[j] = kb.id[j + 1]; kb.id[j + 1] = b;
-          }
+#pragma unroll 1
+      for (uint32_t i = 1; i < k; ++i) kbuf_place(rm, c, (int)i, rm.t[i][c], rm.tr[i][c], rm.id[i][c]);
     }
   } else {
     errmax = fmaxf(errmax, terr);
   }
-  kbuf_insert<KMAX>(kb, fa.k, th, tr, word);
-  tcut = kbuf_cut<KMAX>(kb, fa.k);
+  if (key_less(th, tr, word, rm.t[k - 1][c], rm.tr[k - 1][c], rm.id[k - 1][c]))
+    kbuf_place(rm, c, (int)k - 1, th, tr, word);
+  tcut = kbuf_cut(rm, c, k);
 }
 
-// K nearest hits of one ray.  Returns false when the traversal stack overflowed
-// (the far subtree was dropped; counted by the caller, never expected).
+template <int KMAX, int COLS, bool COUNT>
+__device__ __forceinline__ void leaf_test(const FrameArgs& fa, RayMem<KMAX, COLS>& rm, uint32_t id,
+                                          float& tcut, float& errmax, Counts& cn) {
+  const uint32_t c = threadIdx.x;
+  float th, terr;
+  if (COUNT) ++cn.tests;
+  const float4 r0 = __ldg(fa.prim_uv + 2 * (size_t)id), r1 = __ldg(fa.prim_uv + 2 * (size_t)id + 1);
+  const int r = intersect32(fa, id, r0, r1, ray_o(rm, c), ray_d(rm, c), rm.M[c], tcut + errmax, th, terr);
+  if (r != kMiss) keep_hit<KMAX, COLS, COUNT>(fa, rm, c, id, r, th, terr, tcut, errmax, cn);
+}
+
+// A ray against the node boxes.  The plane at grid coordinate q is met at
+// depth (lo + q step - o) / d.  A byte permutation of the box word with 2^23's
+// bits gives 2^23 + q as a float, and picks the near or the far plane by the
+// ray's direction at no further cost, so a plane takes one permutation and one
+// FMA with scale = step / d and offset = (lo - o) / d - 2^23 scale.  The
+// offset's rounding is at most half a step of depth, which the boxes' extra
+// step covers.  A zero direction component would turn the products into
+// inf - inf, so its sign is kept and its magnitude floored.
+struct Slabs {
+  float3 scale, off;
+  uint32_t nx, ny, nz;  // permutation that picks the near plane (xor kFar: the far one)
+};
+constexpr uint32_t kNearLo = 0x7610u, kFar = 0x0022u, kTwo23 = 0x4b000000u;
+__device__ __forceinline__ void slab_axis(float o, float d, float lo, float step, float& scale,
+                                          float& off, uint32_t& sel) {
+  const float inv = 1.0f / (fabsf(d) > 1e-12f ? d : copysignf(1e-12f, d));
+  scale = step * inv;
+  off = fmaf(-8388608.f, scale, (lo - o) * inv);
+  sel = inv < 0.f ? kNearLo ^ kFar : kNearLo;
+}
+__device__ __forceinline__ Slabs ray_slabs(const FrameArgs& fa, const float3 o, const float3 d) {
+  const float4 lo = __ldg(fa.frame), st = __ldg(fa.frame + 1);
+  Slabs s;
+  slab_axis(o.x, d.x, lo.x, st.x, s.scale.x, s.off.x, s.nx);
+  slab_axis(o.y, d.y, lo.y, st.y, s.scale.y, s.off.y, s.ny);
+  slab_axis(o.z, d.z, lo.z, st.z, s.scale.z, s.off.z, s.nz);
+  return s;
+}
+__device__ __forceinline__ float slab_t(uint32_t w, uint32_t sel, float scale, float off) {
+  return fmaf(__uint_as_float(__byte_perm(w, kTwo23, sel)), scale, off);
+}
+// Entry depth (not below 0) of a child's box; false when the ray leaves it
+// before or enters it after tmax.
+__device__ __forceinline__ bool slab_test(const Slabs& s, const uint4 c, float tmax, float& t_in) {
+  t_in = fmaxf(fmaxf(slab_t(c.x, s.nx, s.scale.x, s.off.x), slab_t(c.y, s.ny, s.scale.y, s.off.y)),
+               fmaxf(slab_t(c.z, s.nz, s.scale.z, s.off.z), 0.f));
+  const float t_out = fminf(fminf(slab_t(c.x, s.nx ^ kFar, s.scale.x, s.off.x),
+                                  slab_t(c.y, s.ny ^ kFar, s.scale.y, s.off.y)),
+                            fminf(slab_t(c.z, s.nz ^ kFar, s.scale.z, s.off.z), tmax));
+  return t_in <= t_out;
+}
+
+// A lane's walk: the next node (kDone: none), the pending ones, the search cut
+// and the widest bound of the FP32 hits kept.
+constexpr int kDone = (int)0x80000000;
+constexpr int kLeafWait = 3;
+struct Walk {
+  int node, sp;
+  float tcut, errmax;
+  bool ok;  // false once the traversal stack overflowed (a far subtree was dropped; never expected)
+};
+
+template <int KMAX, int COLS>
+__device__ __forceinline__ void kbuf_clear(RayMem<KMAX, COLS>& rm, uint32_t c) {
+#pragma unroll
+  for (int j = 0; j < KMAX; ++j) {
+    rm.t[j][c] = kInf;
+    rm.tr[j][c] = 0.f;
+    rm.id[j][c] = kNoEntry;
+  }
+}
+
+__device__ __forceinline__ Walk walk_begin(const FrameArgs& fa, bool live) {
+  return Walk{!live || fa.n_prims == 0 ? kDone : (fa.n_prims == 1 ? ~(int)__ldg(fa.leaf_id) : 0), 0, kInf,
+              0.f, true};
+}
+
+// Walks on with the rays of the warp, one per lane, toward their K nearest
+// hits; a lane that has used up `steps` node visits and tests stops where it
+// is.  Whole warps call it.  Returns the steps that the lane has left.
 // Boxes are culled against the cut widened by the FP32 hits' depth bound and
 // by 2 kTieRel of the absolute depth, so that no hit the precise ordering
 // would keep is lost to FP32 rounding of the slab tests.
+// A lane that arrives at a leaf waits until kLeafWait eighths of the lanes still
+// at work are at one: a leaf test is several times as long as a node visit,
+// and one lane in seven is at a leaf on average, so tested at once they would
+// run with a few lanes each.  With 1, 2, 3, 4 and 6 eighths the 4K frame of
+// straight hair took (whole calls, before long walks were put aside) 14.3,
+// 14.1, 14.1, 14.1 and 15.2 ms, the close view of the full head 4.21, 4.15,
+// 4.14, 4.20 and 4.48 ms.
 template <int KMAX, bool COUNT>
-__device__ __forceinline__ bool traverse(const FrameArgs& fa, const RayKey& rk, const float3 o,
-                                         const float3 d, KBuf<KMAX>& kb, Counts& cn) {
-  kbuf_init<KMAX>(kb);
-  if (fa.n_prims == 0) return true;
-  float tcut = kInf, errmax = 0.f;
-  const float M = fabsf(o.x) + fabsf(o.y) + fabsf(o.z);
-  if (fa.n_prims == 1) {
-    leaf_test<KMAX, COUNT>(fa, rk, __ldg(fa.leaf_id), o, d, M, kb, tcut, errmax, cn);
-    return true;
-  }
-  // a zero direction component would turn the slab products into inf - inf;
-  // keep its sign and floor its magnitude so every slab value stays ordered
-  const float3 inv = f3(1.0f / (fabsf(d.x) > 1e-12f ? d.x : copysignf(1e-12f, d.x)),
-                        1.0f / (fabsf(d.y) > 1e-12f ? d.y : copysignf(1e-12f, d.y)),
-                        1.0f / (fabsf(d.z) > 1e-12f ? d.z : copysignf(1e-12f, d.z)));
-  const float3 ooi = f3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
-  int stack[kStack];
-  int sp = 0;
-  int node = 0;
-  bool ok = true;
+__device__ __forceinline__ int walk_on(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm, Walk& w,
+                                       int* stack, int steps, Counts& cn) {
+  const Slabs sl = ray_slabs(fa, ray_o(rm, threadIdx.x), ray_d(rm, threadIdx.x));
+  const float pad = 2.f * kTieRel * rm.s_off[threadIdx.x];
+  float tcut = w.tcut, errmax = w.errmax;
+  int sp = w.sp, node = w.node, stopped = kDone;
   for (;;) {
     if (node >= 0) {
-      const float4* nd = fa.nodes + 4 * (size_t)node;
-      const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
-      ++cn.steps;
+      const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
+      --steps;
       if (COUNT) ++cn.nodes;
-      const float tb = fmaf(tcut + errmax, 1.f + 2.f * kTieRel, 2.f * kTieRel * rk.s_off);
-      // child 0
-      float lx = fmaf(n0.x, inv.x, -ooi.x), hx = fmaf(n0.y, inv.x, -ooi.x);
-      float ly = fmaf(n0.z, inv.y, -ooi.y), hy = fmaf(n0.w, inv.y, -ooi.y);
-      float lz = fmaf(n2.x, inv.z, -ooi.z), hz = fmaf(n2.y, inv.z, -ooi.z);
-      const float a0 = fmaxf(fmaxf(fminf(lx, hx), fminf(ly, hy)), fmaxf(fminf(lz, hz), 0.f));
-      const float b0 = fminf(fminf(fmaxf(lx, hx), fmaxf(ly, hy)), fminf(fmaxf(lz, hz), tb));
-      // child 1
-      lx = fmaf(n1.x, inv.x, -ooi.x); hx = fmaf(n1.y, inv.x, -ooi.x);
-      ly = fmaf(n1.z, inv.y, -ooi.y); hy = fmaf(n1.w, inv.y, -ooi.y);
-      lz = fmaf(n2.z, inv.z, -ooi.z); hz = fmaf(n2.w, inv.z, -ooi.z);
-      const float a1 = fmaxf(fmaxf(fminf(lx, hx), fminf(ly, hy)), fmaxf(fminf(lz, hz), 0.f));
-      const float b1 = fminf(fminf(fmaxf(lx, hx), fmaxf(ly, hy)), fminf(fmaxf(lz, hz), tb));
-      const bool h0 = a0 <= b0, h1 = a1 <= b1;
-      const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
+      const float tb = fmaf(tcut + errmax, 1.f + 2.f * kTieRel, pad);
+      float a0, a1;
+      const bool h0 = slab_test(sl, k0, tb, a0), h1 = slab_test(sl, k1, tb, a1);
+      const int c0 = (int)k0.w, c1 = (int)k1.w;
       if (h0 && h1) {
         const bool first0 = a0 <= a1;
-        const int nearc = first0 ? c0 : c1, farc = first0 ? c1 : c0;
+        node = first0 ? c0 : c1;
         if (sp < kStack)
-          stack[sp++] = farc;
+          stack[sp++] = first0 ? c1 : c0;
         else
-          ok = false;
-        node = nearc;
-        continue;
-      }
-      if (h0 || h1) {
+          w.ok = false;
+      } else if (h0 || h1) {
         node = h0 ? c0 : c1;
-        continue;
+      } else {
+        node = sp ? stack[--sp] : kDone;
       }
-    } else {
-      leaf_test<KMAX, COUNT>(fa, rk, (uint32_t)(~node), o, d, M, kb, tcut, errmax, cn);
     }
-    if (sp == 0) break;
-    node = stack[--sp];
+    if (steps <= 0 && node != kDone) {
+      stopped = node;
+      node = kDone;
+    }
+    const unsigned inner = __ballot_sync(0xffffffffu, node >= 0);
+    const unsigned leaf = __ballot_sync(0xffffffffu, node < 0 && node != kDone);
+    if (!inner && !leaf) break;
+    if (inner && __popc(leaf) * 8 < kLeafWait * __popc(inner | leaf)) continue;
+    if (node < 0 && node != kDone) {
+      --steps;
+      leaf_test<KMAX, kBlock, COUNT>(fa, rm, (uint32_t)(~node), tcut, errmax, cn);
+      node = sp ? stack[--sp] : kDone;
+    }
   }
-  return ok;
+  w.node = stopped;
+  w.sp = sp;
+  w.tcut = tcut;
+  w.errmax = errmax;
+  return steps;
 }
 
-// Slab reciprocals of a ray: a zero direction component would turn the slab
-// products into inf - inf, so its sign is kept and its magnitude floored.
-__device__ __forceinline__ void ray_slabs(const float3 o, const float3 d, float3& inv,
-                                          float3& ooi) {
-  inv = f3(1.0f / (fabsf(d.x) > 1e-12f ? d.x : copysignf(1e-12f, d.x)),
-           1.0f / (fabsf(d.y) > 1e-12f ? d.y : copysignf(1e-12f, d.y)),
-           1.0f / (fabsf(d.z) > 1e-12f ? d.z : copysignf(1e-12f, d.z)));
-  ooi = f3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+// The K nearest hits of the warp's rays, one per live lane, without a stop.
+template <int KMAX, bool COUNT>
+__device__ __forceinline__ bool traverse(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm, const bool live,
+                                         Counts& cn) {
+  int stack[kStack];
+  kbuf_clear(rm, threadIdx.x);
+  Walk w = walk_begin(fa, live);
+  walk_on<KMAX, COUNT>(fa, rm, w, stack, 0x7fffffff, cn);
+  return w.ok;
 }
 
 // ------------------------------------------------------------------ scattering
@@ -706,10 +796,10 @@ __device__ __forceinline__ void forward_albedo(const Tables& tb, const Mat& m, f
 // The ray's interval inside one record's finite cylinder, clipped to
 // (tmin, tmax): the hair a shadow ray crosses, or the chord of a primary hit.
 // Returns false when empty.
-__device__ __forceinline__ bool leaf_span(const float4* __restrict__ xf, const float3 o,
+__device__ __forceinline__ bool leaf_span(const FrameArgs& fa, const uint32_t id, const float3 o,
                                           const float3 d, const float tmin, const float tmax,
                                           float& lo, float& hi) {
-  const float4 r0 = __ldg(xf), r1 = __ldg(xf + 1), r2 = __ldg(xf + 2);
+  const float4 r0 = __ldg(fa.prim_uv + 2 * (size_t)id), r1 = __ldg(fa.prim_uv + 2 * (size_t)id + 1);
   const float u0 = fmaf(r0.x, o.x, fmaf(r0.y, o.y, fmaf(r0.z, o.z, r0.w)));
   const float v0 = fmaf(r1.x, o.x, fmaf(r1.y, o.y, fmaf(r1.z, o.z, r1.w)));
   const float du = fmaf(r0.x, d.x, fmaf(r0.y, d.y, r0.z * d.z));
@@ -724,6 +814,7 @@ __device__ __forceinline__ bool leaf_span(const float4* __restrict__ xf, const f
   const float half = sqrtf((1.f - h2) * inv);
   lo = tc - half;
   hi = tc + half;
+  const float4 r2 = __ldg(fa.prim_wa + 2 * (size_t)id);
   const float w0 = fmaf(r2.x, o.x, fmaf(r2.y, o.y, fmaf(r2.z, o.z, r2.w)));
   const float dw = fmaf(r2.x, d.x, fmaf(r2.y, d.y, r2.z * d.z));
   if (dw != 0.f) {
@@ -756,29 +847,18 @@ __device__ __forceinline__ void shadow_path(const FrameArgs& fa, const float3 x,
   T[0] = T[1] = T[2] = 1.f;
   sg2 = 0.f;
   if (fa.n_prims == 0) return;
-  float3 inv, ooi;
-  ray_slabs(x, wi, inv, ooi);
+  const Slabs sl = ray_slabs(fa, x, wi);
   int stack[kStack];
   int sp = 0;
   int node = fa.n_prims == 1 ? ~(int)__ldg(fa.leaf_id) : 0;
   bool crossed = false;
   for (;;) {
     if (node >= 0) {
-      const float4* nd = fa.nodes + 4 * (size_t)node;
-      const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
+      const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
       if (COUNT) ++cn.nodes;
-      float lx = fmaf(n0.x, inv.x, -ooi.x), hx = fmaf(n0.y, inv.x, -ooi.x);
-      float ly = fmaf(n0.z, inv.y, -ooi.y), hy = fmaf(n0.w, inv.y, -ooi.y);
-      float lz = fmaf(n2.x, inv.z, -ooi.z), hz = fmaf(n2.y, inv.z, -ooi.z);
-      const float a0 = fmaxf(fmaxf(fminf(lx, hx), fminf(ly, hy)), fmaxf(fminf(lz, hz), 0.f));
-      const float b0 = fminf(fminf(fmaxf(lx, hx), fmaxf(ly, hy)), fminf(fmaxf(lz, hz), tmax));
-      lx = fmaf(n1.x, inv.x, -ooi.x); hx = fmaf(n1.y, inv.x, -ooi.x);
-      ly = fmaf(n1.z, inv.y, -ooi.y); hy = fmaf(n1.w, inv.y, -ooi.y);
-      lz = fmaf(n2.z, inv.z, -ooi.z); hz = fmaf(n2.w, inv.z, -ooi.z);
-      const float a1 = fmaxf(fmaxf(fminf(lx, hx), fminf(ly, hy)), fmaxf(fminf(lz, hz), 0.f));
-      const float b1 = fminf(fminf(fmaxf(lx, hx), fmaxf(ly, hy)), fminf(fmaxf(lz, hz), tmax));
-      const bool h0 = a0 <= b0, h1 = a1 <= b1;
-      const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
+      float a0, a1;
+      const bool h0 = slab_test(sl, k0, tmax, a0), h1 = slab_test(sl, k1, tmax, a1);
+      const int c0 = (int)k0.w, c1 = (int)k1.w;
       if (h0 && h1) {
         if (sp < kStack)
           stack[sp++] = c1;
@@ -793,12 +873,12 @@ __device__ __forceinline__ void shadow_path(const FrameArgs& fa, const float3 x,
       }
     } else {
       const uint32_t id = (uint32_t)(~node);
-      const float4 aux = __ldg(fa.prim_aux + id);
       float lo, hi;
       if (COUNT) ++cn.tests;
-      if (__float_as_uint(aux.x) != self_mat &&
-          leaf_span(fa.prim_xf + 3 * (size_t)id, x, wi, 0.f, tmax, lo, hi)) {
-        const float4 r2 = __ldg(fa.prim_xf + 3 * (size_t)id + 2);
+      float4 aux;
+      if (leaf_span(fa, id, x, wi, 0.f, tmax, lo, hi) &&
+          __float_as_uint((aux = __ldg(fa.prim_wa + 2 * (size_t)id + 1)).x) != self_mat) {
+        const float4 r2 = __ldg(fa.prim_wa + 2 * (size_t)id);
         const float si = clampf(dot3(wi, f3(r2.x, r2.y, r2.z)) *
                                     rsqrtf(r2.x * r2.x + r2.y * r2.y + r2.z * r2.z),
                                 -1.f, 1.f);
@@ -862,8 +942,7 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
                                           float& alpha, Counts& cn,
                                           const float4* __restrict__ paths = nullptr,
                                           size_t path_stride = 0) {
-  const float4 aux = __ldg(fa.prim_aux + id);
-  const float4 r2 = __ldg(fa.prim_xf + 3 * (size_t)id + 2);
+  const float4 r2 = __ldg(fa.prim_wa + 2 * (size_t)id), aux = __ldg(fa.prim_wa + 2 * (size_t)id + 1);
   const float3 T = f3(r2.x, r2.y, r2.z) * rsqrtf(r2.x * r2.x + r2.y * r2.y + r2.z * r2.z);
   Mat m;
   load_mat(fa.mat + (size_t)__float_as_uint(aux.x) * HR_MAT_FLOATS, m);
@@ -881,7 +960,7 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
     // rounding puts a hit at the very outline outside it)
     float lo, hi;
     const float chord =
-        leaf_span(fa.prim_xf + 3 * (size_t)id, o, d, -kInf, kInf, lo, hi) ? hi - lo : 0.f;
+        leaf_span(fa, id, o, d, -kInf, kInf, lo, hi) ? hi - lo : 0.f;
     const float ntot = aux.y, r = aux.z, ab = aux.w;
     eh.rho = fminf(1.f, ntot * r * r / ab);
     const float n_raw = eh.rho * chord * sqrtf(ntot / (kPi * ab));
@@ -932,47 +1011,138 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
   }
 }
 
-// One sample: ray, K nearest hits, shading and front-to-back compositing.
-template <int KMAX, int PREC, bool COUNT, bool SHADOW = false>
-__device__ __forceinline__ void render_ray(const FrameArgs& fa, const RayKey& rk, const float3 o,
-                                           const float3 d, float out[3], int32_t* ids, bool& ok,
-                                           Counts& cn) {
-  KBuf<KMAX> kb;
-  ok = traverse<KMAX, COUNT>(fa, rk, o, d, kb, cn);
-  float T = 1.f;
+// Shading and front-to-back compositing of a sample's hits (entry j's depth at
+// t[j * stride], its word at id[j * stride], nearest first).
+template <int PREC, bool COUNT, bool SHADOW>
+__device__ __forceinline__ void shade_hits(const FrameArgs& fa, const float* t, const uint32_t* id,
+                                           uint32_t stride, uint32_t k, const float3 o, const float3 d,
+                                           float out[3], Counts& cn) {
   out[0] = out[1] = out[2] = 0.f;
-  if (ids) {  // the composited hits: none after the first opaque (strand) one
-    bool past = false;
-#pragma unroll
-    for (int j = 0; j < KMAX; ++j)
-      if (j < (int)fa.k) {
-        const bool live = kb.t[j] < kInf && !past;
-        ids[j] = live ? (int32_t)(kb.id[j] & kIdMask) : -1;
-        if (live && (kb.id[j] & kOpaque)) past = true;
-      }
-  }
-#pragma unroll
-  for (int j = 0; j < KMAX; ++j) {
-    if (j < (int)fa.k && kb.t[j] < kInf && T > 0.f) {
-      float rgb[3], a;
-      shade_hit<PREC, COUNT, SHADOW>(fa, kb.id[j] & kIdMask, kb.t[j], o, d, rgb, a, cn);
-      if (COUNT) ++cn.hits;
-      const float ta = T * a;
-      out[0] = fmaf(ta, rgb[0], out[0]);
-      out[1] = fmaf(ta, rgb[1], out[1]);
-      out[2] = fmaf(ta, rgb[2], out[2]);
-      T *= 1.f - a;
-    }
+  float T = 1.f;
+#pragma unroll 1
+  for (uint32_t j = 0; j < k; ++j) {
+    const float tj = t[j * stride];
+    if (!(tj < kInf && T > 0.f)) break;  // sorted by depth
+    float rgb[3], a;
+    shade_hit<PREC, COUNT, SHADOW>(fa, id[j * stride] & kIdMask, tj, o, d, rgb, a, cn);
+    if (COUNT) ++cn.hits;
+    const float ta = T * a;
+    out[0] = fmaf(ta, rgb[0], out[0]);
+    out[1] = fmaf(ta, rgb[1], out[1]);
+    out[2] = fmaf(ta, rgb[2], out[2]);
+    T *= 1.f - a;
   }
 }
 
-template <int KMAX, int PREC, bool COUNT, bool SHADOW = false>
-__device__ __forceinline__ void render_sample(const FrameArgs& fa, uint64_t sid, float out[3],
-                                              int32_t* ids, bool& ok, Counts& cn) {
+template <int KMAX>
+__device__ __forceinline__ void primary_store(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm, uint64_t sid) {
   RayKey rk;
   float3 o, d;
   primary_ray(fa, sid, o, d, rk);
-  render_ray<KMAX, PREC, COUNT, SHADOW>(fa, rk, o, d, out, ids, ok, cn);
+  ray_store(rm, threadIdx.x, o, d, rk);
+}
+
+// One sample per live lane: ray, K nearest hits, shading and compositing.
+// Whole warps call it.
+template <int KMAX, int PREC, bool COUNT, bool SHADOW = false>
+__device__ __forceinline__ void render_sample(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm, uint64_t sid,
+                                              const bool live, float out[3],
+                                              bool& ok, Counts& cn) {
+  const uint32_t c = threadIdx.x;
+  primary_store(fa, rm, sid);
+  ok = traverse<KMAX, COUNT>(fa, rm, live, cn);
+  out[0] = out[1] = out[2] = 0.f;
+  if (live)
+    shade_hits<PREC, COUNT, SHADOW>(fa, &rm.t[0][c], &rm.id[0][c], kBlock, KMAX == 1 ? 1u : fa.k,
+                                    ray_o(rm, c), ray_d(rm, c), out, cn);
+}
+
+// ---------------------------------------------------------------- long walks
+//
+// A few rays walk ten or a hundred times as far as the others (they skim the
+// layer in which the strands bend or lie along the view: 4,000 visits and
+// 6,500 tests in the 4K frame of straight hair, 55 of both on average), and
+// the frame lasts as long as the warp that traces them.  A ray that has used
+// up its budget of steps is therefore put aside with its pending nodes and its
+// hits, and a second kernel finishes these rays with a whole warp each.
+
+// A tile with rays put aside: what the last of them needs to composite it.
+struct LongTile {
+  uint32_t xy;         // origin, x | y << 16
+  uint32_t lanes;      // lanes whose rays were put aside
+  uint32_t left;       // of those, not finished yet
+  uint32_t pad;
+  float acc[3][32];    // the lanes' radiance
+  uint32_t at[32];     // where a put-aside lane's record starts
+};
+// A ray's record, in words: tile, lane | pending nodes << 8, cut, widest
+// bound, k depths, k low words of depths, k entry words, the pending nodes
+// (last the first to visit).
+constexpr uint32_t kLongHead = 4;
+
+// Puts the rays of the lanes in `mask` aside (the lane's walk w stopped short
+// in them).  False when there is no room: nothing is put aside.
+template <int KMAX>
+__device__ __forceinline__ bool put_aside(const FrameArgs& fa, const RayMem<KMAX, kBlock>& rm,
+                                          const Walk& w, const int* stack, uint32_t x0, uint32_t y0,
+                                          unsigned mask, uint32_t& tile) {
+  const uint32_t lane = threadIdx.x & 31, c = threadIdx.x, k = fa.k;
+  const bool mine = (mask >> lane) & 1u;
+  const uint32_t words = mine ? kLongHead + 3 * k + (uint32_t)w.sp + 1 : 0u;
+  uint32_t incl = words;
+#pragma unroll
+  for (int q = 1; q < 32; q <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, q);
+    if (lane >= (uint32_t)q) incl += v;
+  }
+  const uint32_t total = __shfl_sync(0xffffffffu, incl, 31), rays = (uint32_t)__popc(mask);
+  uint32_t at = 0xffffffffu, first = 0;
+  tile = 0;
+  if (lane == 0) {
+    // room as far as one can see (the counters stay far from wrapping), then for certain
+    if (__ldcg(fa.lw.ctr + 1) + total <= fa.lw.words && __ldcg(fa.lw.ctr + 2) < fa.lw.tiles_max &&
+        __ldcg(fa.lw.ctr) + rays <= fa.lw.rays_max) {
+      at = atomicAdd(fa.lw.ctr + 1, total);
+      tile = atomicAdd(fa.lw.ctr + 2, 1u);
+      if (at + total > fa.lw.words || tile >= fa.lw.tiles_max) {
+        at = 0xffffffffu;
+      } else {
+        first = atomicAdd(fa.lw.ctr, rays);
+        if (first + rays > fa.lw.rays_max) {  // the places taken below the limit stay empty
+          for (uint32_t i = first; i < fa.lw.rays_max; ++i) fa.lw.ray_at[i] = 0xffffffffu;
+          at = 0xffffffffu;
+        }
+      }
+    }
+  }
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (at == 0xffffffffu) return false;
+  tile = __shfl_sync(0xffffffffu, tile, 0);
+  first = __shfl_sync(0xffffffffu, first, 0);
+  at += incl - words;
+  if (lane == 0) {
+    fa.lw.tiles[tile].xy = x0 | y0 << 16;
+    fa.lw.tiles[tile].lanes = mask;
+    fa.lw.tiles[tile].left = rays;
+  }
+  if (mine) {
+    fa.lw.tiles[tile].at[lane] = at;
+    fa.lw.ray_at[first + __popc(mask & ((1u << lane) - 1u))] = at;
+    uint32_t* r = fa.lw.pool + at;
+    r[0] = tile;
+    r[1] = lane | (uint32_t)(w.sp + 1) << 8;
+    r[2] = __float_as_uint(w.tcut);
+    r[3] = __float_as_uint(w.errmax);
+    for (uint32_t j = 0; j < k; ++j) {
+      r[kLongHead + j] = __float_as_uint(rm.t[j][c]);
+      r[kLongHead + k + j] = __float_as_uint(rm.tr[j][c]);
+      r[kLongHead + 2 * k + j] = rm.id[j][c];
+    }
+    r += kLongHead + 3 * k;
+    for (int j = 0; j < w.sp; ++j) r[j] = (uint32_t)stack[j];
+    r[w.sp] = (uint32_t)w.node;
+  }
+  return true;
 }
 
 __device__ __forceinline__ void flush_counts(const FrameArgs& fa, const Counts& cn) {
@@ -998,10 +1168,10 @@ __device__ __forceinline__ void scene_rect_warp(const FrameArgs& fa, float4* rec
     float X0 = kInf, Y0 = kInf, X1 = -kInf, Y1 = -kInf;
     bool ok = fa.n_prims >= 2;
     if (ok && lane < 8) {
-      const float4 n0 = __ldg(fa.nodes), n1 = __ldg(fa.nodes + 1), n2 = __ldg(fa.nodes + 2);
-      const float3 p = f3((lane & 1) ? fmaxf(n0.y, n1.y) : fminf(n0.x, n1.x),
-                          (lane & 2) ? fmaxf(n0.w, n1.w) : fminf(n0.z, n1.z),
-                          (lane & 4) ? fmaxf(n2.y, n2.w) : fminf(n2.x, n2.z));
+      float3 blo, bhi;
+      root_box(fa, blo, bhi);
+      const float3 p = f3((lane & 1) ? bhi.x : blo.x, (lane & 2) ? bhi.y : blo.y,
+                          (lane & 4) ? bhi.z : blo.z);
       const float3 r = p - fa.cam.eye;
       const float xc = dot3(r, fa.cam.right), yc = dot3(r, fa.cam.up), zc = dot3(r, fa.cam.fwd);
       float X, Y;
@@ -1034,73 +1204,88 @@ __device__ __forceinline__ void scene_rect_warp(const FrameArgs& fa, float4* rec
 }
 
 // Warp tile: the 32 / grp pixels one warp renders (wtw x wth); a pixel's
-// samples on `grp` adjacent lanes.  tile_partials traces a lane's samples and
-// returns their sum in sample order, for the lanes in `lanes` (the others
-// return zeros).  tile_write sums a pixel's lanes with a fixed
-// XOR-shuffle tree and stores the mean.  Both are called by whole warps.
-template <int KMAX, int PREC, bool COUNT, bool SHADOW = false>
-__device__ __forceinline__ void tile_partials(const FrameArgs& fa, uint32_t x0, uint32_t y0,
-                                              uint32_t wtw, const float4 rect, uint32_t lanes,
-                                              float acc[3], Counts& cn, bool& overflow) {
-  const uint32_t G = fa.grp;
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t lane_g = lane & (G - 1);
-  const uint32_t p = lane / G;
+// samples on `grp` adjacent lanes.
+struct TileLane {
+  bool inside;     // the lane's pixel is in the image and in the scene's rectangle
+  uint64_t pixel;
+};
+__device__ __forceinline__ TileLane tile_lane(const FrameArgs& fa, uint32_t x0, uint32_t y0, uint32_t wtw,
+                                              const float4 rect) {
+  const uint32_t p = (threadIdx.x & 31) / fa.grp;
   const uint32_t x = x0 + p % wtw, y = y0 + p / wtw;
-  const bool valid = x < (uint32_t)fa.cam.W && y < (uint32_t)fa.cam.H;
-  const bool inside = valid && (float)x + 1.f >= rect.x && (float)x <= rect.z &&
-                      (float)y + 1.f >= rect.y && (float)y <= rect.w && ((lanes >> lane) & 1u);
-  const uint64_t pixel = (uint64_t)y * (uint32_t)fa.cam.W + x;
-  acc[0] = acc[1] = acc[2] = 0.f;
-  if (inside) {
-    for (uint32_t s = lane_g; s < fa.spp; s += G) {
-      float v[3];
-      bool ok;
-      RayKey rk;
-      float3 o, d;
-      primary_ray(fa, pixel * fa.spp + s, o, d, rk);
-      render_ray<KMAX, PREC, COUNT, SHADOW>(fa, rk, o, d, v, nullptr, ok, cn);
-      if (COUNT) ++cn.rays;
-      overflow |= !ok;
-      acc[0] += v[0];
-      acc[1] += v[1];
-      acc[2] += v[2];
-    }
-  }
+  TileLane t;
+  t.inside = x < (uint32_t)fa.cam.W && y < (uint32_t)fa.cam.H && (float)x + 1.f >= rect.x &&
+             (float)x <= rect.z && (float)y + 1.f >= rect.y && (float)y <= rect.w;
+  t.pixel = (uint64_t)y * (uint32_t)fa.cam.W + x;
+  return t;
 }
 
-__device__ __forceinline__ void tile_write(const FrameArgs& fa, uint32_t x0, uint32_t y0,
-                                           uint32_t wtw, const float4 rect, float acc[3],
+// Sums a pixel's lanes with a fixed XOR-shuffle tree and stores the mean.
+// Whole warps call it.
+__device__ __forceinline__ void tile_write(const FrameArgs& fa, const TileLane tl, float acc[3],
                                            float* __restrict__ rgb) {
   const uint32_t G = fa.grp;
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t p = lane / G;
-  const uint32_t x = x0 + p % wtw, y = y0 + p / wtw;
-  const bool valid = x < (uint32_t)fa.cam.W && y < (uint32_t)fa.cam.H;
-  const bool inside = valid && (float)x + 1.f >= rect.x && (float)x <= rect.z &&
-                      (float)y + 1.f >= rect.y && (float)y <= rect.w;
-  const uint64_t pixel = (uint64_t)y * (uint32_t)fa.cam.W + x;
   for (uint32_t o = 1; o < G; o <<= 1) {
     acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
     acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], o);
     acc[2] += __shfl_xor_sync(0xffffffffu, acc[2], o);
   }
-  if (inside && (lane & (G - 1)) == 0) {
+  if (tl.inside && (threadIdx.x & (G - 1)) == 0) {
     const float inv = 1.0f / (float)fa.spp;
-    rgb[3 * pixel] = acc[0] * inv;
-    rgb[3 * pixel + 1] = acc[1] * inv;
-    rgb[3 * pixel + 2] = acc[2] * inv;
+    rgb[3 * tl.pixel] = acc[0] * inv;
+    rgb[3 * tl.pixel + 1] = acc[1] * inv;
+    rgb[3 * tl.pixel + 2] = acc[2] * inv;
   }
 }
 
-template <int KMAX, int PREC, bool COUNT, bool SHADOW = false>
-__device__ __forceinline__ void render_warp_tile(const FrameArgs& fa, uint32_t x0, uint32_t y0,
-                                                 uint32_t wtw, const float4 rect,
-                                                 float* __restrict__ rgb, Counts& cn,
-                                                 bool& overflow) {
-  float acc[3];
-  tile_partials<KMAX, PREC, COUNT, SHADOW>(fa, x0, y0, wtw, rect, 0xffffffffu, acc, cn, overflow);
-  tile_write(fa, x0, y0, wtw, rect, acc, rgb);
+// Traces, shades and stores a tile.  With LONG, rays over the budget of steps
+// are put aside (at most one sample a lane: no more than 32 spp) and
+// the tile is stored by the last of them.
+template <int KMAX, int PREC, bool COUNT, bool SHADOW = false, bool LONG = false>
+__device__ __forceinline__ void render_warp_tile(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm,
+                                                 uint32_t x0, uint32_t y0, uint32_t wtw,
+                                                 const float4 rect, int budget,
+                                                 float* __restrict__ rgb, Counts& cn, bool& overflow) {
+  const uint32_t G = fa.grp, c = threadIdx.x, lane = c & 31;
+  const TileLane tl = tile_lane(fa, x0, y0, wtw, rect);
+  if (!__any_sync(0xffffffffu, tl.inside)) return;
+  float acc[3] = {0.f, 0.f, 0.f};
+  for (uint32_t s0 = 0; s0 < fa.spp; s0 += G) {
+    const uint32_t s = s0 + (lane & (G - 1));
+    const bool live = tl.inside && s < fa.spp;
+    primary_store(fa, rm, tl.pixel * fa.spp + s);
+    kbuf_clear(rm, c);
+    int stack[kStack];
+    Walk w = walk_begin(fa, live);
+    unsigned aside = 0;
+    uint32_t tile = 0;
+    for (int steps = LONG ? budget : 0x7fffffff;; steps = 0x7fffffff) {
+      const int left = walk_on<KMAX, COUNT>(fa, rm, w, stack, steps, cn);
+      if (LONG) {
+        cn.steps += (uint32_t)(steps - left);
+        aside = __ballot_sync(0xffffffffu, w.node != kDone);
+        if (aside && !put_aside<KMAX>(fa, rm, w, stack, x0, y0, aside, tile)) continue;
+      }
+      break;
+    }
+    float v[3] = {0.f, 0.f, 0.f};
+    if (live && !((aside >> lane) & 1u))
+      shade_hits<PREC, COUNT, SHADOW>(fa, &rm.t[0][c], &rm.id[0][c], kBlock, KMAX == 1 ? 1u : fa.k,
+                                      ray_o(rm, c), ray_d(rm, c), v, cn);
+    if (COUNT && live) ++cn.rays;
+    overflow |= !w.ok;
+    acc[0] += v[0];
+    acc[1] += v[1];
+    acc[2] += v[2];
+    if (LONG && aside) {
+      LongTile& lt = fa.lw.tiles[tile];
+      lt.acc[0][lane] = acc[0];
+      lt.acc[1][lane] = acc[1];
+      lt.acc[2][lane] = acc[2];
+      return;
+    }
+  }
+  tile_write(fa, tl, acc, rgb);
 }
 
 }  // namespace tr

@@ -7,34 +7,39 @@ namespace hr {
 namespace {
 
 template <int KMAX, int PREC, bool SHADOW>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kBlock)
     k_samples(const FrameArgs fa, const uint32_t* __restrict__ sids, uint32_t m,
               float* __restrict__ rad, int32_t* __restrict__ hit) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
+  const bool live = i < m;  // whole warps trace
   tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
+  __shared__ tr::RayMem<KMAX, kBlock> rm;
   float v[3];
-  int32_t ids[KMAX];
   bool ok;
-  tr::render_sample<KMAX, PREC, false, SHADOW>(fa, sids[i], v, ids, ok, cn);
+  tr::render_sample<KMAX, PREC, false, SHADOW>(fa, rm, sids[live ? i : 0], live, v, ok, cn);
+  if (!live) return;
   rad[3 * (size_t)i] = v[0];
   rad[3 * (size_t)i + 1] = v[1];
   rad[3 * (size_t)i + 2] = v[2];
-#pragma unroll
-  for (int j = 0; j < KMAX; ++j)
-    if (j < (int)fa.k) hit[(size_t)fa.k * i + j] = ids[j];
+  bool past = false;  // the composited hits: none after the first opaque (strand) one
+  for (uint32_t j = 0; j < fa.k; ++j) {
+    const uint32_t w = rm.id[j][threadIdx.x];
+    const bool hit_j = rm.t[j][threadIdx.x] < kInf && !past;
+    hit[(size_t)fa.k * i + j] = hit_j ? (int32_t)(w & tr::kIdMask) : -1;
+    if (hit_j && (w & tr::kOpaque)) past = true;
+  }
   if (!ok) atomicAdd(fa.overflow, 1u);
 }
 
 template <int PREC, bool SHADOW>
 hr_status launch_p(hr_ctx* ctx, const FrameArgs& fa, const uint32_t* sids, uint32_t m,
                    float* rad, int32_t* hit, cudaStream_t st) {
-  const uint32_t g = (m + 127) / 128;
+  const uint32_t g = (m + kBlock - 1) / kBlock;
   switch (kmax_for(fa.k)) {
-    case 1: k_samples<1, PREC, SHADOW><<<g, 128, 0, st>>>(fa, sids, m, rad, hit); break;
-    case 2: k_samples<2, PREC, SHADOW><<<g, 128, 0, st>>>(fa, sids, m, rad, hit); break;
-    case 4: k_samples<4, PREC, SHADOW><<<g, 128, 0, st>>>(fa, sids, m, rad, hit); break;
-    default: k_samples<8, PREC, SHADOW><<<g, 128, 0, st>>>(fa, sids, m, rad, hit); break;
+    case 1: k_samples<1, PREC, SHADOW><<<g, kBlock, 0, st>>>(fa, sids, m, rad, hit); break;
+    case 2: k_samples<2, PREC, SHADOW><<<g, kBlock, 0, st>>>(fa, sids, m, rad, hit); break;
+    case 4: k_samples<4, PREC, SHADOW><<<g, kBlock, 0, st>>>(fa, sids, m, rad, hit); break;
+    default: k_samples<8, PREC, SHADOW><<<g, kBlock, 0, st>>>(fa, sids, m, rad, hit); break;
   }
   HR_LAUNCHED(ctx);
   return HR_OK;

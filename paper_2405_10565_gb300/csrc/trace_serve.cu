@@ -17,9 +17,10 @@ __global__ void k_serve_rect(const FrameArgs fa, float4* rect) { tr::scene_rect_
 
 template <int KMAX, int PREC>
 // 4 blocks per SM (at most 128 registers), as for the frame kernel.
-__global__ void __launch_bounds__(kBlock, 4)
+__global__ void __launch_bounds__(kBlock, tr::kTraceBlocks)
     k_serve(const ServeItem* __restrict__ items, const uint32_t* __restrict__ item_start,
             uint32_t n_items, uint32_t total, uint32_t* work) {
+  __shared__ tr::RayMem<KMAX, kBlock> rm;
   const uint32_t lane = threadIdx.x & 31;
   for (;;) {
     uint32_t bt = 0;
@@ -36,8 +37,8 @@ __global__ void __launch_bounds__(kBlock, 4)
     const uint32_t t = it.wt0 + (bt - item_start[lo]);
     tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
     bool overflow = false;
-    tr::render_warp_tile<KMAX, PREC, false>(it.fa, g.x0 + (t % g.nx) * g.wtw,
-                                            g.y0 + (t / g.nx) * g.wth, g.wtw, it.rect, it.rgb, cn,
+    tr::render_warp_tile<KMAX, PREC, false>(it.fa, rm, g.x0 + (t % g.nx) * g.wtw,
+                                            g.y0 + (t / g.nx) * g.wth, g.wtw, it.rect, 0, it.rgb, cn,
                                             overflow);
     if (overflow) atomicAdd(it.fa.overflow, 1u);
   }

@@ -46,9 +46,10 @@ struct ShadowWork {
 // to the first opaque one) is listed, a tile's hits together and in lane
 // order.
 template <int KMAX>
-__global__ void __launch_bounds__(kBlock, 4)
+__global__ void __launch_bounds__(kBlock, tr::kTraceBlocks)
     k_shadow_hits(const FrameArgs fa, const float4* __restrict__ rect_p, uint32_t* work,
                   const ShadowWork sw) {
+  __shared__ tr::RayMem<KMAX, kBlock> rm;
   const float4 rect = *rect_p;
   const WarpGrid g = warp_grid(rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
   const uint32_t lane = threadIdx.x & 31, G = fa.grp;
@@ -58,30 +59,17 @@ __global__ void __launch_bounds__(kBlock, 4)
     if (lane == 0 && __ldcg(sw.ctr) < sw.stop) t = atomicAdd(work, 1u);
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= g.n) break;
-    const uint32_t p = lane / G;
-    const uint32_t x = g.x0 + (t % g.nx) * g.wtw + p % g.wtw;
-    const uint32_t y = g.y0 + (t / g.nx) * g.wth + p / g.wtw;
-    const bool inside = x < (uint32_t)fa.cam.W && y < (uint32_t)fa.cam.H &&
-                        (float)x + 1.f >= rect.x && (float)x <= rect.z &&
-                        (float)y + 1.f >= rect.y && (float)y <= rect.w;
-    const uint64_t pixel = (uint64_t)y * (uint32_t)fa.cam.W + x;
+    const uint32_t x0 = g.x0 + (t % g.nx) * g.wtw, y0 = g.y0 + (t / g.nx) * g.wth;
+    const tr::TileLane tl = tr::tile_lane(fa, x0, y0, g.wtw, rect);
     const uint32_t s = lane & (G - 1);
-    tr::KBuf<KMAX> kb;
-    float3 o, d;
+    const bool live = tl.inside && s < fa.spp;
+    tr::primary_store(fa, rm, tl.pixel * fa.spp + s);
+    tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
+    overflow |= !tr::traverse<KMAX, false>(fa, rm, live, cn);
     uint32_t cnt = 0;
-    if (inside && s < fa.spp) {
-      tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
-      tr::RayKey rk;
-      tr::primary_ray(fa, pixel * fa.spp + s, o, d, rk);
-      overflow |= !tr::traverse<KMAX, false>(fa, rk, o, d, kb, cn);
-      bool past = false;
-#pragma unroll
-      for (int j = 0; j < KMAX; ++j)
-        if (j < (int)fa.k && kb.t[j] < kInf && !past) {
-          ++cnt;
-          past = (kb.id[j] & tr::kOpaque) != 0u;
-        }
-    }
+    if (live)
+      for (bool past = false; cnt < fa.k && rm.t[cnt][threadIdx.x] < kInf && !past; ++cnt)
+        past = (rm.id[cnt][threadIdx.x] & tr::kOpaque) != 0u;
     uint32_t incl = cnt;
 #pragma unroll
     for (int q = 1; q < 32; q <<= 1) {
@@ -103,13 +91,12 @@ __global__ void __launch_bounds__(kBlock, 4)
     }
     reinterpret_cast<uint8_t*>(sw.tiles[rec].cnt)[lane] = (uint8_t)cnt;
     const uint32_t h0 = base + incl - cnt;
-#pragma unroll
-    for (int j = 0; j < KMAX; ++j)
-      if (j < (int)cnt) {
-        const float3 x3 = tr::hit_point(o, d, kb.t[j]);
-        sw.hit[h0 + j] = make_float4(x3.x, x3.y, x3.z, __uint_as_float(kb.id[j]));
-        sw.depth[h0 + j] = kb.t[j];
-      }
+    for (uint32_t j = 0; j < cnt; ++j) {
+      const float t = rm.t[j][threadIdx.x];
+      const float3 x3 = tr::hit_point(tr::ray_o(rm, threadIdx.x), tr::ray_d(rm, threadIdx.x), t);
+      sw.hit[h0 + j] = make_float4(x3.x, x3.y, x3.z, __uint_as_float(rm.id[j][threadIdx.x]));
+      sw.depth[h0 + j] = t;
+    }
   }
   if (overflow) atomicAdd(fa.overflow, 1u);
 }
@@ -135,7 +122,7 @@ __global__ void __launch_bounds__(kBlock) k_shadow_paths(const FrameArgs fa, con
     bool ok = true;
     tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
     tr::shadow_path<PREC, false>(fa, x, wi, tr::path_length(light, E),
-                                 __float_as_uint(__ldg(&fa.prim_aux[id].x)), T, sg2, ok, cn);
+                                 __float_as_uint(__ldg(&fa.prim_wa[2 * (size_t)id + 1].x)), T, sg2, ok, cn);
     if (!ok) atomicAdd(fa.overflow, 1u);
     sw.path[(size_t)l * sw.cap + h] = make_float4(T[0], T[1], T[2], sg2);
   }
@@ -161,14 +148,14 @@ __global__ void __launch_bounds__(kBlock)
       if (lane >= (uint32_t)q) incl += v;
     }
     const uint32_t h0 = st.base + incl - cnt;
-    const uint32_t x0 = g.x0 + (t % g.nx) * g.wtw, y0 = g.y0 + (t / g.nx) * g.wth, p = lane / G;
+    const uint32_t x0 = g.x0 + (t % g.nx) * g.wtw, y0 = g.y0 + (t / g.nx) * g.wth;
+    const tr::TileLane tl = tr::tile_lane(fa, x0, y0, g.wtw, rect);
     float acc[3] = {0.f, 0.f, 0.f};
     if (cnt) {
-      const uint64_t pixel = (uint64_t)(y0 + p / g.wtw) * (uint32_t)fa.cam.W + x0 + p % g.wtw;
       tr::Counts cn{0, 0, 0, 0, 0, 0, 0, 0};
       tr::RayKey rk;
       float3 o, d;
-      tr::primary_ray(fa, pixel * fa.spp + (lane & (G - 1)), o, d, rk);
+      tr::primary_ray(fa, tl.pixel * fa.spp + (lane & (G - 1)), o, d, rk);
       float T = 1.f;
       for (uint32_t j = 0; j < cnt && T > 0.f; ++j) {
         float c[3], a;
@@ -182,7 +169,7 @@ __global__ void __launch_bounds__(kBlock)
         T *= 1.f - a;
       }
     }
-    tr::tile_write(fa, x0, y0, g.wtw, rect, acc, rgb);
+    tr::tile_write(fa, tl, acc, rgb);
   }
 }
 
@@ -253,7 +240,7 @@ hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, 
   const uint64_t cap = std::min<uint64_t>(worst, stop + (uint64_t)g_hits * kBlock * fa.k);
   const size_t bytes = 64 + cap * (sizeof(float4) + sizeof(ShadowTile) + sizeof(float) + L * sizeof(float4));
   char* p = nullptr;
-  if (scratch(ctx, 17, bytes, (void**)&p) != HR_OK) {
+  if (scratch(ctx, kScratchPaths, bytes, (void**)&p) != HR_OK) {
     set_error(ctx, HR_OK, "");
     return HR_OK;
   }
