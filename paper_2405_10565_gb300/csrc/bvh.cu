@@ -96,8 +96,8 @@ constexpr size_t kFrameWords = 5;
 // The grid of the node boxes, from the bounds of the strands' and the thick
 // hairs' boxes: low corner (two steps below the bounds), step, 1 / step; and
 // the leaves' bounds and the climb's counts cleared for k_gather_refit.
-__device__ __forceinline__ void begin_refit(const uint32_t* __restrict__ bounds, float4* frame,
-                                            unsigned* counts) {
+__device__ __forceinline__ void begin_refit(const uint32_t* __restrict__ bounds, float4* grid,
+                                            uint32_t* leaf_bounds, unsigned* counts) {
   float lo[3], hi[3], st[3];
   for (int i = 0; i < 3; ++i) {
     lo[i] = from_ordered(bounds[i]);
@@ -110,16 +110,15 @@ __device__ __forceinline__ void begin_refit(const uint32_t* __restrict__ bounds,
     st[i] = fmaxf((hi[i] - lo[i]) * (1.0f / 65520.0f), 1e-30f);
     lo[i] = fmaf(-2.0f, st[i], lo[i]);
   }
-  frame[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
-  frame[1] = make_float4(st[0], st[1], st[2], 0.f);
-  frame[2] = make_float4(1.0f / st[0], 1.0f / st[1], 1.0f / st[2], 0.f);
-  uint32_t* leaf_bounds = reinterpret_cast<uint32_t*>(frame + 3);
-  for (int i = 0; i < 6; ++i) leaf_bounds[i] = i < 3 ? 0xffffffffu : 0u;
+  grid[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
+  grid[1] = make_float4(st[0], st[1], st[2], 0.f);
+  grid[2] = make_float4(1.0f / st[0], 1.0f / st[1], 1.0f / st[2], 0.f);
+  for (int i = 0; leaf_bounds && i < 6; ++i) leaf_bounds[i] = i < 3 ? 0xffffffffu : 0u;
   counts[0] = counts[1] = 0u;
 }
 
 __global__ void k_begin_refit(const uint32_t* __restrict__ bounds, float4* frame, unsigned* counts) {
-  begin_refit(bounds, frame, counts);
+  begin_refit(bounds, frame, reinterpret_cast<uint32_t*>(frame + 3), counts);
 }
 
 // Primitive centroid codes keep the top 7 bits of each axis (21 bits, three
@@ -131,12 +130,8 @@ __global__ void k_begin_refit(const uint32_t* __restrict__ bounds, float4* frame
 // (the cells then hold too many primitives).
 constexpr int kMortonBits = 21;
 
-__global__ void k_prim_morton(const float4* __restrict__ box, const uint32_t* __restrict__ ids,
-                              uint32_t n, const uint32_t* __restrict__ bounds, uint32_t* keys,
-                              float4* frame, unsigned* counts) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) begin_refit(bounds, frame, counts);
-  if (i >= n) return;
+__device__ __forceinline__ uint32_t prim_code(const float4 l, const float4 h,
+                                              const uint32_t* __restrict__ bounds) {
   float3 lo, hi, inv_ext;
   lo.x = from_ordered(__ldg(bounds)), lo.y = from_ordered(__ldg(bounds + 1));
   lo.z = from_ordered(__ldg(bounds + 2)), hi.x = from_ordered(__ldg(bounds + 3));
@@ -144,30 +139,36 @@ __global__ void k_prim_morton(const float4* __restrict__ box, const uint32_t* __
   inv_ext.x = hi.x > lo.x ? 1.f / (hi.x - lo.x) : 0.f;
   inv_ext.y = hi.y > lo.y ? 1.f / (hi.y - lo.y) : 0.f;
   inv_ext.z = hi.z > lo.z ? 1.f / (hi.z - lo.z) : 0.f;
-  const uint32_t id = ids[i];
-  const float4 l = box[2 * (size_t)id], h = box[2 * (size_t)id + 1];
   const float cx = (0.5f * (l.x + h.x) - lo.x) * inv_ext.x;
   const float cy = (0.5f * (l.y + h.y) - lo.y) * inv_ext.y;
   const float cz = (0.5f * (l.z + h.z) - lo.z) * inv_ext.z;
   const uint32_t qx = (uint32_t)min(1023.f, fmaxf(0.f, cx * 1024.f));
   const uint32_t qy = (uint32_t)min(1023.f, fmaxf(0.f, cy * 1024.f));
   const uint32_t qz = (uint32_t)min(1023.f, fmaxf(0.f, cz * 1024.f));
-  keys[i] = ((spread10(qx) << 2) | (spread10(qy) << 1) | spread10(qz)) >> (30 - kMortonBits);
+  return ((spread10(qx) << 2) | (spread10(qy) << 1) | spread10(qz)) >> (30 - kMortonBits);
 }
 
+__global__ void k_prim_morton(const float4* __restrict__ box, const uint32_t* __restrict__ ids,
+                              uint32_t n, const uint32_t* __restrict__ bounds, uint32_t* keys,
+                              float4* frame, unsigned* counts) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) begin_refit(bounds, frame, reinterpret_cast<uint32_t*>(frame + 3), counts);
+  if (i >= n) return;
+  const uint32_t id = ids[i];
+  keys[i] = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], bounds);
+}
 // Length of the common prefix of (key, index) at i and j; -1 outside [0, n).
 __device__ __forceinline__ int delta(const uint32_t* __restrict__ keys, int n, uint32_t ki, int i,
                                      int j) {
   if ((unsigned)j >= (unsigned)n) return -1;
-  const uint32_t x = ki ^ __ldg(keys + j);
+  const uint32_t x = ki ^ keys[j];
   return x ? __clz(x) : 32 + __clz((uint32_t)i ^ (uint32_t)j);
 }
 
-__global__ void k_karras(const uint32_t* __restrict__ keys, int n, int4* child,
-                         int* parent_int, int* parent_leaf) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n - 1) return;
-  const uint32_t ki = __ldg(keys + i);
+// Children and leaf range of internal node i; also writes their parent links.
+__device__ __forceinline__ int4 karras_node(const uint32_t* __restrict__ keys, int n, int i,
+                                            int* parent_int, int* parent_leaf) {
+  const uint32_t ki = keys[i];
   const int d = (delta(keys, n, ki, i, i + 1) - delta(keys, n, ki, i, i - 1)) >= 0 ? 1 : -1;
   const int dmin = delta(keys, n, ki, i, i - d);
   int lmax = 2;
@@ -200,7 +201,13 @@ __global__ void k_karras(const uint32_t* __restrict__ keys, int n, int4* child,
     c1 = gamma + 1;
     parent_int[gamma + 1] = i;
   }
-  child[i] = make_int4(c0, c1, lo, hi);  // children and the node's leaf range
+  return make_int4(c0, c1, lo, hi);
+}
+
+__global__ void k_karras(const uint32_t* __restrict__ keys, int n, int4* child,
+                         int* parent_int, int* parent_leaf) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n - 1) child[i] = karras_node(keys, n, i, parent_int, parent_leaf);
 }
 
 // The global primitive id of every leaf (Morton order).
@@ -220,8 +227,7 @@ __device__ __forceinline__ uint32_t q_axis(float l, float h, float lo, float inv
   const uint32_t qb = (uint32_t)fminf(fmaxf(b, 0.f), 65535.f);
   return qa | ((65535u - qb) << 16);
 }
-__device__ __forceinline__ QBox q_box(const float4 l, const float4 h, const float4* __restrict__ frame) {
-  const float4 lo = __ldg(frame), is = __ldg(frame + 2);
+__device__ __forceinline__ QBox q_box(const float4 l, const float4 h, const float4 lo, const float4 is) {
   return QBox{q_axis(l.x, h.x, lo.x, is.x), q_axis(l.y, h.y, lo.y, is.y), q_axis(l.z, h.z, lo.z, is.z)};
 }
 __device__ __forceinline__ QBox q_union(const QBox a, const QBox b) {
@@ -261,6 +267,52 @@ __device__ __forceinline__ void append_start(bool has, int v, unsigned* count, i
   if (lane == lead) base = atomicAdd(count, (unsigned)__popc(m));
   base = __shfl_sync(0xffffffffu, base, lead);
   if (has) list[base + __popc(m & ((1u << lane) - 1u))] = v;
+}
+
+// The block's bounds (shared memory, ordered float bits) widened by the boxes of
+// the threads with one.  Whole warps call it.
+__device__ __forceinline__ void widen_bounds(const float4 bl, const float4 bh, bool has, uint32_t* bound) {
+  const uint32_t lo[3] = {ordered_bits(bl.x + 0.f), ordered_bits(bl.y + 0.f), ordered_bits(bl.z + 0.f)};
+  const uint32_t hi[3] = {ordered_bits(bh.x + 0.f), ordered_bits(bh.y + 0.f), ordered_bits(bh.z + 0.f)};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t l = __reduce_min_sync(0xffffffffu, has ? lo[i] : 0xffffffffu);
+    const uint32_t h = __reduce_max_sync(0xffffffffu, has ? hi[i] : 0u);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMin(&bound[i], l);
+      atomicMax(&bound[3 + i], h);
+    }
+  }
+}
+
+// Records of the nodes whose leaves lie in the block's (thread j's node is
+// `node`, with children ch, if `local`), one level of readiness per round.
+// The whole block calls it, its leaves' ids and boxes and cleared flags in
+// shared memory.
+__device__ __forceinline__ void local_records(bool local, const int4 ch, int node, int b0, int j,
+                                              const uint32_t* s_id, const QBox* s_lbox, QBox* s_nbox,
+                                              unsigned char* s_done, uint4* nodes) {
+  bool pending = local;
+  for (;;) {
+    bool ready = false;
+    if (pending)
+      ready = (ch.x < 0 || s_done[ch.x - b0]) && (ch.y < 0 || s_done[ch.y - b0]);
+    if (ready) {
+      const QBox c0 = ch.x < 0 ? s_lbox[~ch.x - b0] : s_nbox[ch.x - b0];
+      const QBox c1 = ch.y < 0 ? s_lbox[~ch.y - b0] : s_nbox[ch.y - b0];
+      // a leaf child is named by its primitive id (the leaf lies in this block)
+      store_node(nodes, node, c0, ch.x < 0 ? ~(int)s_id[~ch.x - b0] : ch.x, c1,
+                 ch.y < 0 ? ~(int)s_id[~ch.y - b0] : ch.y);
+      s_nbox[j] = q_union(c0, c1);
+    }
+    const int any = __syncthreads_or(ready);  // this round's reads of s_done are over
+    if (ready) {
+      s_done[j] = 1;
+      pending = false;
+    }
+    if (!any) break;
+    __syncthreads();  // this round's flags are visible
+  }
 }
 
 // Leaf boxes and bottom-up bounds in one kernel.  Thread j of block b owns
@@ -311,7 +363,7 @@ __global__ void __launch_bounds__(B) k_gather_refit(
     s_id[j] = id;
     bl = box[2 * (size_t)id];
     bh = box[2 * (size_t)id + 1];
-    s_lbox[j] = q_box(bl, bh, frame);
+    s_lbox[j] = q_box(bl, bh, __ldg(frame), __ldg(frame + 2));
   }
   if (j < 6) s_bound[j] = j < 3 ? 0xffffffffu : 0u;
   __syncthreads();
@@ -319,19 +371,7 @@ __global__ void __launch_bounds__(B) k_gather_refit(
   // them): the block's, and of those the few that reach further than any so
   // far (one read a block: a read a warp queued up at the one line, 0.17 ms
   // for 4.6M leaves)
-  {
-    const uint32_t lo[3] = {ordered_bits(bl.x + 0.f), ordered_bits(bl.y + 0.f), ordered_bits(bl.z + 0.f)};
-    const uint32_t hi[3] = {ordered_bits(bh.x + 0.f), ordered_bits(bh.y + 0.f), ordered_bits(bh.z + 0.f)};
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const uint32_t l = __reduce_min_sync(0xffffffffu, leaf < n ? lo[i] : 0xffffffffu);
-      const uint32_t h = __reduce_max_sync(0xffffffffu, leaf < n ? hi[i] : 0u);
-      if ((j & 31) == 0) {
-        atomicMin(&s_bound[i], l);
-        atomicMax(&s_bound[3 + i], h);
-      }
-    }
-  }
+  widen_bounds(bl, bh, leaf < n, s_bound);
   __syncthreads();
   if (j < 6) {
     uint32_t* g = reinterpret_cast<uint32_t*>(frame + 3) + j;
@@ -342,28 +382,8 @@ __global__ void __launch_bounds__(B) k_gather_refit(
       atomicMax(g, v);
     }
   }
-  // 2. local subtrees, one level of readiness per round
-  bool pending = node_local;
-  for (;;) {
-    bool ready = false;
-    if (pending)
-      ready = (ch.x < 0 || s_done[ch.x - b0]) && (ch.y < 0 || s_done[ch.y - b0]);
-    if (ready) {
-      const QBox c0 = ch.x < 0 ? s_lbox[~ch.x - b0] : s_nbox[ch.x - b0];
-      const QBox c1 = ch.y < 0 ? s_lbox[~ch.y - b0] : s_nbox[ch.y - b0];
-      // a leaf child is named by its primitive id (the leaf lies in this block)
-      store_node(nodes, node, c0, ch.x < 0 ? ~(int)s_id[~ch.x - b0] : ch.x, c1,
-                 ch.y < 0 ? ~(int)s_id[~ch.y - b0] : ch.y);
-      s_nbox[j] = q_union(c0, c1);
-    }
-    const int any = __syncthreads_or(ready);  // this round's reads of s_done are over
-    if (ready) {
-      s_done[j] = 1;
-      pending = false;
-    }
-    if (!any) break;
-    __syncthreads();  // this round's flags are visible
-  }
+  // 2. local subtrees
+  local_records(node_local, ch, node, b0, j, s_id, s_lbox, s_nbox, s_done, nodes);
   // 3. nodes that span blocks: empty child boxes, widened by k_climb
   const bool spans = has_node && !node_local;
   const unsigned m = __ballot_sync(0xffffffffu, spans);
@@ -413,7 +433,7 @@ __global__ void k_climb(const unsigned* __restrict__ counts, const int* __restri
     int p;
     if (cur < 0) {
       const size_t id = __ldg(leaf_id + ~cur);
-      u = q_box(__ldg(box + 2 * id), __ldg(box + 2 * id + 1), frame);
+      u = q_box(__ldg(box + 2 * id), __ldg(box + 2 * id + 1), __ldg(frame), __ldg(frame + 2));
       p = __ldg(parent_leaf + ~cur);
     } else {
       u = q_union(q_of(__ldg(nodes + 2 * (size_t)cur)), q_of(__ldg(nodes + 2 * (size_t)cur + 1)));
@@ -447,6 +467,108 @@ __global__ void k_span_records(const unsigned* __restrict__ counts, const int* _
     store_node(nodes, node, QBox{r[0] | r[1] << 16, r[2] | r[3] << 16, r[4] | r[5] << 16}, c0,
                QBox{r[6] | r[7] << 16, r[8] | r[9] << 16, r[10] | r[11] << 16}, c1);
   }
+}
+
+// A whole BVH of 2 to 1,024 leaves in one block, a leaf and a node per thread:
+// codes, their stable sort (lanes with equal digits by votes, digits counted
+// per warp, pairs exchanged through shared memory), Karras' nodes, the records
+// and bounds.  `ids` null: every primitive in order.  The nine kernels it
+// takes the place of (79 us for 1,024 leaves, launched one after the other)
+// are latency and no work.
+constexpr int kSmallLeaves = 1024, kSmallWarps = kSmallLeaves / 32;
+struct SmallBvh {
+  union {
+    uint32_t whist[kSmallWarps][256];  // during the sort
+    struct {
+      QBox lbox[kSmallLeaves], nbox[kSmallLeaves];
+    } box;
+  };
+  uint32_t key[kSmallLeaves], id[kSmallLeaves];
+  unsigned char done[kSmallLeaves];
+  uint32_t sum[8], bound[6];
+  float4 grid[3];
+};
+__global__ void __launch_bounds__(kSmallLeaves)
+    k_small_bvh(const float4* __restrict__ box, const uint32_t* __restrict__ ids, int n,
+                const uint32_t* __restrict__ bounds, float4* frame, int4* child, int* parent_int,
+                int* parent_leaf, uint32_t* leaf_id, uint4* nodes) {
+  __shared__ SmallBvh sm;
+  const int j = threadIdx.x, lane = j & 31, w = j >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  if (j == 0) {
+    unsigned counts[2];
+    begin_refit(bounds, sm.grid, nullptr, counts);
+    frame[0] = sm.grid[0], frame[1] = sm.grid[1], frame[2] = sm.grid[2];
+  }
+  if (j < 6) sm.bound[j] = j < 3 ? 0xffffffffu : 0u;
+  const bool valid = j < n;
+  uint32_t id = valid ? (ids ? ids[j] : (uint32_t)j) : 0u, key = 0u;
+  if (valid) key = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], bounds);
+  for (int shift = 0; shift < kMortonBits; shift += 8) {
+    for (int i = j; i < kSmallWarps * 256; i += kSmallLeaves) (&sm.whist[0][0])[i] = 0;
+    __syncthreads();
+    const uint32_t d = (key >> shift) & 0xffu;
+    uint32_t peers = __ballot_sync(0xffffffffu, valid);
+    if (!valid) peers = ~peers;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const bool bit = (d >> b) & 1u;
+      const uint32_t vote = __ballot_sync(0xffffffffu, bit);
+      peers &= bit ? vote : ~vote;
+    }
+    const uint32_t in = __popc(peers & lt);
+    if (valid && in == 0) sm.whist[w][d] = __popc(peers);
+    __syncthreads();
+    uint32_t c = 0, incl = 0;
+    if (j < 256) {
+#pragma unroll 8
+      for (int q = 0; q < kSmallWarps; ++q) {
+        const uint32_t t = sm.whist[q][j];
+        sm.whist[q][j] = c;
+        c += t;
+      }
+      incl = c;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane == 31) sm.sum[w] = incl;
+    }
+    __syncthreads();
+    if (j < 256) {
+      uint32_t start = incl - c;
+      for (int q = 0; q < w; ++q) start += sm.sum[q];
+      for (int q = 0; q < kSmallWarps; ++q) sm.whist[q][j] += start;
+    }
+    __syncthreads();
+    if (valid) {
+      const uint32_t q = sm.whist[w][d] + in;
+      sm.key[q] = key;
+      sm.id[q] = id;
+    }
+    __syncthreads();
+    if (valid) {
+      key = sm.key[j];
+      id = sm.id[j];
+    }
+  }
+  // leaves: boxes on the grid and exact bounds (the whist words are free)
+  __syncthreads();
+  float4 bl = make_float4(0.f, 0.f, 0.f, 0.f), bh = bl;
+  if (valid) {
+    bl = box[2 * (size_t)id];
+    bh = box[2 * (size_t)id + 1];
+    sm.box.lbox[j] = q_box(bl, bh, sm.grid[0], sm.grid[2]);
+    leaf_id[j] = id;
+  }
+  sm.done[j] = 0;
+  widen_bounds(bl, bh, valid, sm.bound);
+  const bool has_node = j < n - 1;
+  int4 ch = make_int4(0, 0, -1, -1);
+  if (has_node) child[j] = ch = karras_node(sm.key, n, j, parent_int, parent_leaf);
+  __syncthreads();
+  if (j < 6) reinterpret_cast<uint32_t*>(frame + 3)[j] = sm.bound[j];
+  local_records(has_node, ch, j, 0, j, sm.id, sm.box.lbox, sm.box.nbox, sm.done, nodes);
 }
 
 __global__ void k_bytes_differ(const uint8_t* __restrict__ x, const uint8_t* __restrict__ y,
@@ -514,9 +636,11 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
   uint32_t* ids = nullptr;
   if (a->C == 0 || a->n_levels == 0 || lod_dev == nullptr) {
     n = N * S;
-    HR_TRY(scratch(ctx, 30, (size_t)n * 4, (void**)&ids));
-    k_iota<<<(n + 255) / 256, 256, 0, st>>>(ids, n);
-    HR_LAUNCHED(ctx);
+    if (n < 2 || n > (uint32_t)kSmallLeaves) {
+      HR_TRY(scratch(ctx, 30, (size_t)n * 4, (void**)&ids));
+      k_iota<<<(n + 255) / 256, 256, 0, st>>>(ids, n);
+      HR_LAUNCHED(ctx);
+    }
   } else {
     const uint32_t C = a->C, L = a->n_levels;
     uint32_t* cnt = nullptr;
@@ -572,6 +696,14 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
     HR_CUDA(ctx, cudaMemcpyAsync(bv.lod_built, lod_dev, a->C, cudaMemcpyDeviceToDevice, st));
   }
   if (n == 0) {
+    bv.valid = 1;
+    bv.topo = 1;
+    return HR_OK;
+  }
+  if (n >= 2 && n <= (uint32_t)kSmallLeaves) {  // all in one block
+    k_small_bvh<<<1, kSmallLeaves, 0, st>>>(a->prim_box, ids, (int)n, a->d_bounds, bv.frame, bv.child,
+                                            bv.par_int, bv.par_leaf, bv.leaf_id, bv.nodes);
+    HR_LAUNCHED(ctx);
     bv.valid = 1;
     bv.topo = 1;
     return HR_OK;
