@@ -288,12 +288,7 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
 // Root quantisation q = min(1023, floor((p - lo) * (1024 / e))) in the roots'
 // bounding cube (lo its low corner, e the largest extent), every operation
 // rounded to FP32 in this order; code = x bits at 3i+2, y at 3i+1, z at 3i.
-__global__ void k_root_morton(const float4* __restrict__ verts, uint32_t N, uint32_t S,
-                              const uint32_t* __restrict__ bounds, uint32_t* keys,
-                              uint32_t* vals) {
-  const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
-  const float4 p = verts[(size_t)s * (S + 1)];
+__device__ __forceinline__ uint32_t root_code(const float4 p, const uint32_t* bounds) {
   const float c[3] = {p.x, p.y, p.z};
   float ext = 0.f;
   for (int i = 0; i < 3; ++i)
@@ -306,7 +301,15 @@ __global__ void k_root_morton(const float4* __restrict__ verts, uint32_t N, uint
     const int qi = (int)floorf(v);
     q[i] = (uint32_t)min(1023, max(0, qi));
   }
-  keys[s] = (spread10(q[0]) << 2) | (spread10(q[1]) << 1) | spread10(q[2]);
+  return (spread10(q[0]) << 2) | (spread10(q[1]) << 1) | spread10(q[2]);
+}
+
+__global__ void k_root_morton(const float4* __restrict__ verts, uint32_t N, uint32_t S,
+                              const uint32_t* __restrict__ bounds, uint32_t* keys,
+                              uint32_t* vals) {
+  const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= N) return;
+  keys[s] = root_code(verts[(size_t)s * (S + 1)], bounds);
   vals[s] = s;
 }
 
@@ -328,6 +331,142 @@ __global__ void k_words_differ(const uint32_t* __restrict__ x, const uint32_t* _
                                uint32_t n, uint32_t* flag) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n && x[i] != y[i]) *flag = 1u;
+}
+
+// The whole of the above for up to 1,024 * IT strands in one block: root
+// bounds, codes, their stable sort (8 bits a pass: lanes with equal digits by
+// votes, digits counted per warp, pairs exchanged through shared memory),
+// whether the order changed, cluster ids and cluster starts.  Each of the
+// twelve kernels and copies it takes the place of is a few microseconds of
+// latency on next to no work, and a frame's clusters lie on the chain that
+// small frames are bound by: for 3,001 strands 63 us of kernels and their gaps
+// became one of 23.
+constexpr uint32_t kSmallThreads = 1024, kSmallWarps = kSmallThreads / 32;
+template <int IT>
+constexpr size_t small_clusters_bytes() {
+  return kSmallWarps * 256 * sizeof(uint32_t) + (size_t)kSmallThreads * IT * (sizeof(uint32_t) + sizeof(uint16_t));
+}
+template <int IT>
+__global__ void __launch_bounds__(kSmallThreads)
+    k_small_clusters(const float4* __restrict__ verts, uint32_t N, uint32_t S, uint32_t C,
+                     uint32_t* order, uint32_t* cluster_of, uint32_t* cl_first, uint32_t* changed) {
+  extern __shared__ uint32_t sm[];
+  uint32_t* whist = sm;                              // [warp][digit]
+  uint32_t* s_key = sm + kSmallWarps * 256;
+  uint16_t* s_val = reinterpret_cast<uint16_t*>(s_key + kSmallThreads * IT);
+  __shared__ uint32_t s_bounds[6], s_sum[8];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, lt = (1u << lane) - 1u;
+  const uint32_t base = w * 32 * IT + lane;  // item j of the thread is rank base + 32 j
+  if (threadIdx.x < 6) s_bounds[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
+  __syncthreads();
+  uint32_t lo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi[3] = {0, 0, 0};
+#pragma unroll
+  for (int j = 0; j < IT; ++j) {
+    const uint32_t p = base + 32 * j;
+    if (p >= N) continue;
+    const float4 v = __ldg(verts + (size_t)p * (S + 1));
+    const uint32_t c[3] = {ordered_bits(v.x), ordered_bits(v.y), ordered_bits(v.z)};
+    for (int i = 0; i < 3; ++i) lo[i] = min(lo[i], c[i]), hi[i] = max(hi[i], c[i]);
+  }
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t l = __reduce_min_sync(0xffffffffu, lo[i]), h = __reduce_max_sync(0xffffffffu, hi[i]);
+    if (lane == 0) {
+      atomicMin(&s_bounds[i], l);
+      atomicMax(&s_bounds[3 + i], h);
+    }
+  }
+  __syncthreads();
+  uint32_t key[IT], val[IT];
+#pragma unroll
+  for (int j = 0; j < IT; ++j) {
+    const uint32_t p = base + 32 * j;
+    key[j] = p < N ? root_code(__ldg(verts + (size_t)p * (S + 1)), s_bounds) : 0u;
+    val[j] = p;
+  }
+  for (int shift = 0; shift < 30; shift += 8) {
+    for (uint32_t i = threadIdx.x; i < kSmallWarps * 256; i += kSmallThreads) whist[i] = 0;
+    __syncthreads();
+    uint32_t* mine = whist + w * 256;
+    uint16_t local[IT];
+#pragma unroll
+    for (int j = 0; j < IT; ++j) {
+      const bool valid = base + 32 * j < N;
+      const uint32_t d = (key[j] >> shift) & 0xffu;
+      uint32_t peers = __ballot_sync(0xffffffffu, valid);
+      if (!valid) peers = ~peers;
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        const bool bit = (d >> b) & 1u;
+        const uint32_t vote = __ballot_sync(0xffffffffu, bit);
+        peers &= bit ? vote : ~vote;
+      }
+      const uint32_t in = __popc(peers & lt), prior = valid ? mine[d] : 0u;
+      local[j] = (uint16_t)(prior + in);
+      __syncwarp();
+      if (valid && in == 0) mine[d] = prior + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    // places of a digit: over the warps, then over the digits
+    uint32_t c = 0, incl = 0;
+    if (threadIdx.x < 256) {
+#pragma unroll 8
+      for (uint32_t q = 0; q < kSmallWarps; ++q) {
+        const uint32_t t = whist[q * 256 + threadIdx.x];
+        whist[q * 256 + threadIdx.x] = c;
+        c += t;
+      }
+      incl = c;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += t;
+      }
+      if (lane == 31) s_sum[w] = incl;
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {
+      uint32_t start = incl - c;
+      for (uint32_t q = 0; q < w; ++q) start += s_sum[q];
+      for (uint32_t q = 0; q < kSmallWarps; ++q) whist[q * 256 + threadIdx.x] += start;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < IT; ++j)
+      if (base + 32 * j < N) {
+        const uint32_t q = mine[(key[j] >> shift) & 0xffu] + local[j];
+        s_key[q] = key[j];
+        s_val[q] = (uint16_t)val[j];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < IT; ++j) {
+      const uint32_t p = base + 32 * j;
+      if (p < N) {
+        key[j] = s_key[p];
+        val[j] = s_val[p];
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < IT; ++j) {
+    const uint32_t p = base + 32 * j;
+    if (p >= N) continue;
+    if (order[p] != val[j]) *changed = 1u;
+    order[p] = val[j];
+    cluster_of[val[j]] = (uint32_t)(((uint64_t)p * C) / N);
+  }
+  for (uint32_t c = threadIdx.x; c <= C; c += kSmallThreads)
+    cl_first[c] = (uint32_t)(((uint64_t)c * N + C - 1) / C);
+}
+
+template <int IT>
+hr_status small_clusters(hr_ctx* ctx, hr_asset* a, uint32_t C, cudaStream_t st) {
+  HR_CUDA(ctx, cudaFuncSetAttribute(k_small_clusters<IT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)small_clusters_bytes<IT>()));
+  k_small_clusters<IT><<<1, kSmallThreads, small_clusters_bytes<IT>(), st>>>(
+      a->verts, a->N, a->S, C, a->order, a->cluster_of, a->cl_first, a->d_bounds + kHierChanged);
+  HR_LAUNCHED(ctx);
+  return HR_OK;
 }
 
 // cluster_of of the strands of cluster c (ranks cl_first[c] .. cl_first[c+1]-1)
@@ -1073,7 +1212,15 @@ hr_status build_hierarchy(hr_ctx* ctx, hr_asset* a, uint32_t C, uint32_t max_lev
   uint64_t E = 0, total = 0;
   HR_TRY(hierarchy_setup(ctx, a, C, max_levels, li, E, total));
   drop_guides(ctx, a);  // a Morton hierarchy replaces a guide-driven one
-  // K1: Morton order of the roots
+  // K1: Morton order of the roots; up to 8,192 in one block (23 us for 3,001,
+  // where the separate kernels take 63 and their gaps; with 16 strands a
+  // thread, 10,000 took 74 us and the separate kernels no more)
+  if (N <= kSmallThreads * 8) {
+    HR_TRY(N <= kSmallThreads       ? small_clusters<1>(ctx, a, C, st)
+           : N <= kSmallThreads * 4 ? small_clusters<4>(ctx, a, C, st)
+                                    : small_clusters<8>(ctx, a, C, st));
+    return hierarchy_finish(ctx, a, li, E, total, fit_begin, fit_end, st_fit);
+  }
   uint32_t *bounds, *keys, *vals, *k2, *v2;
   HR_TRY(scratch(ctx, 0, 64, (void**)&bounds));
   HR_TRY(scratch(ctx, 1, (size_t)N * 4, (void**)&keys));
