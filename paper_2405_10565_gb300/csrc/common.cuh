@@ -218,9 +218,33 @@ hr_status root_morton_order(hr_ctx* ctx, hr_asset* a, uint32_t* codes, uint32_t*
 hr_status build_hierarchy_from(hr_ctx* ctx, hr_asset* a, uint32_t C, uint32_t max_levels,
                                const uint32_t* order_dev, const uint32_t* cl_first_dev);
 
-// The thick-hair materials and segment records from the current
-// cross-sections (after skinning moved them; no new fit).
-hr_status rebuild_eth_records(hr_ctx* ctx, hr_asset* a);
+// The strands moved by the guides' new poses gv: vertices, records and bounds;
+// and the thick hairs' segment records from their moved cross-sections (their
+// materials and radii stay), after skin_strands on the same stream.
+hr_status skin_strands(hr_ctx* ctx, hr_asset* a, const float4* gv);
+hr_status moved_eth_records(hr_ctx* ctx, hr_asset* a);
+
+// The three guides (10 bits each) of a cluster.
+__device__ __forceinline__ void tri_of(uint32_t key, uint32_t& a, uint32_t& b, uint32_t& c) {
+  a = key >> 20;
+  b = (key >> 10) & 1023u;
+  c = key & 1023u;
+}
+// A point from its weights in the prism of three guide points.
+__device__ __forceinline__ float3 skin(const float4 w, const float4 g0, const float4 g1,
+                                       const float4 g2) {
+  if (w.w > 0.5f) return make_float3(g0.x + w.x, g0.y + w.y, g0.z + w.z);
+  const float3 e1 = make_float3(g1.x - g0.x, g1.y - g0.y, g1.z - g0.z);
+  const float3 e2 = make_float3(g2.x - g0.x, g2.y - g0.y, g2.z - g0.z);
+  float3 n = make_float3(e1.y * e2.z - e1.z * e2.y, e1.z * e2.x - e1.x * e2.z,
+                         e1.x * e2.y - e1.y * e2.x);
+  const float nn = sqrtf(n.x * n.x + n.y * n.y + n.z * n.z);
+  const float inv = nn > 0.f ? 1.f / nn : 0.f;
+  n = make_float3(n.x * inv, n.y * inv, n.z * inv);
+  return make_float3(g0.x + w.x * e1.x + w.y * e2.x + w.z * n.x,
+                     g0.y + w.x * e1.y + w.y * e2.y + w.z * n.y,
+                     g0.z + w.x * e1.z + w.y * e2.z + w.z * n.z);
+}
 
 // --- guides.cu
 // Free the guide-driven state of an asset (its hierarchy is being replaced).

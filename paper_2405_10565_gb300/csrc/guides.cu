@@ -626,12 +626,6 @@ __device__ __forceinline__ df df_diff(float x, float y) {
   return df{s, e};
 }
 
-__device__ __forceinline__ void tri_of(uint32_t key, uint32_t& a, uint32_t& b, uint32_t& c) {
-  a = key >> 20;
-  b = (key >> 10) & 1023u;
-  c = key & 1023u;
-}
-
 __device__ __forceinline__ uint32_t eth_cluster(uint32_t e, const uint32_t* off, uint32_t L) {
   uint32_t k = 0;
   while (k + 1 < L && e >= off[k + 1]) ++k;
@@ -704,21 +698,6 @@ __global__ void __launch_bounds__(kWeightBlock)
 }
 
 // ---------------------------------------------------------------- skinning (FP32)
-
-__device__ __forceinline__ float3 skin(const float4 w, const float4 g0, const float4 g1,
-                                       const float4 g2) {
-  if (w.w > 0.5f) return make_float3(g0.x + w.x, g0.y + w.y, g0.z + w.z);
-  const float3 e1 = make_float3(g1.x - g0.x, g1.y - g0.y, g1.z - g0.z);
-  const float3 e2 = make_float3(g2.x - g0.x, g2.y - g0.y, g2.z - g0.z);
-  float3 n = make_float3(e1.y * e2.z - e1.z * e2.y, e1.z * e2.x - e1.x * e2.z,
-                         e1.x * e2.y - e1.y * e2.x);
-  const float nn = sqrtf(n.x * n.x + n.y * n.y + n.z * n.z);
-  const float inv = nn > 0.f ? 1.f / nn : 0.f;
-  n = make_float3(n.x * inv, n.y * inv, n.z * inv);
-  return make_float3(g0.x + w.x * e1.x + w.y * e2.x + w.z * n.x,
-                     g0.y + w.x * e1.y + w.y * e2.y + w.z * n.y,
-                     g0.z + w.x * e1.z + w.y * e2.z + w.z * n.z);
-}
 
 // New strand vertices from the guides' new vertices gv [G][S1] (radius kept).
 __global__ void k_skin_strands(const float4* __restrict__ gv, uint32_t N, uint32_t S1,
@@ -943,10 +922,14 @@ hr_status build_guided_hierarchy(hr_ctx* ctx, hr_asset* a, uint32_t G, uint32_t 
 hr_status skin_asset(hr_ctx* ctx, hr_asset* a, const float4* gv_dev) {
   cudaStream_t st = ctx_stream(ctx);
   const uint32_t N = a->N, S1 = a->S + 1;
-  k_skin_strands<<<blocks_for((uint64_t)N * S1, 256), 256, 0, st>>>(gv_dev, N, S1, a->cluster_of,
-                                                                   a->cl_tri, a->w_strand, a->verts);
-  HR_LAUNCHED(ctx);
-  HR_TRY(refresh_strand_prims(ctx, a));
+  if (S1 <= kUpdateMaxVerts) {
+    HR_TRY(skin_strands(ctx, a, gv_dev));
+  } else {  // strands too long for a block's shared memory
+    k_skin_strands<<<blocks_for((uint64_t)N * S1, 256), 256, 0, st>>>(gv_dev, N, S1, a->cluster_of,
+                                                                     a->cl_tri, a->w_strand, a->verts);
+    HR_LAUNCHED(ctx);
+    HR_TRY(refresh_strand_prims(ctx, a));
+  }
   if (a->E) {
     Offs lv{};
     lv.n_levels = a->n_levels;
@@ -954,7 +937,7 @@ hr_status skin_asset(hr_ctx* ctx, hr_asset* a, const float4* gv_dev) {
     k_skin_eth<<<blocks_for((uint64_t)a->E * S1, 256), 256, 0, st>>>(gv_dev, S1, a->E, lv, a->cl_tri,
                                                                     a->w_eth, a->xsec);
     HR_LAUNCHED(ctx);
-    HR_TRY(rebuild_eth_records(ctx, a));
+    HR_TRY(moved_eth_records(ctx, a));
   }
   a->bvh.valid = 0;
   return HR_OK;

@@ -103,14 +103,13 @@ __device__ __forceinline__ float3 crossf(float3 a, float3 b) {
 // correctly rounded value, and each offset is the compensated dot product of
 // the stored row with c0, so the stored cylinder passes through c0 to within
 // the offset's own rounding.
-__device__ void write_prim(float4* uv, float4* w, float4* box, float3 c0, float3 c1, float3 e1, float a,
-                           float b) {
+__device__ __forceinline__ void write_prim(float4* uv, float4* w, float4* box, float3 c0, float3 c1,
+                                           float3 e1, float a, float b, float4& lo, float4& hi) {
   const float3 ax = sub3(c1, c0);
   const float L2 = dotf(ax, ax);
   if (!(L2 > 0.f)) {
     uv[0] = uv[1] = w[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-    box[0] = make_float4(c0.x, c0.y, c0.z, 0.f);
-    box[1] = box[0];
+    box[0] = box[1] = lo = hi = make_float4(c0.x, c0.y, c0.z, 0.f);
     return;
   }
   const float3 t = mul3(ax, 1.0f / sqrtf(L2));
@@ -126,9 +125,9 @@ __device__ void write_prim(float4* uv, float4* w, float4* box, float3 c0, float3
   const float hx = sqrtf(fmaf(a * e1.x, a * e1.x, (b * e2.x) * (b * e2.x))) * ga;
   const float hy = sqrtf(fmaf(a * e1.y, a * e1.y, (b * e2.y) * (b * e2.y))) * ga;
   const float hz = sqrtf(fmaf(a * e1.z, a * e1.z, (b * e2.z) * (b * e2.z))) * ga;
-  box[0] = make_float4(__fsub_rd(fminf(c0.x, c1.x), hx), __fsub_rd(fminf(c0.y, c1.y), hy),
+  box[0] = lo = make_float4(__fsub_rd(fminf(c0.x, c1.x), hx), __fsub_rd(fminf(c0.y, c1.y), hy),
                        __fsub_rd(fminf(c0.z, c1.z), hz), 0.f);
-  box[1] = make_float4(__fadd_ru(fmaxf(c0.x, c1.x), hx), __fadd_ru(fmaxf(c0.y, c1.y), hy),
+  box[1] = hi = make_float4(__fadd_ru(fmaxf(c0.x, c1.x), hx), __fadd_ru(fmaxf(c0.y, c1.y), hy),
                        __fadd_ru(fmaxf(c0.z, c1.z), hz), 0.f);
 }
 
@@ -183,26 +182,79 @@ __global__ void k_strand_prims(const float4* __restrict__ verts, const float4* _
     e1 = make_float3(fmaf(b1.x, sh.x, b2.x * sh.y), fmaf(b1.y, sh.x, b2.y * sh.y),
                      fmaf(b1.z, sh.x, b2.z * sh.y));
   }
-  write_prim(uv + idx * 2, wa + idx * 2, box + idx * 2, p0, p1, e1, sh.z, sh.w);
+  float4 lo, hi;
+  write_prim(uv + idx * 2, wa + idx * 2, box + idx * 2, p0, p1, e1, sh.z, sh.w, lo, hi);
   wa[idx * 2 + 1] = make_float4(__uint_as_float(s), 0.f, r, sh.z * sh.w);
 }
 
-// New strand positions in one pass: each block reads the vertices of
-// `per_block` whole strands once, from device memory or from page-locked host
-// memory mapped into the device's address space (so the transfer and the
-// record build overlap), keeps them in shared memory, writes the asset's
-// device copy, and builds every segment record of its strands exactly as
-// k_strand_shape and k_strand_prims do.
-__global__ void k_strand_update(const float4* __restrict__ src, float4* __restrict__ verts,
+// Ordered float bits of a box widened into a thread's bounds, and a block's
+// bounds folded into the global ones: nothing to do once another block has
+// reached as far.  The whole block calls fold_bounds.
+__device__ __forceinline__ void widen(uint32_t b[6], const float4 l, const float4 h) {
+  b[0] = min(b[0], ordered_bits(l.x)), b[1] = min(b[1], ordered_bits(l.y)), b[2] = min(b[2], ordered_bits(l.z));
+  b[3] = max(b[3], ordered_bits(h.x)), b[4] = max(b[4], ordered_bits(h.y)), b[5] = max(b[5], ordered_bits(h.z));
+}
+__device__ __forceinline__ void fold_bounds(const uint32_t b[6], uint32_t* bounds) {
+  __shared__ uint32_t s_b[6];
+  if (threadIdx.x < 6) s_b[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const uint32_t v = i < 3 ? __reduce_min_sync(0xffffffffu, b[i]) : __reduce_max_sync(0xffffffffu, b[i]);
+    if ((threadIdx.x & 31) == 0) {
+      if (i < 3) atomicMin(&s_b[i], v); else atomicMax(&s_b[i], v);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    const uint32_t v = s_b[threadIdx.x], g = __ldcg(bounds + threadIdx.x);
+    if (threadIdx.x < 3) {
+      if (v < g) atomicMin(bounds + threadIdx.x, v);
+    } else if (v > g) {
+      atomicMax(bounds + threadIdx.x, v);
+    }
+  }
+}
+
+// Where a strand's new vertices come from: given ones, or the guides' new
+// poses through the skinning weights (the radius is kept).
+struct GivenVerts {
+  const float4* src;
+  __device__ __forceinline__ float4 operator()(uint32_t, uint32_t, size_t idx) const { return src[idx]; }
+};
+struct SkinnedVerts {
+  const float4 *guides, *weights, *old;
+  const uint32_t *cluster_of, *cl_tri;
+  uint32_t S1;
+  __device__ __forceinline__ float4 operator()(uint32_t strand, uint32_t k, size_t idx) const {
+    uint32_t ga, gb, gc;
+    tri_of(__ldg(cl_tri + __ldg(cluster_of + strand)), ga, gb, gc);
+    const float3 p = skin(__ldg(weights + idx), __ldg(guides + (size_t)ga * S1 + k),
+                          __ldg(guides + (size_t)gb * S1 + k), __ldg(guides + (size_t)gc * S1 + k));
+    return make_float4(p.x, p.y, p.z, old[idx].w);
+  }
+};
+
+// New strand positions in one pass: each block takes the vertices of
+// `per_block` whole strands once (from device memory, from page-locked host
+// memory mapped into the device's address space, so that the transfer and the
+// record build overlap, or skinned), keeps them in shared memory, writes the
+// asset's device copy, builds every segment record of its strands exactly as
+// k_strand_shape and k_strand_prims do and folds their boxes into the scene's
+// bounds (a pass over the boxes by itself took 69 us for 6.4M segments; skinned
+// vertices, shapes, records and bounds in four kernels 260 us).
+template <typename Src>
+__global__ void k_strand_update(const Src src, float4* verts,
                                 const float2* __restrict__ shape, uint32_t N, uint32_t S,
-                                uint32_t per_block, float4* uv, float4* box, float4* wa) {
+                                uint32_t per_block, float4* uv, float4* box, float4* wa,
+                                uint32_t* bounds) {
   extern __shared__ float4 sv[];  // per_block * (S + 1) vertices, then per_block shapes
   const uint32_t s0 = blockIdx.x * per_block;
   const uint32_t ns = min(per_block, N - s0);
   const uint32_t nv = ns * (S + 1);
   const size_t v0 = (size_t)s0 * (S + 1);
   for (uint32_t i = threadIdx.x; i < nv; i += blockDim.x) {
-    const float4 v = src[v0 + i];
+    const float4 v = src(s0 + i / (S + 1), i % (S + 1), v0 + i);
     sv[i] = v;
     verts[v0 + i] = v;
   }
@@ -217,6 +269,7 @@ __global__ void k_strand_update(const float4* __restrict__ src, float4* __restri
     ssh[threadIdx.x] = make_float4(cp, sp, r / q, r * q);
   }
   __syncthreads();
+  uint32_t b[6] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
   for (uint32_t i = threadIdx.x; i < ns * S; i += blockDim.x) {
     const uint32_t ls = i / S, k = i % S;
     const float4* P = sv + ls * (S + 1);
@@ -234,9 +287,12 @@ __global__ void k_strand_update(const float4* __restrict__ src, float4* __restri
                        fmaf(b1.z, sh.x, b2.z * sh.y));
     }
     const size_t idx = (size_t)(s0 + ls) * S + k;
-    write_prim(uv + idx * 2, wa + idx * 2, box + idx * 2, p0, p1, e1, sh.z, sh.w);
+    float4 lo, hi;
+    write_prim(uv + idx * 2, wa + idx * 2, box + idx * 2, p0, p1, e1, sh.z, sh.w, lo, hi);
     wa[idx * 2 + 1] = make_float4(__uint_as_float(s0 + ls), 0.f, r, sh.z * sh.w);
+    widen(b, lo, hi);
   }
+  fold_bounds(b, bounds);
 }
 
 // ------------------------------------------------------------ Morton clusters
@@ -904,7 +960,7 @@ __global__ void k_eth_material(const float4* __restrict__ verts, uint32_t N, uin
 __device__ __forceinline__ bool eth_prim(const float4* __restrict__ xsec, uint32_t N, uint32_t S,
                                          const uint32_t* __restrict__ cl_first, const LevelInfo& li,
                                          const float* __restrict__ eth_r, uint64_t idx, float4* uv,
-                                         float4* box, float4* wa) {
+                                         float4* box, float4* wa, float4& lo, float4& hi) {
   const uint32_t e = (uint32_t)(idx / S), k = (uint32_t)(idx % S);
   const float4* x0 = xsec + ((size_t)e * (S + 1) + k) * 3;
   const float4 q0 = __ldg(x0), q1 = __ldg(x0 + 1), r0 = __ldg(x0 + 3), r1 = __ldg(x0 + 4);
@@ -927,8 +983,9 @@ __device__ __forceinline__ bool eth_prim(const float4* __restrict__ xsec, uint32
     wa[p * 2 + 1] = make_float4(__uint_as_float(N + e), 0.f, 0.f, 0.f);
     return false;
   }
-  write_prim(uv + p * 2, wa + p * 2, box + p * 2, c0, c1, e1, a, b);
-  wa[p * 2 + 1] = make_float4(__uint_as_float(N + e), (float)cnt, eth_r[e], a * b);
+  write_prim(uv + p * 2, wa + p * 2, box + p * 2, c0, c1, e1, a, b, lo, hi);
+  const float r = eth_r ? eth_r[e] : wa[p * 2 + 1].z;  // none given: the radius stays
+  wa[p * 2 + 1] = make_float4(__uint_as_float(N + e), (float)cnt, r, a * b);
   return true;
 }
 
@@ -940,35 +997,11 @@ __global__ void k_eth_prims(const float4* __restrict__ xsec, uint32_t N, uint32_
                             const float* __restrict__ eth_r, float4* uv, float4* box,
                             float4* wa, uint32_t* bounds) {
   const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  __shared__ uint32_t s_b[6];
-  if (threadIdx.x < 6) s_b[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
-  __syncthreads();
-  const bool live = idx < (uint64_t)E * S &&
-                    eth_prim(xsec, N, S, cl_first, li, eth_r, idx, uv, box, wa);
-  uint32_t b[6];
-  const size_t p = (size_t)N * S + idx;
-  if (live) {
-    const float4 l = box[2 * p], h = box[2 * p + 1];
-    b[0] = ordered_bits(l.x), b[1] = ordered_bits(l.y), b[2] = ordered_bits(l.z);
-    b[3] = ordered_bits(h.x), b[4] = ordered_bits(h.y), b[5] = ordered_bits(h.z);
-  }
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const uint32_t v = i < 3 ? __reduce_min_sync(0xffffffffu, live ? b[i] : 0xffffffffu)
-                             : __reduce_max_sync(0xffffffffu, live ? b[i] : 0u);
-    if ((threadIdx.x & 31) == 0) {
-      if (i < 3) atomicMin(&s_b[i], v); else atomicMax(&s_b[i], v);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < 6) {  // nothing to do once another block has reached as far
-    const uint32_t v = s_b[threadIdx.x], g = __ldcg(bounds + threadIdx.x);
-    if (threadIdx.x < 3) {
-      if (v < g) atomicMin(bounds + threadIdx.x, v);
-    } else if (v > g) {
-      atomicMax(bounds + threadIdx.x, v);
-    }
-  }
+  uint32_t b[6] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
+  float4 lo, hi;
+  if (idx < (uint64_t)E * S && eth_prim(xsec, N, S, cl_first, li, eth_r, idx, uv, box, wa, lo, hi))
+    widen(b, lo, hi);
+  fold_bounds(b, bounds);
 }
 
 // Scene bounds over all primitive boxes (ordered-bit atomics).
@@ -1002,6 +1035,12 @@ __global__ void k_init_bounds(uint32_t* bounds) {
   else if (threadIdx.x < 6) bounds[threadIdx.x] = 0u;
 }
 
+// The strands' and the thick hairs' bounds of an asset.
+__global__ void k_init_all_bounds(uint32_t* bounds) {
+  const uint32_t i = threadIdx.x & 7;
+  if (i < 6) bounds[(threadIdx.x < 8 ? 0 : kEthBounds) + i] = i < 3 ? 0xffffffffu : 0u;
+}
+
 // Bounds of the first n primitive boxes into a->d_bounds (ordered float
 // bits: lo xyz, hi xyz), on the stream; nothing is read back.
 hr_status scene_bounds(hr_ctx* ctx, hr_asset* a, uint64_t n, cudaStream_t st = nullptr) {
@@ -1029,18 +1068,39 @@ hr_status build_strand_prims(hr_ctx* ctx, hr_asset* a) {
   return refresh_strand_prims(ctx, a);
 }
 
-// Strand segment records and scene bounds from the current vertices, into
-// the asset's existing arrays (the first N * S records).
-hr_status update_strands(hr_ctx* ctx, hr_asset* a, const float4* src_dev, cudaStream_t st) {
-  if (!st) st = ctx_stream(ctx);
+namespace {
+
+template <typename Src>
+hr_status launch_strand_update(hr_ctx* ctx, hr_asset* a, const Src& src, cudaStream_t st) {
   const uint32_t S1 = a->S + 1;
   const uint32_t per_block = std::min<uint32_t>(256u, kUpdateMaxVerts / S1);
   const size_t smem = ((size_t)per_block * S1 + per_block) * sizeof(float4);
   const uint32_t blocks = (a->N + per_block - 1) / per_block;
-  k_strand_update<<<blocks, 256, smem, st>>>(src_dev, a->verts, a->shape, a->N, a->S, per_block,
-                                             a->prim_uv, a->prim_box, a->prim_wa);
+  k_strand_update<<<blocks, 256, smem, st>>>(src, a->verts, a->shape, a->N, a->S, per_block, a->prim_uv,
+                                             a->prim_box, a->prim_wa, a->d_bounds);
   HR_LAUNCHED(ctx);
-  return scene_bounds(ctx, a, (uint64_t)a->N * a->S, st);
+  return HR_OK;
+}
+
+}  // namespace
+
+// Strand segment records and scene bounds from the current vertices, into
+// the asset's existing arrays (the first N * S records).
+hr_status update_strands(hr_ctx* ctx, hr_asset* a, const float4* src_dev, cudaStream_t st) {
+  if (!st) st = ctx_stream(ctx);
+  k_init_bounds<<<1, 32, 0, st>>>(a->d_bounds);
+  HR_LAUNCHED(ctx);
+  return launch_strand_update(ctx, a, GivenVerts{src_dev}, st);
+}
+
+// Strands moved by the guides' new poses: vertices, records and bounds (the
+// thick hairs' bounds are cleared for their records).
+hr_status skin_strands(hr_ctx* ctx, hr_asset* a, const float4* gv) {
+  cudaStream_t st = ctx_stream(ctx);
+  k_init_all_bounds<<<1, 16, 0, st>>>(a->d_bounds);
+  HR_LAUNCHED(ctx);
+  return launch_strand_update(
+      ctx, a, SkinnedVerts{gv, a->w_strand, a->verts, a->cluster_of, a->cl_tri, a->S + 1}, st);
 }
 
 hr_status refresh_strand_prims(hr_ctx* ctx, hr_asset* a) {
@@ -1247,21 +1307,15 @@ hr_status build_hierarchy(hr_ctx* ctx, hr_asset* a, uint32_t C, uint32_t max_lev
   return hierarchy_finish(ctx, a, li, E, total, fit_begin, fit_end, st_fit);
 }
 
-hr_status rebuild_eth_records(hr_ctx* ctx, hr_asset* a) {
+hr_status moved_eth_records(hr_ctx* ctx, hr_asset* a) {
   cudaStream_t st = ctx_stream(ctx);
-  const uint32_t N = a->N, S = a->S, E = a->E;
+  const uint32_t S = a->S, E = a->E;
   if (E == 0) return HR_OK;
   LevelInfo li{};
   li.n_levels = a->n_levels;
   for (uint32_t k = 0; k <= a->n_levels && k < 16; ++k) li.off[k] = a->eth_offset[k];
-  float* eth_r = nullptr;
-  HR_TRY(scratch(ctx, 5, (size_t)E * sizeof(float), (void**)&eth_r));
-  k_eth_material<<<(unsigned)(((uint64_t)E * (HR_MAT_FLOATS + 1) + 127) / 128), 128, 0, st>>>(
-      a->verts, N, S, a->order, a->cl_first, li, E, a->mat, eth_r,
-      a->d_bounds + kEthBounds);
-  HR_LAUNCHED(ctx);
   k_eth_prims<<<(unsigned)(((uint64_t)E * S + 255) / 256), 256, 0, st>>>(
-      a->xsec, N, S, E, a->cl_first, li, eth_r, a->prim_uv, a->prim_box, a->prim_wa,
+      a->xsec, a->N, S, E, a->cl_first, li, nullptr, a->prim_uv, a->prim_box, a->prim_wa,
       a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   return HR_OK;

@@ -51,3 +51,30 @@ def test_guides_and_clusters_bit_exact(ctx, n, S, G, iters, copies):
             assert np.array_equal(cl, want.cluster_of)
     finally:
         hr.hr_asset_destroy(ctx, a)
+
+
+@pytest.mark.parametrize("n,S", [(300, 9), (24, 2100)])  # in one pass; strands too long for it
+def test_skinning_to_the_rest_pose_keeps_the_image(ctx, n, S):
+    v = scenegen.make_strands(n, S, seed=3, jitter=0.002, hang=0.08, radius=4e-3)
+    sc = scenegen.Scene(v, scenegen.material_from_melanin(np.full(n, 0.5), np.full(n, 0.2)),
+                        np.zeros((n, 2), np.float32))
+    cam = scenegen.frame_camera(*sc.aabb(), 48, 48, perspective=True, fill=0.7).pack()
+    lights = scenegen.point_lights(2, np.zeros(3), seed=1)
+    a = hr.hr_asset_create(ctx, v, sc.mat, sc.shape)
+    try:
+        hr.hr_build_guided_clusters(ctx, a, 5, 2)
+        guides = np.zeros(5, np.int32)
+        hr.hr_guides_export(ctx, a, guides)
+        d = hr.render_desc(cam, lights, 4, 3, 1, 0, hr.HR_FLAG_KEEP_HIERARCHY)
+        img = [np.zeros((48, 48, 3), np.float32) for _ in range(2)]
+        hr.hr_render_frame(ctx, a, 0, 0.5, 0, d, img[0])
+        hr.hr_asset_skin(ctx, a, np.ascontiguousarray(v[np.maximum(guides, 0)]))
+        back = np.zeros_like(v)
+        hr.hr_vertex_export(ctx, a, back)
+        assert np.allclose(back, v, atol=2e-6)
+        hr.hr_render_frame(ctx, a, 0, 0.5, 0, d, img[1])
+        # vertices moved by a few 1e-7 change few pixels at the fibres' edges
+        assert img[0].max() > 0
+        assert np.linalg.norm(img[1] - img[0]) <= 0.1 * np.linalg.norm(img[0])
+    finally:
+        hr.hr_asset_destroy(ctx, a)
