@@ -4,7 +4,7 @@
 //  * Camera: sample sid = pixel * spp + s; sub-pixel position from SplitMix64
 //    outputs 2 sid and 2 sid + 1 of the frame seed (top 24 bits each).
 //  * Traversal: stack-based over the binary LBVH whose nodes hold both
-//    children's boxes (one 64-byte node fetch tests two boxes); nearer child
+//    children's boxes (one 32-byte node fetch tests two boxes); nearer child
 //    first.  The search interval shrinks to the K-th nearest hit and to the
 //    nearest opaque (strand) hit: nothing behind an opaque hit can contribute.
 //  * Intersection: the record maps the ray into the cylinder's unit frame;
@@ -840,76 +840,99 @@ __device__ __forceinline__ bool leaf_span(const FrameArgs& fa, const uint32_t id
 // path (all crossings count) and stops early once T < 1e-7 in every channel,
 // where the light's contribution is below FP32 resolution of the pixel.
 constexpr float kDF = 0.7f;
-template <int PREC, bool COUNT>
-__device__ __forceinline__ void shadow_path(const FrameArgs& fa, const float3 x, const float3 wi,
-                                            const float tmax, const uint32_t self_mat, float T[3],
-                                            float& sg2, bool& ok, Counts& cn) {
-  T[0] = T[1] = T[2] = 1.f;
-  sg2 = 0.f;
-  if (fa.n_prims == 0) return;
+struct LightPath {
+  float T[3], sg2;
+  bool crossed;
+};
+
+// The path across primitive `id`; false once the light is used up.
+template <int PREC>
+__device__ __forceinline__ bool cross_leaf(const FrameArgs& fa, uint32_t id, const float3 x,
+                                           const float3 wi, const float tmax, const uint32_t self_mat,
+                                           LightPath& lp) {
+  float lo, hi;
+  float4 aux;
+  if (!leaf_span(fa, id, x, wi, 0.f, tmax, lo, hi) ||
+      __float_as_uint((aux = __ldg(fa.prim_wa + 2 * (size_t)id + 1)).x) == self_mat)
+    return true;
+  const float4 r2 = __ldg(fa.prim_wa + 2 * (size_t)id);
+  const float si = clampf(dot3(wi, f3(r2.x, r2.y, r2.z)) *
+                              rsqrtf(r2.x * r2.x + r2.y * r2.y + r2.z * r2.z),
+                          -1.f, 1.f);
+  Mat m;
+  load_mat(fa.mat + (size_t)__float_as_uint(aux.x) * HR_MAT_FLOATS, m);
+  float aF[3], s2;
+  forward_albedo<PREC>(fa.tables, m, fabsf(asinf(si)), (fa.flags & HR_FLAG_TRT) != 0, aF, s2);
+  if (aux.y > 0.f) {  // thick hair: its hair number over the chord
+    const float ntot = aux.y, r = aux.z, ab = aux.w;
+    const float rho = fminf(1.f, ntot * r * r / ab);
+    const float n = rho * (hi - lo) * sqrtf(ntot / (kPi * ab));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lp.T[c] *= exp2f(n * __log2f(aF[c]));
+    lp.sg2 = fmaf(n, s2, lp.sg2);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lp.T[c] *= aF[c];
+    lp.sg2 += s2;
+  }
+  lp.crossed = true;
+  return !(fmaxf(lp.T[0], fmaxf(lp.T[1], lp.T[2])) < 1e-7f);
+}
+
+// One node of a path: the next node, the other hit child on the stack.
+__device__ __forceinline__ int path_node(const FrameArgs& fa, const Slabs& sl, int node, const float tmax,
+                                         int* stack, int& sp, bool& ok) {
+  const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
+  float a0, a1;
+  const bool h0 = slab_test(sl, k0, tmax, a0), h1 = slab_test(sl, k1, tmax, a1);
+  const int c0 = (int)k0.w, c1 = (int)k1.w;
+  if (h0 && h1) {
+    if (sp < kStack)
+      stack[sp++] = c1;
+    else
+      ok = false;
+    return c0;
+  }
+  if (h0 || h1) return h0 ? c0 : c1;
+  return sp ? stack[--sp] : kDone;
+}
+
+// The light paths of a warp's lanes (lanes that are not live have none); with
+// WHOLE the whole warp calls it and leaves wait for one another as in walk_on,
+// without it each lane walks by itself.
+template <int PREC, bool COUNT, bool WHOLE>
+__device__ __forceinline__ void shadow_path(const FrameArgs& fa, bool live, const float3 x,
+                                            const float3 wi, const float tmax, const uint32_t self_mat,
+                                            float T[3], float& sg2, bool& ok, Counts& cn) {
+  LightPath lp{{1.f, 1.f, 1.f}, 0.f, false};
   const Slabs sl = ray_slabs(fa, x, wi);
   int stack[kStack];
   int sp = 0;
-  int node = fa.n_prims == 1 ? ~(int)__ldg(fa.leaf_id) : 0;
-  bool crossed = false;
+  int node = !live || fa.n_prims == 0 ? kDone : (fa.n_prims == 1 ? ~(int)__ldg(fa.leaf_id) : 0);
   for (;;) {
     if (node >= 0) {
-      const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
       if (COUNT) ++cn.nodes;
-      float a0, a1;
-      const bool h0 = slab_test(sl, k0, tmax, a0), h1 = slab_test(sl, k1, tmax, a1);
-      const int c0 = (int)k0.w, c1 = (int)k1.w;
-      if (h0 && h1) {
-        if (sp < kStack)
-          stack[sp++] = c1;
-        else
-          ok = false;
-        node = c0;
-        continue;
-      }
-      if (h0 || h1) {
-        node = h0 ? c0 : c1;
-        continue;
-      }
-    } else {
-      const uint32_t id = (uint32_t)(~node);
-      float lo, hi;
-      if (COUNT) ++cn.tests;
-      float4 aux;
-      if (leaf_span(fa, id, x, wi, 0.f, tmax, lo, hi) &&
-          __float_as_uint((aux = __ldg(fa.prim_wa + 2 * (size_t)id + 1)).x) != self_mat) {
-        const float4 r2 = __ldg(fa.prim_wa + 2 * (size_t)id);
-        const float si = clampf(dot3(wi, f3(r2.x, r2.y, r2.z)) *
-                                    rsqrtf(r2.x * r2.x + r2.y * r2.y + r2.z * r2.z),
-                                -1.f, 1.f);
-        Mat m;
-        load_mat(fa.mat + (size_t)__float_as_uint(aux.x) * HR_MAT_FLOATS, m);
-        float aF[3], s2;
-        forward_albedo<PREC>(fa.tables, m, fabsf(asinf(si)), (fa.flags & HR_FLAG_TRT) != 0, aF, s2);
-        if (aux.y > 0.f) {  // thick hair: its hair number over the chord
-          const float ntot = aux.y, r = aux.z, ab = aux.w;
-          const float rho = fminf(1.f, ntot * r * r / ab);
-          const float n = rho * (hi - lo) * sqrtf(ntot / (kPi * ab));
-#pragma unroll
-          for (int c = 0; c < 3; ++c) T[c] *= exp2f(n * __log2f(aF[c]));
-          sg2 = fmaf(n, s2, sg2);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) T[c] *= aF[c];
-          sg2 += s2;
-        }
-        crossed = true;
-        if (fmaxf(T[0], fmaxf(T[1], T[2])) < 1e-7f) break;
-      }
+      node = path_node(fa, sl, node, tmax, stack, sp, ok);
     }
-    if (sp == 0) break;
-    node = stack[--sp];
+    if (WHOLE) {
+      const unsigned inner = __ballot_sync(0xffffffffu, node >= 0);
+      const unsigned leaf = __ballot_sync(0xffffffffu, node < 0 && node != kDone);
+      if (!inner && !leaf) break;
+      if (inner && __popc(leaf) * 8 < kLeafWait * __popc(inner | leaf)) continue;
+    } else {
+      if (node == kDone) break;
+    }
+    if (node < 0 && node != kDone) {
+      if (COUNT) ++cn.tests;
+      node = !cross_leaf<PREC>(fa, (uint32_t)(~node), x, wi, tmax, self_mat, lp) || !sp ? kDone
+                                                                                       : stack[--sp];
+    }
   }
-  if (crossed) {
-    T[0] *= kDF;
-    T[1] *= kDF;
-    T[2] *= kDF;
-  }
+  const float dF = lp.crossed ? kDF : 1.f;
+  T[0] = lp.T[0] * dF;
+  T[1] = lp.T[1] * dF;
+  T[2] = lp.T[2] * dF;
+  sg2 = lp.sg2;
 }
 
 // Direction from x toward a light and its falloff E; the length of the light
@@ -984,8 +1007,8 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
     float Tl[3] = {1.f, 1.f, 1.f}, sg2 = 0.f;
     if (SHADOW) {
       bool sok = true;
-      shadow_path<PREC, COUNT>(fa, x, wi, path_length(L, E), __float_as_uint(aux.x), Tl, sg2, sok,
-                               cn);
+      shadow_path<PREC, COUNT, false>(fa, true, x, wi, path_length(L, E), __float_as_uint(aux.x), Tl, sg2,
+                                      sok, cn);
       if (!sok) atomicAdd(fa.overflow, 1u);
     }
     if (PATHS) {
