@@ -12,10 +12,11 @@
 // radix sort of (code, position in the active list), one thread per internal
 // node finds its key range and split from the longest common prefix (ties
 // between equal codes broken by index).  Bounds go bottom-up in two kernels:
-// k_gather_refit copies the leaf records into Morton order and finishes the
-// nodes whose leaf range lies inside its thread block's leaves (nearly all of
-// them) in barrier-separated rounds in shared memory; k_climb finishes the few
-// nodes that span blocks by float atomic min / max from each climb start.
+// k_gather_refit gathers the leaf boxes in Morton order and finishes the nodes
+// whose leaf range lies inside its thread block's leaves (nearly all of them)
+// in barrier-separated rounds in shared memory; k_climb finishes the few nodes
+// that span blocks by atomic minima of the quantised planes from each climb
+// start, and k_span_records packs those nodes.
 //
 // Node layout (2 x uint4 = 32 bytes, one sector), children's boxes stored in
 // the parent: per child the x, y and z intervals and the child index.  An
@@ -189,17 +190,17 @@ __device__ __forceinline__ int4 karras_node(const uint32_t* __restrict__ keys, i
   int c0, c1;
   if (lo == gamma) {
     c0 = ~gamma;
-    parent_leaf[gamma] = i;
+    parent_leaf[gamma] = 2 * i;
   } else {
     c0 = gamma;
-    parent_int[gamma] = i;
+    parent_int[gamma] = 2 * i;
   }
   if (hi == gamma + 1) {
     c1 = ~(gamma + 1);
-    parent_leaf[gamma + 1] = i;
+    parent_leaf[gamma + 1] = 2 * i + 1;
   } else {
     c1 = gamma + 1;
-    parent_int[gamma + 1] = i;
+    parent_int[gamma + 1] = 2 * i + 1;
   }
   return make_int4(c0, c1, lo, hi);
 }
@@ -358,7 +359,7 @@ __global__ void __launch_bounds__(B) k_gather_refit(
   float4 bl = make_float4(0.f, 0.f, 0.f, 0.f), bh = bl;
   if (leaf < n) {
     const uint32_t id = sorted_ids[leaf];
-    lparent = parent_leaf[leaf];
+    lparent = parent_leaf[leaf] >> 1;
     leaf_id[leaf] = id;
     s_id[j] = id;
     bl = box[2 * (size_t)id];
@@ -407,7 +408,7 @@ __global__ void __launch_bounds__(B) k_gather_refit(
     start_leaf = !(lparent >= b0 && lparent < b0 + B && s_child[lparent - b0].z >= b0 &&
                    s_child[lparent - b0].w < b0 + B);
   if (node_local && node != 0) {
-    const int p = __ldg(parent_int + node);
+    const int p = __ldg(parent_int + node) >> 1;
     start_node = !(p >= b0 && p < b0 + B && s_child[p - b0].z >= b0 && s_child[p - b0].w < b0 + B);
   }
   append_start(start_leaf, ~leaf, counts, starts);
@@ -422,15 +423,15 @@ __global__ void __launch_bounds__(B) k_gather_refit(
 // at least as wide from another start below it, which carries it on up.  No
 // ordering between starts is needed.
 __global__ void k_climb(const unsigned* __restrict__ counts, const int* __restrict__ starts,
-                        const int4* __restrict__ child, const int* __restrict__ parent_int,
-                        const int* __restrict__ parent_leaf, const float4* __restrict__ box,
-                        const float4* __restrict__ frame, const uint32_t* __restrict__ leaf_id,
-                        const uint4* __restrict__ nodes, uint32_t* span) {
+                        const int* __restrict__ parent_int, const int* __restrict__ parent_leaf,
+                        const float4* __restrict__ box, const float4* __restrict__ frame,
+                        const uint32_t* __restrict__ leaf_id, const uint4* __restrict__ nodes,
+                        uint32_t* span) {
   const unsigned m = *counts;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    int cur = __ldg(starts + i);
+    const int cur = __ldg(starts + i);
     QBox u;
-    int p;
+    int p;  // 2 * node + side; negative above the root
     if (cur < 0) {
       const size_t id = __ldg(leaf_id + ~cur);
       u = q_box(__ldg(box + 2 * id), __ldg(box + 2 * id + 1), __ldg(frame), __ldg(frame + 2));
@@ -441,17 +442,21 @@ __global__ void k_climb(const unsigned* __restrict__ counts, const int* __restri
     }
     const uint32_t b[6] = {u.x & 0xffffu, u.x >> 16, u.y & 0xffffu, u.y >> 16, u.z & 0xffffu, u.z >> 16};
     unsigned live = 0x3fu;
+    // A start is a chain of levels, its time their latency: the links of the
+    // level above are read while this level's atomics are out, and a node's
+    // side comes with its link (a thumbnail of 3,001 strands 261 -> 248 us a call)
+    uint32_t slot = __ldg(&nodes[2 * (size_t)(p >> 1)].x);
     while (p >= 0) {
-      const int first = __ldg(&child[p].x);
-      const int up = p == 0 ? -1 : __ldg(parent_int + p);
-      uint32_t* r = span + 12 * (size_t)__ldg(&nodes[2 * (size_t)p].x) + (first == cur ? 0 : 6);
+      uint32_t* r = span + 12 * (size_t)slot + 6 * (p & 1);
+      uint32_t old[6];
+#pragma unroll
+      for (int q = 0; q < 6; ++q) old[q] = (live >> q) & 1u ? atomicMin(r + q, b[q]) : 0u;
+      p = p >> 1 ? __ldg(parent_int + (p >> 1)) : -1;
+      if (p >= 0) slot = __ldg(&nodes[2 * (size_t)(p >> 1)].x);
 #pragma unroll
       for (int q = 0; q < 6; ++q)
-        if ((live >> q) & 1u)
-          if (atomicMin(r + q, b[q]) <= b[q]) live &= ~(1u << q);
+        if (old[q] <= b[q]) live &= ~(1u << q);
       if (!live) break;
-      cur = p;
-      p = up;
     }
   }
 }
@@ -605,7 +610,7 @@ hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, c
     climb_grid = sms * per;
   }
   const unsigned grid = (unsigned)std::min<size_t>((size_t)climb_grid, ((size_t)n * 2 + 255) / 256);
-  k_climb<<<grid, 256, 0, st>>>(counts, starts, bv.child, bv.par_int, bv.par_leaf, a->prim_box,
+  k_climb<<<grid, 256, 0, st>>>(counts, starts, bv.par_int, bv.par_leaf, a->prim_box,
                                 bv.frame, bv.leaf_id, bv.nodes, span);
   HR_LAUNCHED(ctx);
   k_span_records<<<grid, 256, 0, st>>>(counts, span_node, span, bv.nodes);

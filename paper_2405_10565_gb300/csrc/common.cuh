@@ -43,8 +43,8 @@ struct Bvh {
   // topology kept for refits: children + leaf range, parents; the LoD and
   // hierarchy shape it was built for
   int4* child = nullptr;       // [cap]
-  int* par_int = nullptr;      // [cap]
-  int* par_leaf = nullptr;     // [cap]
+  int* par_int = nullptr;      // [cap] parent of each node, and of each leaf,
+  int* par_leaf = nullptr;     // [cap] as 2 * parent + which child it is
   uint8_t* lod_built = nullptr;  // [lod_cap] copy of the LoD of the build (none: all strands)
   uint32_t lod_cap = 0, built_C = 0, built_E = 0, built_total = 0;
   int built_with_lod = 0;
