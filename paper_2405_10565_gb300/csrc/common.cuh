@@ -430,8 +430,6 @@ struct ServeItem {
   uint32_t wt0;     // first warp tile (of the request's grid) in this item
   uint32_t nwt;     // warp tiles in this item
 };
-// Projected scene rectangle of a frame into rect_dev (one warp; device).
-hr_status launch_scene_rect(hr_ctx* ctx, const FrameArgs& fa, float4* rect_dev, cudaStream_t st);
 // items_dev[i] covers batch tiles [item_start_dev[i], item_start_dev[i+1]);
 // every item of one launch has the same k-buffer bound and precision.
 hr_status launch_serve_batch(hr_ctx* ctx, int kmax, int precision, const ServeItem* items_dev,

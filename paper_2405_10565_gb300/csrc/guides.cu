@@ -207,8 +207,8 @@ __global__ void k_key_starts(const uint32_t* __restrict__ key, uint32_t n, uint3
 // Centroid of every cluster: the members' vertices summed in ascending strand
 // id (FP32), divided by the count; an empty cluster keeps its centroid.  One
 // thread per coordinate: the sum is a chain, so its latency is hidden by 16
-// members' loads in flight (one at a time took 235 us for 100k strands in 256
-// clusters, the longest cluster's chain) and the coordinates of a cluster are
+// members' loads in flight (84 us for 100k strands in 256 clusters, the longest
+// cluster's chain; one load at a time took 235) and the coordinates of a cluster are
 // spread over several blocks.
 constexpr uint32_t kUpdateBlock = 64;
 __global__ void __launch_bounds__(kUpdateBlock)
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kUpdateBlock)
 // non-negative, so the FP32 sum is within a relative gamma_(m + S1 + 5) of it.
 // Only members whose lower bound does not exceed the least upper bound can be
 // the medoid; the FP32 sums are formed for these alone (a few per cluster,
-// where all m^2 pairs took 16.9 ms for 100k strands in 256 clusters).  Where
+// where all m^2 pairs took 16.9 ms for 100k strands in 256 clusters; 0.2 now).  Where
 // the bounds are not finite every member stays a candidate.
 
 struct MedoidWork {
@@ -643,8 +643,8 @@ struct Offs {
 // guides there once in FP64 (1 / 64 of the FP32 rate) and takes every point at
 // k through it in double-word FP32, whose weights differ from FP64 ones by
 // less than their final FP32 rounding.  Neighbouring threads read and write
-// neighbouring vertices.  FP64 prisms per point took 1.51 ms for 100k strands
-// x 65 and 0.81 ms for 22k thick hairs.
+// neighbouring vertices.  255 us for 100k strands x 65 and 22k thick hairs;
+// FP64 prisms per point took 1.51 and 0.81 ms.
 constexpr uint32_t kWeightBlock = 256;
 __global__ void __launch_bounds__(kWeightBlock)
     k_prism_weights(const float4* __restrict__ verts, uint32_t S1,

@@ -13,8 +13,6 @@
 namespace hr {
 namespace {
 
-__global__ void k_serve_rect(const FrameArgs fa, float4* rect) { tr::scene_rect_warp(fa, rect); }
-
 template <int KMAX, int PREC>
 // 4 blocks per SM (at most 128 registers), as for the frame kernel.
 __global__ void __launch_bounds__(kBlock, tr::kTraceBlocks)
@@ -76,12 +74,6 @@ int serve_grid(int kmax, int precision) {
     blocks = 4;
   }
   return sms * std::max(1, blocks);
-}
-
-hr_status launch_scene_rect(hr_ctx* ctx, const FrameArgs& fa, float4* rect_dev, cudaStream_t st) {
-  k_serve_rect<<<1, 32, 0, st>>>(fa, rect_dev);
-  HR_LAUNCHED(ctx);
-  return HR_OK;
 }
 
 hr_status launch_serve_batch(hr_ctx* ctx, int kmax, int precision, const ServeItem* items_dev,
