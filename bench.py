@@ -302,7 +302,7 @@ def frame_tail(hr, ctx, asset, desc, img, capacity: int = 1 << 20):
     dur = (t1 - t0) / 1e3
     span = (t1.max() - t0.min()) / 1e3
     slow = int(np.argmax(dur))
-    warps = len(np.unique(rec["sm"])) * 16  # 4 blocks of 4 warps per SM
+    warps = len(np.unique(rec["sm"])) * 28  # 7 blocks of 4 warps per SM
     visits = int(rec["max_node_visits"][slow])
     return {"tiles": n, "recorded": int(rec.size), "span_us": span,
             "tile_us": {"median": float(np.median(dur)), "p99": float(np.percentile(dur, 99)),
@@ -581,7 +581,7 @@ def main():
     tile_schedule = {"heavy_tiles": int(fp32_st[-1].heavy_tiles), "frame_ms_warm": fp32_ms,
                      "frame_ms_fixed_order_warm": fixed_ms,
                      "note": "warm frames alone: the previous frame's heaviest warp tiles traced "
-                             "first, four rays per warp, against the fixed tile order; the images "
+                             "first, against the fixed tile order; the images "
                              "are identical"}
     # the same frame with dual-scattering light paths (a shadow ray per hit and
     # light, HR_FLAG_SHADOWS), outside the timed region

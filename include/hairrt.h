@@ -161,14 +161,13 @@ typedef struct hr_light {
 /* The frame kernel normally carries a schedule from one frame of an asset to
  * the next (no counterpart in the paper): the warp tiles whose slowest lane
  * took the most traversal steps in the previous frame (at most 16, at least
- * half the steps of that frame's slowest) are traced first, four rays per
- * warp, so that the frame is not held up by 32 long rays sharing one warp.
- * Their pixels are composited with the same summation order, so the image
- * does not depend on the schedule.  The schedule lives in the asset and is
+ * half the steps of that frame's slowest) are traced first, so that the frame
+ * is not held up by long rays that start late.  The image does not depend on
+ * the schedule.  The schedule lives in the asset and is
  * dropped when the image size or spp changes.  A frame right after an
  * overlapped hr_asset_update (the call before it) uses the fixed order and
  * leaves the schedule as it is, and so does HR_FLAG_FIXED_TILE_ORDER, which
- * traces every tile whole, in raster order.  Counting renders (HR_FLAG_COUNT,
+ * hands out the tiles in raster order.  Counting renders (HR_FLAG_COUNT,
  * hr_render_profile) and frames with HR_FLAG_SHADOWS always use the fixed
  * order. */
 #define HR_FLAG_FIXED_TILE_ORDER 8192u
@@ -211,8 +210,8 @@ typedef struct hr_stats {
                                search cut or another hit, or a wide FP32 bound) */
   uint64_t refined_entries; /* kept FP32 hits decided precisely afterwards (their
                                order against a precise hit was open) */
-  uint32_t heavy_tiles;     /* warp tiles traced a few rays per warp from the previous
-                               frame's schedule (see HR_FLAG_FIXED_TILE_ORDER) */
+  uint32_t heavy_tiles;     /* warp tiles traced first by the previous frame's
+                               schedule (see HR_FLAG_FIXED_TILE_ORDER) */
   uint32_t reserved;
 } hr_stats;
 
