@@ -361,7 +361,7 @@ struct FrameArgs {
   uint32_t tile_cap;         // records tile_log holds
   uint32_t* tile_count;      // the frame's number of warp tiles (written when tile_log is set)
   TileSched* sched;          // plain frame kernel: the heavy-tile schedule, or null
-  uint32_t frame_warps;      // with sched: resident warps of the frame kernel
+  uint32_t frame_warps;      // resident warps of the frame kernel (0: hand out whole tiles)
   LongWork lw;               // plain frame kernel: rays put aside
 };
 
@@ -387,9 +387,11 @@ hr_status launch_frame(hr_ctx* ctx, const FrameArgs& fa, int precision, bool cou
 hr_status launch_frame_shadow(hr_ctx* ctx, const FrameArgs& fa, int precision, bool count,
                        float* rgb_dev, cudaStream_t st);
 // Tiles of a frame with shadow rays by separate hit, light-path and shading
-// kernels; *left: tiles from *work on may be left for the one-kernel form.
+// kernels; *left: tiles may be left for the one-kernel form, *begun: whole
+// tiles, from *work on.
 hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, const float4* rect,
-                               uint32_t* work, float* rgb, cudaStream_t st, bool* left);
+                               uint32_t* work, float* rgb, cudaStream_t st, bool* left,
+                               bool* begun);
 hr_status launch_samples(hr_ctx* ctx, const FrameArgs& fa, int precision, const uint32_t* sids,
                          uint32_t m, float* rad_dev, int32_t* hit_dev, cudaStream_t st);
 // IM(theta, beta) lookups at m device points (test export of the shading code)

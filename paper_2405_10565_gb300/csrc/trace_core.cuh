@@ -1094,7 +1094,7 @@ struct LongTile {
   uint32_t xy;         // origin, x | y << 16
   uint32_t lanes;      // lanes whose rays were put aside
   uint32_t left;       // of those, not finished yet
-  uint32_t pad;
+  uint32_t part;       // lanes whose pixels it stores (small frames: a part of the tile)
   float acc[3][32];    // the lanes' radiance
   uint32_t at[32];     // where a put-aside lane's record starts
 };
@@ -1108,7 +1108,7 @@ constexpr uint32_t kLongHead = 4;
 template <int KMAX>
 __device__ __forceinline__ bool put_aside(const FrameArgs& fa, const RayMem<KMAX, kBlock>& rm,
                                           const Walk& w, const int* stack, uint32_t x0, uint32_t y0,
-                                          unsigned mask, uint32_t& tile) {
+                                          unsigned mask, bool inside, uint32_t& tile) {
   const uint32_t lane = threadIdx.x & 31, c = threadIdx.x, k = fa.k;
   const bool mine = (mask >> lane) & 1u;
   const uint32_t words = mine ? kLongHead + 3 * k + (uint32_t)w.sp + 1 : 0u;
@@ -1143,10 +1143,12 @@ __device__ __forceinline__ bool put_aside(const FrameArgs& fa, const RayMem<KMAX
   tile = __shfl_sync(0xffffffffu, tile, 0);
   first = __shfl_sync(0xffffffffu, first, 0);
   at += incl - words;
+  const unsigned part = __ballot_sync(0xffffffffu, inside);
   if (lane == 0) {
     fa.lw.tiles[tile].xy = x0 | y0 << 16;
     fa.lw.tiles[tile].lanes = mask;
     fa.lw.tiles[tile].left = rays;
+    fa.lw.tiles[tile].part = part;
   }
   if (mine) {
     fa.lw.tiles[tile].at[lane] = at;
@@ -1261,16 +1263,18 @@ __device__ __forceinline__ void tile_write(const FrameArgs& fa, const TileLane t
   }
 }
 
-// Traces, shades and stores a tile.  With LONG, rays over the budget of steps
+// Traces, shades and stores the part of a tile (whole pixels).  With LONG, rays over the budget of steps
 // are put aside (at most one sample a lane: no more than 32 spp) and
 // the tile is stored by the last of them.
 template <int KMAX, int PREC, bool COUNT, bool SHADOW = false, bool LONG = false>
 __device__ __forceinline__ void render_warp_tile(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm,
                                                  uint32_t x0, uint32_t y0, uint32_t wtw,
                                                  const float4 rect, int budget,
-                                                 float* __restrict__ rgb, Counts& cn, bool& overflow) {
+                                                 float* __restrict__ rgb, Counts& cn, bool& overflow,
+                                                 const unsigned part = 0xffffffffu) {
   const uint32_t G = fa.grp, c = threadIdx.x, lane = c & 31;
-  const TileLane tl = tile_lane(fa, x0, y0, wtw, rect);
+  TileLane tl = tile_lane(fa, x0, y0, wtw, rect);
+  tl.inside = tl.inside && ((part >> lane) & 1u);
   if (!__any_sync(0xffffffffu, tl.inside)) return;
   float acc[3] = {0.f, 0.f, 0.f};
   for (uint32_t s0 = 0; s0 < fa.spp; s0 += G) {
@@ -1287,7 +1291,7 @@ __device__ __forceinline__ void render_warp_tile(const FrameArgs& fa, RayMem<KMA
       if (LONG) {
         cn.steps += (uint32_t)(steps - left);
         aside = __ballot_sync(0xffffffffu, w.node != kDone);
-        if (aside && !put_aside<KMAX>(fa, rm, w, stack, x0, y0, aside, tile)) continue;
+        if (aside && !put_aside<KMAX>(fa, rm, w, stack, x0, y0, aside, tl.inside, tile)) continue;
       }
       break;
     }

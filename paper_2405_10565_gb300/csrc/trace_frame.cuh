@@ -115,9 +115,24 @@ __global__ void __launch_bounds__(kRectThreads) k_scene_rect(const FrameArgs fa,
 // 1.59, 1.39; a thumbnail (0.09) 0.29, 0.32, 0.38, 0.38, 0.40; the 4K frame of
 // straight hair (39; 100, 10,600) 11.0, 11.1, 10.0, 9.9, 14.5; the close view
 // (55; 44, 1,200) 6.2, 4.4, 3.91, 3.85, 3.83.
+// Below a tile per warp, where parts of tiles are handed out, 40, 64 and 96
+// steps: 262, 271, 277 us at 0.09 tiles per warp, 379, 360, 361 at 0.19,
+// 760, 739, 728 and 301, 292, 304 at half a tile, 341, 327, 335 at 0.9.
 __device__ __forceinline__ int step_budget(uint32_t tiles, uint32_t warps) {
   const float per = (float)tiles / (float)warps;
-  return (int)fminf(fmaxf(64.f * per * per, 40.f), 1024.f);
+  return (int)fminf(fmaxf(64.f * per * per, per < 0.125f ? 40.f : 64.f), 1024.f);
+}
+
+// Small frames hand out parts of a tile, 2^n of them of whole pixels, as far as
+// there are warps for them: a warp's lanes go through nodes and leaves
+// together, so the fewer rays share a warp, the sooner its last one is done
+// (a 94 x 70 frame of 2,812 strands 387 us a call whole, 379 in parts and 360
+// with the budget that this allows; with shadow rays, 203 strands at 78 x 48,
+// 132 and 86).
+__device__ __forceinline__ uint32_t tile_split(uint32_t tiles, uint32_t warps, uint32_t grp) {
+  uint32_t ls = 0;
+  while ((grp << (ls + 1)) <= 32u && ((uint64_t)tiles << (ls + 1)) <= warps) ++ls;
+  return ls;
 }
 
 // Persistent frame kernel.  The image has been cleared to background; the
@@ -144,18 +159,21 @@ __global__ void __launch_bounds__(kBlock, SHADOW ? 1 : tr::kTraceBlocks)
   const uint32_t thresh = sc ? sc->thresh : 0u;
   uint32_t wmax = 0;  // the warp's largest tile step count
   const int budget = LONG && fa.lw.words ? step_budget(g.n, fa.frame_warps) : 0x7fffffff;
+  const uint32_t ls = COUNT ? 0u : tile_split(g.n, fa.frame_warps, fa.grp);
   for (;;) {
     uint32_t t = 0;
     if (lane == 0) t = atomicAdd(work, 1u);
     t = __shfl_sync(0xffffffffu, t, 0);
     uint32_t x0, y0;
+    const unsigned part = (0xffffffffu >> (32u - (32u >> ls))) << ((t & ((1u << ls) - 1u)) * (32u >> ls));
+    t >>= ls;
     if (t < nh) {  // a tile of the previous frame's grid; one that is not of this grid is skipped
       const uint32_t xy = sc->heavy[t];
       x0 = xy & 0xffffu, y0 = xy >> 16;
       const uint32_t gx = (x0 - g.x0) / g.wtw, gy = (y0 - g.y0) / g.wth;
       if (x0 < g.x0 || y0 < g.y0 || (x0 - g.x0) % g.wtw || (y0 - g.y0) % g.wth || gx >= g.nx ||
-          gy * g.nx + gx >= g.n)
-        continue;
+          gy * g.nx + gx >= g.n || __any_sync(0xffffffffu, lane < t && sc->heavy[lane] == xy))
+        continue;  // (or, from two of its parts, listed twice)
       t = gy * g.nx + gx;
     } else {
       t -= nh;
@@ -172,7 +190,7 @@ __global__ void __launch_bounds__(kBlock, SHADOW ? 1 : tr::kTraceBlocks)
       tests0 = cn.tests;
     }
     tr::render_warp_tile<KMAX, PREC, COUNT, SHADOW, LONG>(fa, rm, x0, y0, g.wtw, rect, budget,
-                                                          rgb, cn, overflow);
+                                                          rgb, cn, overflow, part);
     if (sc) {
       // the tile's slowest-lane steps: the warp's maximum, and a candidate for
       // the next frame's heavy tiles at or above the threshold
@@ -338,7 +356,8 @@ __global__ void __launch_bounds__(kBlock, 6)
     if (left != 1u) continue;
     __threadfence();
     // the tile's last ray: shade the lanes put aside and store the tile
-    const tr::TileLane tl = tr::tile_lane(fa, x0, y0, g.wtw, rect);
+    tr::TileLane tl = tr::tile_lane(fa, x0, y0, g.wtw, rect);
+    tl.inside = (lt.part >> lane) & 1u;
     float acc[3] = {__ldcg(&lt.acc[0][lane]), __ldcg(&lt.acc[1][lane]), __ldcg(&lt.acc[2][lane])};
     if ((lt.lanes >> lane) & 1u) {
       const uint32_t* rec = fa.lw.pool + lt.at[lane];
@@ -420,11 +439,13 @@ hr_status launch_k(hr_ctx* ctx, const FrameArgs& fa, bool count, float* rgb, cud
     k_frame<KMAX, PREC, true, SHADOW><<<g, kBlock, 0, st>>>(f, rect, work, rgb);
   } else {
     if (SHADOW) {  // the one-kernel form takes what the rounds leave over
-      bool left = true;
-      HR_TRY(launch_shadow_rounds(ctx, f, PREC, rect, work, rgb, st, &left));
+      bool left = true, begun = false;
+      HR_TRY(launch_shadow_rounds(ctx, f, PREC, rect, work, rgb, st, &left, &begun));
       if (!left) return HR_OK;
+      if (begun) f.frame_warps = 0;  // *work counts whole tiles: no parts
     }
-    const int g = (int)std::min<uint32_t>(tiles, frame_grid<KMAX, PREC, false, SHADOW>());
+    // up to 32 parts a tile, four warps a block
+    const int g = (int)std::min<uint64_t>(8ull * tiles, (uint64_t)frame_grid<KMAX, PREC, false, SHADOW>());
     k_frame<KMAX, PREC, false, SHADOW><<<g, kBlock, 0, st>>>(f, rect, work, rgb);
   }
   HR_LAUNCHED(ctx);

@@ -225,13 +225,14 @@ hr_status launch_rounds_k(hr_ctx* ctx, const FrameArgs& fa, const float4* rect, 
 }  // namespace
 
 // The tiles that the rounds take; *left says whether tiles can be left over
-// (from *work on, for the one-kernel form).  Nothing is launched (and *left is
+// (for the one-kernel form: from *work on, where rounds have *begun).  Nothing is launched (and *left is
 // set) where the buffers do not fit the context's budget or a lane traces
 // more than one sample of a pixel (more than 32 spp: its hits would need
 // an order of their own).
 hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, const float4* rect,
-                               uint32_t* work, float* rgb, cudaStream_t st, bool* left) {
+                               uint32_t* work, float* rgb, cudaStream_t st, bool* left, bool* begun) {
   *left = true;
+  *begun = false;
   if (fa.spp > fa.grp) return HR_OK;
   const uint64_t L = (uint64_t)fa.lights.n;
   const uint64_t worst = (uint64_t)fa.cam.W * fa.cam.H * fa.spp * fa.k;
@@ -256,6 +257,7 @@ hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, 
   sw.cap = (uint32_t)cap;
   const uint32_t rounds = (uint32_t)std::min<uint64_t>((worst + stop - 1) / stop, kMaxRounds);
   *left = (uint64_t)rounds * stop < worst;
+  *begun = true;
   return precision == HR_PREC_FP16
              ? launch_rounds_k<HR_PREC_FP16>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st)
              : launch_rounds_k<HR_PREC_FP32>(ctx, fa, rect, work, sw, rounds, g_hits, rgb, st);

@@ -108,3 +108,28 @@ def test_long_walks_finish_as_short_ones(ctx, res, spp, k, setting):
         assert np.allclose(img[2], img[0], rtol=1e-4, atol=1e-6)
     finally:
         hr.hr_asset_destroy(ctx, a)
+
+
+@pytest.mark.parametrize("res,spp,k", [(3, 1, 4), (16, 1, 1), (24, 2, 2), (33, 5, 8), (64, 8, 4), (20, 32, 3)])
+def test_parts_of_tiles_equal_whole_tiles(res, spp, k):
+    """Small frames hand out parts of a tile, with rays put aside from them;
+    counting renders trace whole tiles."""
+    from paper_2405_10565_gb300.build import build
+    build()
+    w = scenegen.clustered(n=1500, S=8, res=res, spp=spp, n_clusters=40)
+    ctx = hr.hr_create(0)
+    try:
+        a = hr.hr_asset_create(ctx, w.scene.verts, w.scene.mat, w.scene.shape)
+        hr.hr_build_clusters(ctx, a, w.n_clusters)
+        C, n_levels, _ = hr.hr_hierarchy_info(ctx, a)
+        hr.hr_build_bvh(ctx, a, scenegen.lod_preset("half", C, n_levels))
+        img = [np.zeros((res, res, 3), np.float32) for _ in range(4)]
+        for i, flags in enumerate((hr.HR_FLAG_COUNT, hr.HR_FLAG_FIXED_TILE_ORDER, 0, 0)):
+            d = hr.render_desc(w.camera.pack(), w.lights, spp, k, 7, 0, flags)
+            hr.hr_render(ctx, a, d, img[i], stats=True)
+        assert img[0].max() > 0
+        # the same operations in the same order; the compiler may contract them differently
+        assert np.allclose(img[1], img[0], rtol=1e-5, atol=1e-7), np.abs(img[1] - img[0]).max()
+        assert np.array_equal(img[1], img[2]) and np.array_equal(img[1], img[3])
+    finally:
+        hr.hr_destroy(ctx)
