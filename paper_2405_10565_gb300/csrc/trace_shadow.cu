@@ -26,6 +26,16 @@ namespace {
 
 constexpr uint64_t kPathBudget = 1ull << 24;  // 256 MB of path records
 constexpr uint32_t kMaxRounds = 3;
+// A round costs about 25 us more than the one-kernel form where little is
+// walked (four launches in a row for one); that form walks a hit's paths one
+// after the other, so its time goes with the lights and with the depth of the
+// scene.  Rounds / one kernel, us a call at 400 x 300, 2 spp, 1, 2, 4, 8 lights:
+// 2.8k segments 109 / 80, 112 / 97, 116 / 142, 120 / 199; 9k segments 197 / 148,
+// 197 / 183, 205 / 284, 219 / 479; 44k segments of curls 465 / 357, 509 / 571;
+// 96k straight ones 1739 / 3687; 256k 685 / 1134.  So the smallest scenes by
+// the number of lights are left to the one kernel, up to the 1M samples measured.
+constexpr uint32_t kOneKernelPrims = 49152;  // over the cube of the lights
+constexpr uint64_t kOneKernelSamples = 1ull << 20;
 
 struct ShadowTile {
   uint32_t tile;      // index in the frame's warp grid
@@ -226,7 +236,8 @@ hr_status launch_rounds_k(hr_ctx* ctx, const FrameArgs& fa, const float4* rect, 
 
 // The tiles that the rounds take; *left says whether tiles can be left over
 // (for the one-kernel form: from *work on, where rounds have *begun).  Nothing is launched (and *left is
-// set) where the buffers do not fit the context's budget or a lane traces
+// set) for the smallest scenes, where the buffers do not fit the context's
+// budget, or where a lane traces
 // more than one sample of a pixel (more than 32 spp: its hits would need
 // an order of their own).
 hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, const float4* rect,
@@ -235,6 +246,9 @@ hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, 
   *begun = false;
   if (fa.spp > fa.grp) return HR_OK;
   const uint64_t L = (uint64_t)fa.lights.n;
+  if (L * L * L * fa.n_prims <= kOneKernelPrims &&
+      (uint64_t)fa.cam.W * fa.cam.H * fa.spp <= kOneKernelSamples)
+    return HR_OK;
   const uint64_t worst = (uint64_t)fa.cam.W * fa.cam.H * fa.spp * fa.k;
   const uint64_t stop = std::min<uint64_t>(worst, kPathBudget / L);
   // every launched warp can be at a tile of 32 lanes and k hits when the round
