@@ -14,7 +14,7 @@ namespace hr {
 namespace {
 
 template <int KMAX, int PREC>
-// 4 blocks per SM (at most 128 registers), as for the frame kernel.
+// kTraceBlocks blocks per SM (72 registers), as for the frame kernel.
 __global__ void __launch_bounds__(kBlock, tr::kTraceBlocks)
     k_serve(const ServeItem* __restrict__ items, const uint32_t* __restrict__ item_start,
             uint32_t n_items, uint32_t total, uint32_t* work) {

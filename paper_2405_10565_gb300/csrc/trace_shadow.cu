@@ -235,11 +235,10 @@ hr_status launch_rounds_k(hr_ctx* ctx, const FrameArgs& fa, const float4* rect, 
 }  // namespace
 
 // The tiles that the rounds take; *left says whether tiles can be left over
-// (for the one-kernel form: from *work on, where rounds have *begun).  Nothing is launched (and *left is
-// set) for the smallest scenes, where the buffers do not fit the context's
-// budget, or where a lane traces
-// more than one sample of a pixel (more than 32 spp: its hits would need
-// an order of their own).
+// (for the one-kernel form: from *work on, where rounds have *begun).  Nothing
+// is launched (and *left is set) for the smallest scenes, where the buffers do
+// not fit the context's budget, or where a lane traces more than one sample of
+// a pixel (more than 32 spp: its hits would need an order of their own).
 hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, const float4* rect,
                                uint32_t* work, float* rgb, cudaStream_t st, bool* left, bool* begun) {
   *left = true;
