@@ -379,6 +379,7 @@ hr_status hr_asset_update(hr_ctx* ctx, hr_asset* a, const float* vertices) {
   API_ENTER(ctx);
   if (!a || !vertices) return set_error(ctx, HR_EINVAL, "hr_asset_update: null argument");
   if (ctx->server) serve_forget_asset(ctx, ctx->server, a);
+  a->radii_old = true;  // a strand's radius comes with its vertices
   cudaStream_t st = ctx->stream;
   // a device-readable source (device memory, page-locked host memory) is read
   // once by the kernel that rebuilds the records, so the transfer overlaps

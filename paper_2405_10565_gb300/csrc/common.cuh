@@ -101,6 +101,7 @@ struct hr_asset {
   float4* w_strand = nullptr;     // [N * (S + 1)] prism weights of the strand vertices
   float4* w_eth = nullptr;        // [E * (S + 1) * 5] of thick-hair centres and corners
   uint32_t guided_C = 0, guided_E = 0;  // shape the weights were taken for
+  bool radii_old = false;  // vertices (and radii) were given since the thick hairs took their radii
   // frame-kernel schedule carried between frames (TileSched)
   hr::TileSched* sched = nullptr;
 };
@@ -219,8 +220,9 @@ hr_status build_hierarchy_from(hr_ctx* ctx, hr_asset* a, uint32_t C, uint32_t ma
                                const uint32_t* order_dev, const uint32_t* cl_first_dev);
 
 // The strands moved by the guides' new poses gv: vertices, records and bounds;
-// and the thick hairs' segment records from their moved cross-sections (their
-// materials and radii stay), after skin_strands on the same stream.
+// and the thick hairs' segment records from their moved cross-sections, after
+// skin_strands on the same stream (their radii are taken again where
+// hr_asset_update has given vertices since they were; their materials stay).
 hr_status skin_strands(hr_ctx* ctx, hr_asset* a, const float4* gv);
 hr_status moved_eth_records(hr_ctx* ctx, hr_asset* a);
 

@@ -1252,6 +1252,7 @@ hr_status hierarchy_finish(hr_ctx* ctx, hr_asset* a, const LevelInfo& li, uint64
                                                              a->mat, eth_r,
       a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
+  a->radii_old = false;
   const uint64_t ne = E * S;
   k_eth_prims<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(a->xsec, N, S, (uint32_t)E,
                                                            a->cl_first, li, eth_r, a->prim_uv,
@@ -1314,8 +1315,18 @@ hr_status moved_eth_records(hr_ctx* ctx, hr_asset* a) {
   LevelInfo li{};
   li.n_levels = a->n_levels;
   for (uint32_t k = 0; k <= a->n_levels && k < 16; ++k) li.off[k] = a->eth_offset[k];
+  // Skinning keeps every radius, so the records' own stand, unless vertices
+  // with other radii were given (57 us for 22k thick hairs of 100k strands)
+  float* eth_r = nullptr;
+  if (a->radii_old) {
+    HR_TRY(scratch(ctx, 5, (size_t)E * sizeof(float), (void**)&eth_r));
+    k_eth_material<<<(unsigned)(((uint64_t)E * (HR_MAT_FLOATS + 1) + 127) / 128), 128, 0, st>>>(
+        a->verts, a->N, S, a->order, a->cl_first, li, E, a->mat, eth_r, a->d_bounds + kEthBounds);
+    HR_LAUNCHED(ctx);
+    a->radii_old = false;
+  }
   k_eth_prims<<<(unsigned)(((uint64_t)E * S + 255) / 256), 256, 0, st>>>(
-      a->xsec, a->N, S, E, a->cl_first, li, nullptr, a->prim_uv, a->prim_box, a->prim_wa,
+      a->xsec, a->N, S, E, a->cl_first, li, eth_r, a->prim_uv, a->prim_box, a->prim_wa,
       a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   return HR_OK;
