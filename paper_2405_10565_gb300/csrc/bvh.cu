@@ -223,6 +223,7 @@ struct QBox {
   uint32_t x, y, z;
 };
 __device__ __forceinline__ uint32_t q_axis(float l, float h, float lo, float inv_step) {
+  if (!(l <= h)) return 0xffffffffu;  // not a number (its record is never hit): empty, adds nothing
   const float a = floorf((l - lo) * inv_step) - 1.f, b = ceilf((h - lo) * inv_step) + 1.f;
   const uint32_t qa = (uint32_t)fminf(fmaxf(a, 0.f), 65535.f);
   const uint32_t qb = (uint32_t)fminf(fmaxf(b, 0.f), 65535.f);
@@ -273,8 +274,8 @@ __device__ __forceinline__ void append_start(bool has, int v, unsigned* count, i
 // The block's bounds (shared memory, ordered float bits) widened by the boxes of
 // the threads with one.  Whole warps call it.
 __device__ __forceinline__ void widen_bounds(const float4 bl, const float4 bh, bool has, uint32_t* bound) {
-  const uint32_t lo[3] = {ordered_bits(bl.x + 0.f), ordered_bits(bl.y + 0.f), ordered_bits(bl.z + 0.f)};
-  const uint32_t hi[3] = {ordered_bits(bh.x + 0.f), ordered_bits(bh.y + 0.f), ordered_bits(bh.z + 0.f)};
+  const uint32_t lo[3] = {low_bits(bl.x + 0.f), low_bits(bl.y + 0.f), low_bits(bl.z + 0.f)};
+  const uint32_t hi[3] = {high_bits(bh.x + 0.f), high_bits(bh.y + 0.f), high_bits(bh.z + 0.f)};
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const uint32_t l = __reduce_min_sync(0xffffffffu, has ? lo[i] : 0xffffffffu);

@@ -204,6 +204,10 @@ __device__ __forceinline__ uint32_t ordered_bits(float f) {
 __device__ __forceinline__ float from_ordered(uint32_t u) {
   return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
+// The same of a box's low and high corner for a minimum and a maximum: a NaN
+// (a vertex that is not a number) changes neither.
+__device__ __forceinline__ uint32_t low_bits(float f) { return f == f ? ordered_bits(f) : 0xffffffffu; }
+__device__ __forceinline__ uint32_t high_bits(float f) { return f == f ? ordered_bits(f) : 0u; }
 // st_fit: run the clusters and the fit on this stream (the side stream of a
 // pipelined hr_render_frame), the thick-hair records on the main stream after
 // them; null: everything on the main stream.

@@ -191,8 +191,8 @@ __global__ void k_strand_prims(const float4* __restrict__ verts, const float4* _
 // bounds folded into the global ones: nothing to do once another block has
 // reached as far.  The whole block calls fold_bounds.
 __device__ __forceinline__ void widen(uint32_t b[6], const float4 l, const float4 h) {
-  b[0] = min(b[0], ordered_bits(l.x)), b[1] = min(b[1], ordered_bits(l.y)), b[2] = min(b[2], ordered_bits(l.z));
-  b[3] = max(b[3], ordered_bits(h.x)), b[4] = max(b[4], ordered_bits(h.y)), b[5] = max(b[5], ordered_bits(h.z));
+  b[0] = min(b[0], low_bits(l.x)), b[1] = min(b[1], low_bits(l.y)), b[2] = min(b[2], low_bits(l.z));
+  b[3] = max(b[3], high_bits(h.x)), b[4] = max(b[4], high_bits(h.y)), b[5] = max(b[5], high_bits(h.z));
 }
 __device__ __forceinline__ void fold_bounds(const uint32_t b[6], uint32_t* bounds) {
   __shared__ uint32_t s_b[6];
@@ -1010,12 +1010,12 @@ __global__ void k_prim_bounds(const float4* __restrict__ box, uint64_t n, uint32
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (uint64_t)gridDim.x * blockDim.x) {
     const float4 l = box[2 * i], h = box[2 * i + 1];
-    lo[0] = min(lo[0], ordered_bits(l.x));
-    lo[1] = min(lo[1], ordered_bits(l.y));
-    lo[2] = min(lo[2], ordered_bits(l.z));
-    hi[0] = max(hi[0], ordered_bits(h.x));
-    hi[1] = max(hi[1], ordered_bits(h.y));
-    hi[2] = max(hi[2], ordered_bits(h.z));
+    lo[0] = min(lo[0], low_bits(l.x));
+    lo[1] = min(lo[1], low_bits(l.y));
+    lo[2] = min(lo[2], low_bits(l.z));
+    hi[0] = max(hi[0], high_bits(h.x));
+    hi[1] = max(hi[1], high_bits(h.y));
+    hi[2] = max(hi[2], high_bits(h.z));
   }
   for (int i = 0; i < 3; ++i) {
     for (int o = 16; o; o >>= 1) {
