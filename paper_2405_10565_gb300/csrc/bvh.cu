@@ -15,17 +15,21 @@
 // k_gather_refit gathers the leaf boxes in Morton order and finishes the nodes
 // whose leaf range lies inside its thread block's leaves (nearly all of them)
 // in barrier-separated rounds in shared memory; k_climb finishes the few nodes
-// that span blocks by atomic minima of the quantised planes from each climb
-// start, and k_span_records packs those nodes.
+// that span blocks by atomic minima of the planes from each climb start, and
+// k_span_records packs those nodes.
 //
-// Node layout (2 x uint4 = 32 bytes, one sector), children's boxes stored in
-// the parent: per child the x, y and z intervals and the child index.  An
-// interval is lo | hi << 16 on the BVH's grid (Bvh::frame: 65,520 steps over
-// the bounds of every strand and thick-hair box), rounded outward and widened
-// by one step more, which covers the half step that the traversal's decoding
-// can be off.  A child index >= 0 is an internal node, < 0 is primitive
-// ~index.  FP32 boxes took two sectors: a far larger part of the traversal's
-// loads missed L1 (the 4K frame of 500k strands: 25% of the sectors).
+// Node layouts, children's boxes stored in the parent; a child index >= 0 is
+// an internal node, < 0 is primitive ~index:
+//  * On a grid (2 x uint4 = 32 bytes, one sector): per child the x, y and z
+//    intervals and the child index.  An interval is lo | hi << 16 on the BVH's
+//    grid (Bvh::frame: 65,520 steps over the bounds of every strand and
+//    thick-hair box), rounded outward and widened by one step more, which
+//    covers the half step that the traversal's decoding can be off.  FP32
+//    boxes take two sectors: a far larger part of the traversal's loads missed
+//    L1 (the 4K frame of 500k strands: 25% of the sectors).
+//  * In FP32 (4 x float4 = 64 bytes), for scenes that the grid does not
+//    resolve (scene_grid): (lo0.x, hi0.x, lo0.y, hi0.y), (lo1.x, hi1.x, lo1.y,
+//    hi1.y), (lo0.z, hi0.z, lo1.z, hi1.z), (child0, child1, -, -).
 #include <algorithm>
 #include <vector>
 
@@ -48,11 +52,135 @@ __global__ void k_cluster_counts(const uint8_t* __restrict__ lod, const uint32_t
   if (l < L) atomicAdd(counts + C + 1, eths * S);
 }
 
-__global__ void k_cluster_fill(const uint8_t* __restrict__ lod, const uint32_t* __restrict__ cl_first,
+__device__ __forceinline__ uint32_t spread10(uint32_t v) {
+  v &= 0x3ffu;
+  v = (v | (v << 16)) & 0x030000FFu;
+  v = (v | (v << 8)) & 0x0300F00Fu;
+  v = (v | (v << 4)) & 0x030C30C3u;
+  v = (v | (v << 2)) & 0x09249249u;
+  return v;
+}
+
+constexpr size_t kFrameWords = 7;
+
+// What a build or refit takes from the scene as a whole (Bvh::frame), and the
+// leaves' bounds and the climb's counts cleared for k_gather_refit:
+//  * The grid of the node boxes, from the bounds of the strands' and the thick
+//    hairs' boxes: low corner (two steps below the bounds; its fourth word says
+//    whether the nodes are in FP32), step, 1 / step.
+//  * The centroid codes' low corner and 1 / extent.
+// A whole block of WARPS warps calls it.
+// The grid resolves a scene whose boxes are many steps long; one far vertex or
+// parts of very different scale make it so coarse that neighbouring boxes
+// become the same, and so does the codes' cell.  So the block looks at 1,024
+// strand segments, spread evenly (and not in step with the strands): where more than one in kCoarsePart is not
+// kFineSteps steps long in any axis, or the bounds are not finite, the nodes are
+// in FP32, and the codes spread over the bulk of the segments instead of the
+// bounds: of 32 groups of 32 the 25th least minimum and the 25th greatest
+// maximum (three groups in four may hold far ones) and half as much on each side.
+// BVH and image, us a frame of 100k strands, one vertex put ever farther away,
+// on the grid / in FP32 by the steps of the median segment: a close view at 202
+// steps 3,692 / 3,821, at 113 3,844 / 3,820, at 60 4,080 / 3,814, at 16 5,577 /
+// 3,812, at 1 136,091 / 3,817; a far view at 113 1,535 / 1,629, at 60 1,628 /
+// 1,626, at 16 1,709 / 1,631, at 1 4,979 / 1,623.
+constexpr float kFineSteps = 64.f;
+constexpr uint32_t kCoarsePart = 8;
+template <int WARPS>
+__device__ __forceinline__ void scene_grid(const uint32_t* __restrict__ bounds,
+                                           const float4* __restrict__ box, uint32_t n, float4* frame,
+                                           unsigned* counts) {
+  __shared__ uint32_t s_coarse, s_lo[3][32], s_hi[3][32];
+  constexpr int R = 32 / WARPS;  // groups a warp takes
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float4 l[R], h[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const size_t at = __umulhi(((w * R + r) * 32 + lane) * 2654435769u, n);  // golden-ratio steps
+    l[r] = box[2 * at], h[r] = box[2 * at + 1];
+  }
+  if (threadIdx.x == 0) s_coarse = 0u;
+  __syncthreads();
+  float lo[3], hi[3], st[3], clo[3], cinv[3];
+  for (int i = 0; i < 3; ++i) {
+    lo[i] = clo[i] = from_ordered(bounds[i]);
+    hi[i] = from_ordered(bounds[3 + i]);
+    cinv[i] = hi[i] > lo[i] ? 1.f / (hi[i] - lo[i]) : 0.f;
+    const uint32_t el = bounds[kEthBounds + i], eh = bounds[kEthBounds + 3 + i];
+    if (el <= eh) {  // there are thick hairs
+      lo[i] = fminf(lo[i], from_ordered(el));
+      hi[i] = fmaxf(hi[i], from_ordered(eh));
+    }
+    st[i] = fmaxf((hi[i] - lo[i]) * (1.0f / 65520.0f), 1e-30f);
+    lo[i] = fmaf(-2.0f, st[i], lo[i]);
+  }
+  uint32_t coarse = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const bool fine = h[r].x - l[r].x >= kFineSteps * st[0] || h[r].y - l[r].y >= kFineSteps * st[1] ||
+                      h[r].z - l[r].z >= kFineSteps * st[2];
+    coarse += __popc(__ballot_sync(0xffffffffu, !fine));
+  }
+  if (lane == 0 && coarse) atomicAdd(&s_coarse, coarse);
+  __syncthreads();
+  const bool finite = fabsf(lo[0] + lo[1] + lo[2]) + st[0] + st[1] + st[2] < __int_as_float(0x7f800000);
+  const bool wide = s_coarse * kCoarsePart > 1024u || !finite;
+  if (wide) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float c[3] = {0.5f * (l[r].x + h[r].x), 0.5f * (l[r].y + h[r].y), 0.5f * (l[r].z + h[r].z)};
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const uint32_t a = __reduce_min_sync(0xffffffffu, low_bits(c[i]));
+        const uint32_t b = __reduce_max_sync(0xffffffffu, high_bits(c[i]));
+        if (lane == 0) s_lo[i][w * R + r] = a, s_hi[i][w * R + r] = b;
+      }
+    }
+    __syncthreads();
+    for (int i = 0; i < 3; ++i) {
+      uint32_t a = 0, b = 0;  // the group whose minimum, maximum is the 25th
+      for (uint32_t g = 0; g < 32; ++g) {
+        uint32_t ra = 0, rb = 0;
+        for (uint32_t q = 0; q < 32; ++q) {
+          ra += s_lo[i][q] < s_lo[i][g] || (s_lo[i][q] == s_lo[i][g] && q < g);
+          rb += s_hi[i][q] > s_hi[i][g] || (s_hi[i][q] == s_hi[i][g] && q < g);
+        }
+        if (ra == 24) a = g;
+        if (rb == 24) b = g;
+      }
+      const float l = from_ordered(s_lo[i][a]), h = from_ordered(s_hi[i][b]), e = h - l;
+      const bool some = e > 0.f && e < 1e38f;
+      clo[i] = some ? fmaf(-0.5f, e, l) : 0.f;
+      cinv[i] = some ? 0.5f / e : 0.f;
+    }
+  }
+  if (threadIdx.x) return;
+  frame[0] = make_float4(lo[0], lo[1], lo[2], wide ? 1.f : 0.f);
+  frame[1] = make_float4(st[0], st[1], st[2], 0.f);
+  frame[2] = make_float4(1.0f / st[0], 1.0f / st[1], 1.0f / st[2], 0.f);
+  uint32_t* leaf_bounds = reinterpret_cast<uint32_t*>(frame + 3);
+  for (int i = 0; i < 6; ++i) leaf_bounds[i] = i < 3 ? 0xffffffffu : 0u;
+  frame[5] = make_float4(clo[0], clo[1], clo[2], 0.f);
+  frame[6] = make_float4(cinv[0], cinv[1], cinv[2], 0.f);
+  if (counts) counts[0] = counts[1] = 0u;
+}
+
+__global__ void __launch_bounds__(256)
+    k_scene_grid(const uint32_t* __restrict__ bounds, const float4* __restrict__ box, uint32_t n,
+                 float4* frame, unsigned* counts) {
+  scene_grid<8>(bounds, box, n, frame, counts);
+}
+
+__global__ void __launch_bounds__(256, 8) k_cluster_fill(const uint8_t* __restrict__ lod, const uint32_t* __restrict__ cl_first,
                                const uint32_t* __restrict__ order, const uint32_t* __restrict__ offs,
                                const uint32_t* __restrict__ eth_off, uint32_t C, uint32_t L,
-                               uint32_t N, uint32_t S, uint32_t* ids) {
-  const uint32_t c = blockIdx.x;
+                               uint32_t N, uint32_t S, uint32_t* ids,
+                               const uint32_t* __restrict__ bounds, const float4* __restrict__ box,
+                               float4* frame, unsigned* counts) {
+  if (blockIdx.x == 0) {
+    scene_grid<8>(bounds, box, N * S, frame, counts);
+    return;
+  }
+  const uint32_t c = blockIdx.x - 1;
   const uint32_t l = min((uint32_t)lod[c], L);
   const uint32_t base = offs[c];
   if (l == L) {
@@ -78,48 +206,14 @@ __global__ void k_cluster_fill(const uint8_t* __restrict__ lod, const uint32_t* 
   }
 }
 
-__global__ void k_iota(uint32_t* ids, uint32_t n) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) ids[i] = i;
-}
-
-__device__ __forceinline__ uint32_t spread10(uint32_t v) {
-  v &= 0x3ffu;
-  v = (v | (v << 16)) & 0x030000FFu;
-  v = (v | (v << 8)) & 0x0300F00Fu;
-  v = (v | (v << 4)) & 0x030C30C3u;
-  v = (v | (v << 2)) & 0x09249249u;
-  return v;
-}
-
-constexpr size_t kFrameWords = 5;
-
-// The grid of the node boxes, from the bounds of the strands' and the thick
-// hairs' boxes: low corner (two steps below the bounds), step, 1 / step; and
-// the leaves' bounds and the climb's counts cleared for k_gather_refit.
-__device__ __forceinline__ void begin_refit(const uint32_t* __restrict__ bounds, float4* grid,
-                                            uint32_t* leaf_bounds, unsigned* counts) {
-  float lo[3], hi[3], st[3];
-  for (int i = 0; i < 3; ++i) {
-    lo[i] = from_ordered(bounds[i]);
-    hi[i] = from_ordered(bounds[3 + i]);
-    const uint32_t el = bounds[kEthBounds + i], eh = bounds[kEthBounds + 3 + i];
-    if (el <= eh) {  // there are thick hairs
-      lo[i] = fminf(lo[i], from_ordered(el));
-      hi[i] = fmaxf(hi[i], from_ordered(eh));
-    }
-    st[i] = fmaxf((hi[i] - lo[i]) * (1.0f / 65520.0f), 1e-30f);
-    lo[i] = fmaf(-2.0f, st[i], lo[i]);
+__global__ void __launch_bounds__(256, 8) k_iota(uint32_t* ids, uint32_t n, const uint32_t* __restrict__ bounds,
+                       const float4* __restrict__ box, float4* frame, unsigned* counts) {
+  if (blockIdx.x == 0) {
+    scene_grid<8>(bounds, box, n, frame, counts);
+    return;
   }
-  grid[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
-  grid[1] = make_float4(st[0], st[1], st[2], 0.f);
-  grid[2] = make_float4(1.0f / st[0], 1.0f / st[1], 1.0f / st[2], 0.f);
-  for (int i = 0; leaf_bounds && i < 6; ++i) leaf_bounds[i] = i < 3 ? 0xffffffffu : 0u;
-  counts[0] = counts[1] = 0u;
-}
-
-__global__ void k_begin_refit(const uint32_t* __restrict__ bounds, float4* frame, unsigned* counts) {
-  begin_refit(bounds, frame, reinterpret_cast<uint32_t*>(frame + 3), counts);
+  const uint32_t i = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
+  if (i < n) ids[i] = i;
 }
 
 // Primitive centroid codes keep the top 7 bits of each axis (21 bits, three
@@ -131,15 +225,8 @@ __global__ void k_begin_refit(const uint32_t* __restrict__ bounds, float4* frame
 // (the cells then hold too many primitives).
 constexpr int kMortonBits = 21;
 
-__device__ __forceinline__ uint32_t prim_code(const float4 l, const float4 h,
-                                              const uint32_t* __restrict__ bounds) {
-  float3 lo, hi, inv_ext;
-  lo.x = from_ordered(__ldg(bounds)), lo.y = from_ordered(__ldg(bounds + 1));
-  lo.z = from_ordered(__ldg(bounds + 2)), hi.x = from_ordered(__ldg(bounds + 3));
-  hi.y = from_ordered(__ldg(bounds + 4)), hi.z = from_ordered(__ldg(bounds + 5));
-  inv_ext.x = hi.x > lo.x ? 1.f / (hi.x - lo.x) : 0.f;
-  inv_ext.y = hi.y > lo.y ? 1.f / (hi.y - lo.y) : 0.f;
-  inv_ext.z = hi.z > lo.z ? 1.f / (hi.z - lo.z) : 0.f;
+__device__ __forceinline__ uint32_t prim_code(const float4 l, const float4 h, const float4* frame) {
+  const float4 lo = frame[5], inv_ext = frame[6];
   const float cx = (0.5f * (l.x + h.x) - lo.x) * inv_ext.x;
   const float cy = (0.5f * (l.y + h.y) - lo.y) * inv_ext.y;
   const float cz = (0.5f * (l.z + h.z) - lo.z) * inv_ext.z;
@@ -150,13 +237,11 @@ __device__ __forceinline__ uint32_t prim_code(const float4 l, const float4 h,
 }
 
 __global__ void k_prim_morton(const float4* __restrict__ box, const uint32_t* __restrict__ ids,
-                              uint32_t n, const uint32_t* __restrict__ bounds, uint32_t* keys,
-                              float4* frame, unsigned* counts) {
+                              uint32_t n, const float4* __restrict__ frame, uint32_t* keys) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) begin_refit(bounds, frame, reinterpret_cast<uint32_t*>(frame + 3), counts);
   if (i >= n) return;
   const uint32_t id = ids[i];
-  keys[i] = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], bounds);
+  keys[i] = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], frame);
 }
 // Length of the common prefix of (key, index) at i and j; -1 outside [0, n).
 __device__ __forceinline__ int delta(const uint32_t* __restrict__ keys, int n, uint32_t ki, int i,
@@ -217,11 +302,16 @@ __global__ void k_gather(const uint32_t* __restrict__ sorted_ids, uint32_t n, ui
   if (i < n) leaf_id[i] = sorted_ids[i];
 }
 
-// A box on the grid: per axis lo | (65535 - hi) << 16, so that the union of
-// two boxes is the smaller of each half.
+// Boxes of the two node layouts.  Both have: the box of a leaf, the union,
+// the six words whose minima are the union's (k_climb), a node's two children's
+// boxes out of its record, and the record.
+//
+// On the grid: per axis lo | (65535 - hi) << 16, so that the union of two
+// boxes is the smaller of each half.
 struct QBox {
   uint32_t x, y, z;
 };
+constexpr uint32_t kFlipHi = 0xffff0000u;  // 65535 - hi <-> hi
 __device__ __forceinline__ uint32_t q_axis(float l, float h, float lo, float inv_step) {
   if (!(l <= h)) return 0xffffffffu;  // not a number (its record is never hit): empty, adds nothing
   const float a = floorf((l - lo) * inv_step) - 1.f, b = ceilf((h - lo) * inv_step) + 1.f;
@@ -229,34 +319,102 @@ __device__ __forceinline__ uint32_t q_axis(float l, float h, float lo, float inv
   const uint32_t qb = (uint32_t)fminf(fmaxf(b, 0.f), 65535.f);
   return qa | ((65535u - qb) << 16);
 }
-__device__ __forceinline__ QBox q_box(const float4 l, const float4 h, const float4 lo, const float4 is) {
-  return QBox{q_axis(l.x, h.x, lo.x, is.x), q_axis(l.y, h.y, lo.y, is.y), q_axis(l.z, h.z, lo.z, is.z)};
+__device__ __forceinline__ void leaf_box(QBox& b, const float4 l, const float4 h, const float4* grid) {
+  const float4 lo = grid[0], is = grid[2];
+  b = QBox{q_axis(l.x, h.x, lo.x, is.x), q_axis(l.y, h.y, lo.y, is.y), q_axis(l.z, h.z, lo.z, is.z)};
 }
-__device__ __forceinline__ QBox q_union(const QBox a, const QBox b) {
+__device__ __forceinline__ QBox box_union(const QBox a, const QBox b) {
   return QBox{__vminu2(a.x, b.x), __vminu2(a.y, b.y), __vminu2(a.z, b.z)};
 }
-constexpr uint32_t kFlipHi = 0xffff0000u;  // 65535 - hi <-> hi
+__device__ __forceinline__ void box_words(const QBox b, uint32_t w[6]) {
+  w[0] = b.x & 0xffffu, w[1] = b.x >> 16, w[2] = b.y & 0xffffu, w[3] = b.y >> 16;
+  w[4] = b.z & 0xffffu, w[5] = b.z >> 16;
+}
+__device__ __forceinline__ void words_box(QBox& b, const uint32_t* w) {
+  b = QBox{w[0] | w[1] << 16, w[2] | w[3] << 16, w[4] | w[5] << 16};
+}
+__device__ __forceinline__ void child_boxes(QBox& a, QBox& b, const uint4* nodes, int node) {
+  const uint4 c0 = nodes[2 * (size_t)node], c1 = nodes[2 * (size_t)node + 1];
+  a = QBox{c0.x ^ kFlipHi, c0.y ^ kFlipHi, c0.z ^ kFlipHi};
+  b = QBox{c1.x ^ kFlipHi, c1.y ^ kFlipHi, c1.z ^ kFlipHi};
+}
 
-__device__ __forceinline__ QBox q_of(const uint4 child) {  // a node record's child box
-  return QBox{child.x ^ kFlipHi, child.y ^ kFlipHi, child.z ^ kFlipHi};
+// In FP32.  fminf and fmaxf leave a NaN out of a union; a box that is not a
+// number in an axis does not bound its record there.
+struct FBox {
+  float lx, ly, lz, hx, hy, hz;
+};
+__device__ __forceinline__ void leaf_box(FBox& b, const float4 l, const float4 h, const float4*) {
+  b = FBox{l.x, l.y, l.z, h.x, h.y, h.z};
+}
+__device__ __forceinline__ FBox box_union(const FBox a, const FBox b) {
+  return FBox{fminf(a.lx, b.lx), fminf(a.ly, b.ly), fminf(a.lz, b.lz),
+              fmaxf(a.hx, b.hx), fmaxf(a.hy, b.hy), fmaxf(a.hz, b.hz)};
+}
+__device__ __forceinline__ void box_words(const FBox b, uint32_t w[6]) {
+  w[0] = low_bits(b.lx), w[2] = low_bits(b.ly), w[4] = low_bits(b.lz);
+  w[1] = ~high_bits(b.hx), w[3] = ~high_bits(b.hy), w[5] = ~high_bits(b.hz);
+}
+__device__ __forceinline__ void words_box(FBox& b, const uint32_t* w) {
+  b = FBox{from_ordered(w[0]), from_ordered(w[2]), from_ordered(w[4]),
+           from_ordered(~w[1]), from_ordered(~w[3]), from_ordered(~w[5])};
+}
+__device__ __forceinline__ void child_boxes(FBox& a, FBox& b, const uint4* nodes, int node) {
+  const float4* r = reinterpret_cast<const float4*>(nodes) + 4 * (size_t)node;
+  const float4 n0 = r[0], n1 = r[1], n2 = r[2];
+  a = FBox{n0.x, n0.z, n2.x, n0.y, n0.w, n2.y};
+  b = FBox{n1.x, n1.z, n2.z, n1.y, n1.w, n2.w};
 }
 
 // The record of a node from its children's boxes and indices.  The records are
 // stored with an L2 evict-last policy: the frame kernel that follows the build
 // reads them (with 64-byte records the full-head frame took 0.60 instead of
 // 0.63 ms).
-__device__ __forceinline__ void store_node(uint4* nodes, int node, const QBox c0, int i0, const QBox c1,
-                                           int i1) {
-  uint4* o = nodes + 2 * (size_t)node;
+template <int N>
+__device__ __forceinline__ void store_record(uint4* o, const uint4 (&v)[N]) {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-  const uint4 v[2] = {make_uint4(c0.x ^ kFlipHi, c0.y ^ kFlipHi, c0.z ^ kFlipHi, (uint32_t)i0),
-                      make_uint4(c1.x ^ kFlipHi, c1.y ^ kFlipHi, c1.z ^ kFlipHi, (uint32_t)i1)};
 #pragma unroll
-  for (int q = 0; q < 2; ++q)
+  for (int q = 0; q < N; ++q)
     asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;"
                  :: "l"(o + q), "r"(v[q].x), "r"(v[q].y), "r"(v[q].z), "r"(v[q].w), "l"(pol)
                  : "memory");
+}
+__device__ __forceinline__ void store_node(uint4* nodes, int node, const QBox c0, int i0, const QBox c1,
+                                           int i1) {
+  const uint4 v[2] = {make_uint4(c0.x ^ kFlipHi, c0.y ^ kFlipHi, c0.z ^ kFlipHi, (uint32_t)i0),
+                      make_uint4(c1.x ^ kFlipHi, c1.y ^ kFlipHi, c1.z ^ kFlipHi, (uint32_t)i1)};
+  store_record(nodes + 2 * (size_t)node, v);
+}
+__device__ __forceinline__ void store_node(uint4* nodes, int node, const FBox a, int i0, const FBox b,
+                                           int i1) {
+  auto u = [](float f) { return __float_as_uint(f); };
+  const uint4 v[4] = {make_uint4(u(a.lx), u(a.hx), u(a.ly), u(a.hy)),
+                      make_uint4(u(b.lx), u(b.hx), u(b.ly), u(b.hy)),
+                      make_uint4(u(a.lz), u(a.hz), u(b.lz), u(b.hz)),
+                      make_uint4((uint32_t)i0, (uint32_t)i1, 0u, 0u)};
+  store_record(nodes + 4 * (size_t)node, v);
+}
+
+// What a node that spans blocks keeps in its record until k_span_records: its
+// slot in the first word, and its children's indices in their places.
+template <typename Box>
+constexpr size_t kNodeWords = sizeof(Box) == sizeof(QBox) ? 2 : 4;
+template <typename Box>
+__device__ __forceinline__ void span_note(uint4* nodes, int node, unsigned slot, int i0, int i1) {
+  uint4* o = nodes + kNodeWords<Box> * (size_t)node;
+  if (kNodeWords<Box> == 2) {
+    o[0] = make_uint4(slot, 0u, 0u, (uint32_t)i0);
+    o[1] = make_uint4(0u, 0u, 0u, (uint32_t)i1);
+  } else {
+    o[0] = make_uint4(slot, 0u, 0u, 0u);
+    o[3] = make_uint4((uint32_t)i0, (uint32_t)i1, 0u, 0u);
+  }
+}
+template <typename Box>
+__device__ __forceinline__ int2 span_children(const uint4* nodes, int node) {
+  const uint4* o = nodes + kNodeWords<Box> * (size_t)node;
+  return kNodeWords<Box> == 2 ? make_int2((int)o[0].w, (int)o[1].w) : make_int2((int)o[3].x, (int)o[3].y);
 }
 
 // Warp-aggregated append of one child (node index, or ~leaf) per lane that
@@ -289,10 +447,11 @@ __device__ __forceinline__ void widen_bounds(const float4 bl, const float4 bh, b
 
 // Records of the nodes whose leaves lie in the block's (thread j's node is
 // `node`, with children ch, if `local`), one level of readiness per round.
-// The whole block calls it, its leaves' ids and boxes and cleared flags in
-// shared memory.
+// The whole block calls it, its leaves' ids and cleared flags in shared
+// memory; leaf(i) is the box of the block's leaf i.
+template <typename Box, typename Leaf>
 __device__ __forceinline__ void local_records(bool local, const int4 ch, int node, int b0, int j,
-                                              const uint32_t* s_id, const QBox* s_lbox, QBox* s_nbox,
+                                              const uint32_t* s_id, const Leaf leaf, Box* s_nbox,
                                               unsigned char* s_done, uint4* nodes) {
   bool pending = local;
   for (;;) {
@@ -300,12 +459,12 @@ __device__ __forceinline__ void local_records(bool local, const int4 ch, int nod
     if (pending)
       ready = (ch.x < 0 || s_done[ch.x - b0]) && (ch.y < 0 || s_done[ch.y - b0]);
     if (ready) {
-      const QBox c0 = ch.x < 0 ? s_lbox[~ch.x - b0] : s_nbox[ch.x - b0];
-      const QBox c1 = ch.y < 0 ? s_lbox[~ch.y - b0] : s_nbox[ch.y - b0];
+      const Box c0 = ch.x < 0 ? leaf(~ch.x - b0) : s_nbox[ch.x - b0];
+      const Box c1 = ch.y < 0 ? leaf(~ch.y - b0) : s_nbox[ch.y - b0];
       // a leaf child is named by its primitive id (the leaf lies in this block)
       store_node(nodes, node, c0, ch.x < 0 ? ~(int)s_id[~ch.x - b0] : ch.x, c1,
                  ch.y < 0 ? ~(int)s_id[~ch.y - b0] : ch.y);
-      s_nbox[j] = q_union(c0, c1);
+      s_nbox[j] = box_union(c0, c1);
     }
     const int any = __syncthreads_or(ready);  // this round's reads of s_done are over
     if (ready) {
@@ -317,12 +476,25 @@ __device__ __forceinline__ void local_records(bool local, const int4 ch, int nod
   }
 }
 
+// The same in FP32, the leaves' boxes read from memory.
+__device__ __forceinline__ void wide_records(bool local, const int4 ch, int node, int b0, int j,
+                                          const uint32_t* s_id, const float4* box, FBox* s_nbox,
+                                          unsigned char* s_done, uint4* nodes) {
+  auto leaf = [&](int i) {
+    FBox b;
+    leaf_box(b, box[2 * (size_t)s_id[i]], box[2 * (size_t)s_id[i] + 1], nullptr);
+    return b;
+  };
+  local_records(local, ch, node, b0, j, s_id, leaf, s_nbox, s_done, nodes);
+}
+
 // Leaf boxes and bottom-up bounds in one kernel.  Thread j of block b owns
 // leaf b0 + j and internal node b0 + j (b0 = b * B).  A node record names a
 // leaf child by ~(its global primitive id), so the frame kernel reads the
 // primitive's records where they are (no copy into leaf order).
 //  1. Gather: each thread reads its leaf's box (and id) into shared memory, on
-//     the grid: three words, united by three 16-bit pair minima.
+//     the grid: three words, united by three 16-bit pair minima.  (FP32 boxes
+//     take that room for the nodes and are read from memory again.)
 //  2. Local subtrees: node i's leaf range starts or ends at leaf i, so a node
 //     whose range lies inside the block's leaves ("local") is owned by a
 //     thread of the block and so are its children.  These are finished in
@@ -335,21 +507,26 @@ __device__ __forceinline__ void local_records(bool local, const int4 ch, int nod
 //     leaf) whose parent spans blocks lists it as a climb start, so that no
 //     block stays resident behind a climb.
 template <int B>
-__global__ void __launch_bounds__(B) k_gather_refit(
+__global__ void __launch_bounds__(B, 8) k_gather_refit(
     const int4* __restrict__ child, const int* __restrict__ parent_int,
     const int* __restrict__ parent_leaf, const float4* __restrict__ box,
     float4* frame, const uint32_t* sorted_ids, int n, uint4* nodes,
     uint32_t* leaf_id, unsigned* counts, int* starts, int* span_node, uint32_t* span) {
   __shared__ int4 s_child[B];
   __shared__ uint32_t s_id[B];  // global primitive id of each of the block's leaves
-  __shared__ QBox s_lbox[B];    // leaf boxes
-  __shared__ QBox s_nbox[B];    // unions of the block's local nodes
+  __shared__ union {
+    struct {
+      QBox lbox[B], nbox[B];  // leaf boxes, unions of the block's local nodes
+    } q;
+    FBox nbox[B];
+  } s_box;
   __shared__ unsigned char s_done[B];
   __shared__ uint32_t s_bound[6];
   const int b0 = blockIdx.x * B;
   const int j = threadIdx.x;
   const int leaf = b0 + j, node = b0 + j;
   const bool has_node = node <= n - 2;
+  const bool wide = __ldg(&frame[0].w) != 0.f;
   int4 ch = make_int4(0, 0, -1, -1);
   if (has_node) ch = __ldg(child + node);
   s_child[j] = ch;
@@ -365,7 +542,7 @@ __global__ void __launch_bounds__(B) k_gather_refit(
     s_id[j] = id;
     bl = box[2 * (size_t)id];
     bh = box[2 * (size_t)id + 1];
-    s_lbox[j] = q_box(bl, bh, __ldg(frame), __ldg(frame + 2));
+    if (!wide) leaf_box(s_box.q.lbox[j], bl, bh, frame);
   }
   if (j < 6) s_bound[j] = j < 3 ? 0xffffffffu : 0u;
   __syncthreads();
@@ -385,7 +562,11 @@ __global__ void __launch_bounds__(B) k_gather_refit(
     }
   }
   // 2. local subtrees
-  local_records(node_local, ch, node, b0, j, s_id, s_lbox, s_nbox, s_done, nodes);
+  if (!wide)
+    local_records(node_local, ch, node, b0, j, s_id, [&](int i) { return s_box.q.lbox[i]; }, s_box.q.nbox,
+                  s_done, nodes);
+  else
+    wide_records(node_local, ch, node, b0, j, s_id, box, s_box.nbox, s_done, nodes);
   // 3. nodes that span blocks: empty child boxes, widened by k_climb
   const bool spans = has_node && !node_local;
   const unsigned m = __ballot_sync(0xffffffffu, spans);
@@ -400,8 +581,8 @@ __global__ void __launch_bounds__(B) k_gather_refit(
       for (int q = 0; q < 12; ++q) span[12 * (size_t)slot + q] = 0xffffffffu;
       const int c0 = ch.x < 0 ? ~(int)sorted_ids[~ch.x] : ch.x;
       const int c1 = ch.y < 0 ? ~(int)sorted_ids[~ch.y] : ch.y;
-      nodes[2 * (size_t)node] = make_uint4(slot, 0u, 0u, (uint32_t)c0);
-      nodes[2 * (size_t)node + 1] = make_uint4(0u, 0u, 0u, (uint32_t)c1);
+      if (!wide) span_note<QBox>(nodes, node, slot, c0, c1);
+      else span_note<FBox>(nodes, node, slot, c0, c1);
     }
   }
   bool start_leaf = false, start_node = false;
@@ -423,37 +604,43 @@ __global__ void __launch_bounds__(B) k_gather_refit(
 // the first ancestor that it does not change: that one already holds a value
 // at least as wide from another start below it, which carries it on up.  No
 // ordering between starts is needed.
-__global__ void k_climb(const unsigned* __restrict__ counts, const int* __restrict__ starts,
-                        const int* __restrict__ parent_int, const int* __restrict__ parent_leaf,
-                        const float4* __restrict__ box, const float4* __restrict__ frame,
-                        const uint32_t* __restrict__ leaf_id, const uint4* __restrict__ nodes,
-                        uint32_t* span) {
+template <typename Box>
+__device__ __forceinline__ void climb(const unsigned* __restrict__ counts, const int* __restrict__ starts,
+                                      const int* __restrict__ parent_int,
+                                      const int* __restrict__ parent_leaf, const float4* __restrict__ box,
+                                      const float4* __restrict__ frame,
+                                      const uint32_t* __restrict__ leaf_id,
+                                      const uint4* __restrict__ nodes, uint32_t* span) {
+  constexpr size_t W = kNodeWords<Box>;
   const unsigned m = *counts;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
     const int cur = __ldg(starts + i);
-    QBox u;
+    Box u;
     int p;  // 2 * node + side; negative above the root
     if (cur < 0) {
       const size_t id = __ldg(leaf_id + ~cur);
-      u = q_box(__ldg(box + 2 * id), __ldg(box + 2 * id + 1), __ldg(frame), __ldg(frame + 2));
+      leaf_box(u, __ldg(box + 2 * id), __ldg(box + 2 * id + 1), frame);
       p = __ldg(parent_leaf + ~cur);
     } else {
-      u = q_union(q_of(__ldg(nodes + 2 * (size_t)cur)), q_of(__ldg(nodes + 2 * (size_t)cur + 1)));
+      Box c0, c1;
+      child_boxes(c0, c1, nodes, cur);
+      u = box_union(c0, c1);
       p = __ldg(parent_int + cur);
     }
-    const uint32_t b[6] = {u.x & 0xffffu, u.x >> 16, u.y & 0xffffu, u.y >> 16, u.z & 0xffffu, u.z >> 16};
+    uint32_t b[6];
+    box_words(u, b);
     unsigned live = 0x3fu;
     // A start is a chain of levels, its time their latency: the links of the
     // level above are read while this level's atomics are out, and a node's
     // side comes with its link (a thumbnail of 3,001 strands 261 -> 248 us a call)
-    uint32_t slot = __ldg(&nodes[2 * (size_t)(p >> 1)].x);
+    uint32_t slot = __ldg(&nodes[W * (size_t)(p >> 1)].x);
     while (p >= 0) {
       uint32_t* r = span + 12 * (size_t)slot + 6 * (p & 1);
       uint32_t old[6];
 #pragma unroll
       for (int q = 0; q < 6; ++q) old[q] = (live >> q) & 1u ? atomicMin(r + q, b[q]) : 0u;
       p = p >> 1 ? __ldg(parent_int + (p >> 1)) : -1;
-      if (p >= 0) slot = __ldg(&nodes[2 * (size_t)(p >> 1)].x);
+      if (p >= 0) slot = __ldg(&nodes[W * (size_t)(p >> 1)].x);
 #pragma unroll
       for (int q = 0; q < 6; ++q)
         if (old[q] <= b[q]) live &= ~(1u << q);
@@ -461,18 +648,37 @@ __global__ void k_climb(const unsigned* __restrict__ counts, const int* __restri
     }
   }
 }
+__global__ void k_climb(const unsigned* __restrict__ counts, const int* __restrict__ starts,
+                        const int* __restrict__ parent_int, const int* __restrict__ parent_leaf,
+                        const float4* __restrict__ box, const float4* __restrict__ frame,
+                        const uint32_t* __restrict__ leaf_id, const uint4* __restrict__ nodes,
+                        uint32_t* span) {
+  if (__ldg(&frame[0].w) == 0.f)
+    climb<QBox>(counts, starts, parent_int, parent_leaf, box, frame, leaf_id, nodes, span);
+  else
+    climb<FBox>(counts, starts, parent_int, parent_leaf, box, frame, leaf_id, nodes, span);
+}
 
 // The records of the nodes that span blocks, from their slots.
-__global__ void k_span_records(const unsigned* __restrict__ counts, const int* __restrict__ span_node,
-                               const uint32_t* __restrict__ span, uint4* nodes) {
-  const unsigned m = counts[1];
+template <typename Box>
+__device__ __forceinline__ void span_records(unsigned m, const int* __restrict__ span_node,
+                                             const uint32_t* __restrict__ span, uint4* nodes) {
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    const uint32_t* r = span + 12 * (size_t)i;
     const int node = span_node[i];
-    const int c0 = (int)nodes[2 * (size_t)node].w, c1 = (int)nodes[2 * (size_t)node + 1].w;
-    store_node(nodes, node, QBox{r[0] | r[1] << 16, r[2] | r[3] << 16, r[4] | r[5] << 16}, c0,
-               QBox{r[6] | r[7] << 16, r[8] | r[9] << 16, r[10] | r[11] << 16}, c1);
+    const int2 ch = span_children<Box>(nodes, node);
+    Box c0, c1;
+    words_box(c0, span + 12 * (size_t)i);
+    words_box(c1, span + 12 * (size_t)i + 6);
+    store_node(nodes, node, c0, ch.x, c1, ch.y);
   }
+}
+__global__ void k_span_records(const unsigned* __restrict__ counts, const int* __restrict__ span_node,
+                               const uint32_t* __restrict__ span, const float4* __restrict__ frame,
+                               uint4* nodes) {
+  if (__ldg(&frame[0].w) == 0.f)
+    span_records<QBox>(counts[1], span_node, span, nodes);
+  else
+    span_records<FBox>(counts[1], span_node, span, nodes);
 }
 
 // A whole BVH of 2 to 1,024 leaves in one block, a leaf and a node per thread:
@@ -488,28 +694,25 @@ struct SmallBvh {
     struct {
       QBox lbox[kSmallLeaves], nbox[kSmallLeaves];
     } box;
+    FBox nbox[kSmallLeaves];
   };
   uint32_t key[kSmallLeaves], id[kSmallLeaves];
   unsigned char done[kSmallLeaves];
-  uint32_t sum[8], bound[6];
-  float4 grid[3];
+  uint32_t sum[8];
+  float4 frame[kFrameWords];
 };
 __global__ void __launch_bounds__(kSmallLeaves)
-    k_small_bvh(const float4* __restrict__ box, const uint32_t* __restrict__ ids, int n,
+    k_small_bvh(const float4* __restrict__ box, const uint32_t* __restrict__ ids, int n, uint32_t NS,
                 const uint32_t* __restrict__ bounds, float4* frame, int4* child, int* parent_int,
                 int* parent_leaf, uint32_t* leaf_id, uint4* nodes) {
   __shared__ SmallBvh sm;
   const int j = threadIdx.x, lane = j & 31, w = j >> 5;
   const uint32_t lt = (1u << lane) - 1u;
-  if (j == 0) {
-    unsigned counts[2];
-    begin_refit(bounds, sm.grid, nullptr, counts);
-    frame[0] = sm.grid[0], frame[1] = sm.grid[1], frame[2] = sm.grid[2];
-  }
-  if (j < 6) sm.bound[j] = j < 3 ? 0xffffffffu : 0u;
+  scene_grid<kSmallWarps>(bounds, box, NS, sm.frame, nullptr);
+  __syncthreads();
   const bool valid = j < n;
   uint32_t id = valid ? (ids ? ids[j] : (uint32_t)j) : 0u, key = 0u;
-  if (valid) key = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], bounds);
+  if (valid) key = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], sm.frame);
   for (int shift = 0; shift < kMortonBits; shift += 8) {
     for (int i = j; i < kSmallWarps * 256; i += kSmallLeaves) (&sm.whist[0][0])[i] = 0;
     __syncthreads();
@@ -560,21 +763,26 @@ __global__ void __launch_bounds__(kSmallLeaves)
   }
   // leaves: boxes on the grid and exact bounds (the whist words are free)
   __syncthreads();
+  const bool wide = sm.frame[0].w != 0.f;
   float4 bl = make_float4(0.f, 0.f, 0.f, 0.f), bh = bl;
   if (valid) {
     bl = box[2 * (size_t)id];
     bh = box[2 * (size_t)id + 1];
-    sm.box.lbox[j] = q_box(bl, bh, sm.grid[0], sm.grid[2]);
+    if (!wide) leaf_box(sm.box.lbox[j], bl, bh, sm.frame);
     leaf_id[j] = id;
   }
   sm.done[j] = 0;
-  widen_bounds(bl, bh, valid, sm.bound);
+  widen_bounds(bl, bh, valid, reinterpret_cast<uint32_t*>(sm.frame + 3));
   const bool has_node = j < n - 1;
   int4 ch = make_int4(0, 0, -1, -1);
   if (has_node) child[j] = ch = karras_node(sm.key, n, j, parent_int, parent_leaf);
   __syncthreads();
-  if (j < 6) reinterpret_cast<uint32_t*>(frame + 3)[j] = sm.bound[j];
-  local_records(has_node, ch, j, 0, j, sm.id, sm.box.lbox, sm.box.nbox, sm.done, nodes);
+  if (j < (int)kFrameWords) frame[j] = sm.frame[j];
+  if (!wide)
+    local_records(has_node, ch, j, 0, j, sm.id, [&](int i) { return sm.box.lbox[i]; }, sm.box.nbox, sm.done,
+                  nodes);
+  else
+    wide_records(has_node, ch, j, 0, j, sm.id, box, sm.nbox, sm.done, nodes);
 }
 
 __global__ void k_bytes_differ(const uint8_t* __restrict__ x, const uint8_t* __restrict__ y,
@@ -584,7 +792,7 @@ __global__ void k_bytes_differ(const uint8_t* __restrict__ x, const uint8_t* __r
 }
 
 // Every node's record over the topology in bv and the primitives `ids` in leaf
-// order, after begin_refit on the same stream.
+// order, after scene_grid on the same stream.
 hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, cudaStream_t st) {
   const uint32_t n = bv.n;
   unsigned* counts = nullptr;  // climb starts, nodes that span blocks
@@ -614,7 +822,7 @@ hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, c
   k_climb<<<grid, 256, 0, st>>>(counts, starts, bv.par_int, bv.par_leaf, a->prim_box,
                                 bv.frame, bv.leaf_id, bv.nodes, span);
   HR_LAUNCHED(ctx);
-  k_span_records<<<grid, 256, 0, st>>>(counts, span_node, span, bv.nodes);
+  k_span_records<<<grid, 256, 0, st>>>(counts, span_node, span, bv.frame, bv.nodes);
   HR_LAUNCHED(ctx);
   return HR_OK;
 }
@@ -623,7 +831,7 @@ hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, c
 
 void free_bvh(hr_ctx* ctx, Bvh& bv) {
   if (bv.cap) {
-    dfree(ctx, bv.nodes, (size_t)std::max(bv.cap, 2u) * 2 * sizeof(uint4));
+    dfree(ctx, bv.nodes, (size_t)std::max(bv.cap, 2u) * 4 * sizeof(uint4));
     dfree(ctx, bv.frame, kFrameWords * sizeof(float4));
     dfree(ctx, bv.leaf_id, (size_t)bv.cap * 4);
     dfree(ctx, bv.child, (size_t)bv.cap * sizeof(int4));
@@ -637,22 +845,17 @@ void free_bvh(hr_ctx* ctx, Bvh& bv) {
 hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, cudaStream_t st) {
   const uint32_t N = a->N, S = a->S;
   bv.valid = 0;
-  // 1. active primitive ids
+  // 1. active primitives
   uint32_t n = 0, n_eth = 0;
-  uint32_t* ids = nullptr;
-  if (a->C == 0 || a->n_levels == 0 || lod_dev == nullptr) {
+  const bool strands = a->C == 0 || a->n_levels == 0 || lod_dev == nullptr;
+  uint32_t* cnt = nullptr;
+  if (strands) {
     n = N * S;
-    if (n < 2 || n > (uint32_t)kSmallLeaves) {
-      HR_TRY(scratch(ctx, 30, (size_t)n * 4, (void**)&ids));
-      k_iota<<<(n + 255) / 256, 256, 0, st>>>(ids, n);
-      HR_LAUNCHED(ctx);
-    }
   } else {
-    const uint32_t C = a->C, L = a->n_levels;
-    uint32_t* cnt = nullptr;
+    const uint32_t C = a->C;
     HR_TRY(scratch(ctx, 31, (size_t)(C + 2) * 4, (void**)&cnt));
     HR_CUDA(ctx, cudaMemsetAsync(cnt + C, 0, 8, st));
-    k_cluster_counts<<<(C + 255) / 256, 256, 0, st>>>(lod_dev, a->cl_first, C, L, S, cnt);
+    k_cluster_counts<<<(C + 255) / 256, 256, 0, st>>>(lod_dev, a->cl_first, C, a->n_levels, S, cnt);
     HR_LAUNCHED(ctx);
     HR_TRY(scan_u32(ctx, cnt, C + 1, st));
     uint32_t tot[2] = {0, 0};  // active primitives, of which thick-hair segments
@@ -660,12 +863,6 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
     HR_CUDA(ctx, cudaStreamSynchronize(st));
     n = tot[0];
     n_eth = tot[1];
-    uint32_t* eoff = nullptr;
-    HR_TRY(scratch(ctx, 32, 16 * 4, (void**)&eoff));
-    HR_CUDA(ctx, cudaMemcpyAsync(eoff, a->eth_offset, 16 * 4, cudaMemcpyHostToDevice, st));
-    HR_TRY(scratch(ctx, 30, (size_t)std::max(n, 1u) * 4, (void**)&ids));
-    k_cluster_fill<<<C, 256, 0, st>>>(lod_dev, a->cl_first, a->order, cnt, eoff, C, L, N, S, ids);
-    HR_LAUNCHED(ctx);
   }
   // 2. storage (grow only)
   if (n > bv.cap) {
@@ -673,7 +870,7 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
       HR_CUDA(ctx, cudaStreamSynchronize(st));
       free_bvh(ctx, bv);
     }
-    HR_TRY(dalloc(ctx, (void**)&bv.nodes, (size_t)std::max(n, 2u) * 2 * sizeof(uint4), "BVH nodes"));
+    HR_TRY(dalloc(ctx, (void**)&bv.nodes, (size_t)std::max(n, 2u) * 4 * sizeof(uint4), "BVH nodes"));
     HR_TRY(dalloc(ctx, (void**)&bv.frame, kFrameWords * sizeof(float4), "BVH grid"));
     HR_TRY(dalloc(ctx, (void**)&bv.leaf_id, (size_t)n * 4, "BVH leaf ids"));
     HR_TRY(dalloc(ctx, (void**)&bv.child, (size_t)n * sizeof(int4), "BVH children"));
@@ -684,6 +881,26 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
   // (after the grow: free_bvh resets every field)
   bv.n = n;
   bv.n_eth = n_eth;
+  // their ids, and the scene's grid in a block of its own
+  uint32_t* ids = nullptr;
+  unsigned* counts = nullptr;
+  const bool small = n >= 2 && n <= (uint32_t)kSmallLeaves;
+  HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
+  if (strands) {
+    if (!small) {
+      HR_TRY(scratch(ctx, 30, (size_t)n * 4, (void**)&ids));
+      k_iota<<<(n + 255) / 256 + 1, 256, 0, st>>>(ids, n, a->d_bounds, a->prim_box, bv.frame, counts);
+      HR_LAUNCHED(ctx);
+    }
+  } else if (n) {
+    uint32_t* eoff = nullptr;
+    HR_TRY(scratch(ctx, 32, 16 * 4, (void**)&eoff));
+    HR_CUDA(ctx, cudaMemcpyAsync(eoff, a->eth_offset, 16 * 4, cudaMemcpyHostToDevice, st));
+    HR_TRY(scratch(ctx, 30, (size_t)n * 4, (void**)&ids));
+    k_cluster_fill<<<a->C + 1, 256, 0, st>>>(lod_dev, a->cl_first, a->order, cnt, eoff, a->C, a->n_levels,
+                                             N, S, ids, a->d_bounds, a->prim_box, bv.frame, counts);
+    HR_LAUNCHED(ctx);
+  }
   // what the topology is built for (checked by refit_bvh); the hierarchy as it is now
   HR_CUDA(ctx, cudaMemsetAsync(a->d_bounds + kHierChanged, 0, 4, st));
   bv.topo = 0;
@@ -706,8 +923,8 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
     bv.topo = 1;
     return HR_OK;
   }
-  if (n >= 2 && n <= (uint32_t)kSmallLeaves) {  // all in one block
-    k_small_bvh<<<1, kSmallLeaves, 0, st>>>(a->prim_box, ids, (int)n, a->d_bounds, bv.frame, bv.child,
+  if (small) {  // all in one block
+    k_small_bvh<<<1, kSmallLeaves, 0, st>>>(a->prim_box, ids, (int)n, N * S, a->d_bounds, bv.frame, bv.child,
                                             bv.par_int, bv.par_leaf, bv.leaf_id, bv.nodes);
     HR_LAUNCHED(ctx);
     bv.valid = 1;
@@ -719,10 +936,7 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
   HR_TRY(scratch(ctx, 33, (size_t)n * 4, (void**)&keys));
   HR_TRY(scratch(ctx, 34, (size_t)n * 4, (void**)&k2));
   HR_TRY(scratch(ctx, 35, (size_t)n * 4, (void**)&v2));
-  unsigned* counts = nullptr;
-  HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
-  k_prim_morton<<<(n + 255) / 256, 256, 0, st>>>(a->prim_box, ids, n, a->d_bounds, keys, bv.frame,
-                                                 counts);
+  k_prim_morton<<<(n + 255) / 256, 256, 0, st>>>(a->prim_box, ids, n, bv.frame, keys);
   HR_LAUNCHED(ctx);
   HR_TRY(radix_sort_pairs(ctx, keys, ids, k2, v2, n, kMortonBits, st, kLookbackPolls, &keys, &ids));
   if (n == 1) {
@@ -768,7 +982,7 @@ hr_status refit_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
   if (n > 1) {
     unsigned* counts = nullptr;
     HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
-    k_begin_refit<<<1, 1, 0, st>>>(a->d_bounds, bv.frame, counts);
+    k_scene_grid<<<1, 256, 0, st>>>(a->d_bounds, a->prim_box, a->N * a->S, bv.frame, counts);
     HR_LAUNCHED(ctx);
     HR_TRY(gather_refit(ctx, a, bv, bv.leaf_id, st));
   }

@@ -34,9 +34,11 @@ struct TileSched;
 struct Bvh {
   uint32_t n = 0;           // active primitives (leaves)
   uint32_t cap = 0;         // allocated leaves
-  uint4* nodes = nullptr;   // [(n-1) * 2] quantised boxes (see bvh.cu); a leaf child is ~(global primitive id)
-  float4* frame = nullptr;  // [5] the boxes' grid: low corner, step, 1 / step; then, as ordered float
-                            // bits, the leaves' exact bounds lo xyz, hi xyz
+  uint4* nodes = nullptr;   // [(n-1) * 2] on a grid or [(n-1) * 4] in FP32 (see bvh.cu); a leaf
+                            // child is ~(global primitive id)
+  float4* frame = nullptr;  // [7] the boxes' grid: low corner (its fourth word not 0: boxes in FP32),
+                            // step, 1 / step; as ordered float bits, the leaves' exact bounds lo xyz,
+                            // hi xyz; the centroid codes' low corner and 1 / extent
   uint32_t* leaf_id = nullptr; // [n] global primitive id of every leaf, Morton order
   uint32_t n_eth = 0;
   int valid = 0;               // bounds and leaf records match the primitives

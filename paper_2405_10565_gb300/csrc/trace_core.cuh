@@ -4,7 +4,7 @@
 //  * Camera: sample sid = pixel * spp + s; sub-pixel position from SplitMix64
 //    outputs 2 sid and 2 sid + 1 of the frame seed (top 24 bits each).
 //  * Traversal: stack-based over the binary LBVH whose nodes hold both
-//    children's boxes (one 32-byte node fetch tests two boxes); nearer child
+//    children's boxes (one node fetch tests two boxes); nearer child
 //    first.  The search interval shrinks to the K-th nearest hit and to the
 //    nearest opaque (strand) hit: nothing behind an opaque hit can contribute.
 //  * Intersection: the record maps the ray into the cylinder's unit frame;
@@ -476,32 +476,35 @@ __device__ __forceinline__ void leaf_test(const FrameArgs& fa, RayMem<KMAX, COLS
   if (r != kMiss) keep_hit<KMAX, COLS, COUNT>(fa, rm, c, id, r, th, terr, tcut, errmax, cn);
 }
 
-// A ray against the node boxes.  The plane at grid coordinate q is met at
+// A ray against the node boxes (bvh.cu).  The plane at grid coordinate q is met at
 // depth (lo + q step - o) / d.  A byte permutation of the box word with 2^23's
 // bits gives 2^23 + q as a float, and picks the near or the far plane by the
 // ray's direction at no further cost, so a plane takes one permutation and one
 // FMA with scale = step / d and offset = (lo - o) / d - 2^23 scale.  The
 // offset's rounding is at most half a step of depth, which the boxes' extra
 // step covers.  A zero direction component would turn the products into
-// inf - inf, so its sign is kept and its magnitude floored.
+// inf - inf, so its sign is kept and its magnitude floored.  For boxes in FP32
+// scale is 1 / d and offset -o / d.
 struct Slabs {
   float3 scale, off;
   uint32_t nx, ny, nz;  // permutation that picks the near plane (xor kFar: the far one)
+  bool wide;            // the boxes are in FP32
 };
 constexpr uint32_t kNearLo = 0x7610u, kFar = 0x0022u, kTwo23 = 0x4b000000u;
-__device__ __forceinline__ void slab_axis(float o, float d, float lo, float step, float& scale,
+__device__ __forceinline__ void slab_axis(float o, float d, float lo, float step, bool wide, float& scale,
                                           float& off, uint32_t& sel) {
   const float inv = 1.0f / (fabsf(d) > 1e-12f ? d : copysignf(1e-12f, d));
-  scale = step * inv;
-  off = fmaf(-8388608.f, scale, (lo - o) * inv);
+  scale = wide ? inv : step * inv;
+  off = wide ? -(o * inv) : fmaf(-8388608.f, scale, (lo - o) * inv);
   sel = inv < 0.f ? kNearLo ^ kFar : kNearLo;
 }
 __device__ __forceinline__ Slabs ray_slabs(const FrameArgs& fa, const float3 o, const float3 d) {
   const float4 lo = __ldg(fa.frame), st = __ldg(fa.frame + 1);
   Slabs s;
-  slab_axis(o.x, d.x, lo.x, st.x, s.scale.x, s.off.x, s.nx);
-  slab_axis(o.y, d.y, lo.y, st.y, s.scale.y, s.off.y, s.ny);
-  slab_axis(o.z, d.z, lo.z, st.z, s.scale.z, s.off.z, s.nz);
+  s.wide = lo.w != 0.f;
+  slab_axis(o.x, d.x, lo.x, st.x, s.wide, s.scale.x, s.off.x, s.nx);
+  slab_axis(o.y, d.y, lo.y, st.y, s.wide, s.scale.y, s.off.y, s.ny);
+  slab_axis(o.z, d.z, lo.z, st.z, s.wide, s.scale.z, s.off.z, s.nz);
   return s;
 }
 __device__ __forceinline__ float slab_t(uint32_t w, uint32_t sel, float scale, float off) {
@@ -516,6 +519,44 @@ __device__ __forceinline__ bool slab_test(const Slabs& s, const uint4 c, float t
                                   slab_t(c.y, s.ny ^ kFar, s.scale.y, s.off.y)),
                             fminf(slab_t(c.z, s.nz ^ kFar, s.scale.z, s.off.z), tmax));
   return t_in <= t_out;
+}
+
+// The same for a box in FP32: (lo.x, hi.x, lo.y, hi.y) and (lo.z, hi.z).
+__device__ __forceinline__ bool slab_test(const Slabs& s, const float4 xy, float lz, float hz, float tmax,
+                                          float& t_in) {
+  const float x0 = fmaf(xy.x, s.scale.x, s.off.x), x1 = fmaf(xy.y, s.scale.x, s.off.x);
+  const float y0 = fmaf(xy.z, s.scale.y, s.off.y), y1 = fmaf(xy.w, s.scale.y, s.off.y);
+  const float z0 = fmaf(lz, s.scale.z, s.off.z), z1 = fmaf(hz, s.scale.z, s.off.z);
+  t_in = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fmaxf(fminf(z0, z1), 0.f));
+  const float t_out = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fminf(fmaxf(z0, z1), tmax));
+  return t_in <= t_out;
+}
+
+// A node's children: which of them the ray meets before tmax, and where.  The
+// walks are compiled for either kind of node and choose once a ray: a choice at
+// every node took 4 to 5% of the frames on the grid.
+struct Children {
+  bool h0, h1;
+  float a0, a1;
+  int c0, c1;
+};
+template <bool WIDE>
+__device__ __forceinline__ Children node_test(const FrameArgs& fa, const Slabs& s, int node, float tmax) {
+  Children r;
+  if (WIDE) {
+    const float4* n = reinterpret_cast<const float4*>(fa.nodes) + 4 * (size_t)node;
+    const float4 n0 = __ldg(n), n1 = __ldg(n + 1), n2 = __ldg(n + 2);
+    const int2 ch = __ldg(reinterpret_cast<const int2*>(n + 3));
+    r.h0 = slab_test(s, n0, n2.x, n2.y, tmax, r.a0);
+    r.h1 = slab_test(s, n1, n2.z, n2.w, tmax, r.a1);
+    r.c0 = ch.x, r.c1 = ch.y;
+  } else {
+    const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
+    r.h0 = slab_test(s, k0, tmax, r.a0);
+    r.h1 = slab_test(s, k1, tmax, r.a1);
+    r.c0 = (int)k0.w, r.c1 = (int)k1.w;
+  }
+  return r;
 }
 
 // A lane's walk: the next node (kDone: none), the pending ones, the search cut
@@ -556,31 +597,26 @@ __device__ __forceinline__ Walk walk_begin(const FrameArgs& fa, bool live) {
 // straight hair took (whole calls, before long walks were put aside) 14.3,
 // 14.1, 14.1, 14.1 and 15.2 ms, the close view of the full head 4.21, 4.15,
 // 4.14, 4.20 and 4.48 ms.
-template <int KMAX, bool COUNT>
-__device__ __forceinline__ int walk_on(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm, Walk& w,
-                                       int* stack, int steps, Counts& cn) {
-  const Slabs sl = ray_slabs(fa, ray_o(rm, threadIdx.x), ray_d(rm, threadIdx.x));
+template <int KMAX, bool COUNT, bool WIDE>
+__device__ __forceinline__ int walk_nodes(const FrameArgs& fa, const Slabs& sl, RayMem<KMAX, kBlock>& rm,
+                                          Walk& w, int* stack, int steps, Counts& cn) {
   const float pad = 2.f * kTieRel * rm.s_off[threadIdx.x];
   float tcut = w.tcut, errmax = w.errmax;
   int sp = w.sp, node = w.node, stopped = kDone;
   for (;;) {
     if (node >= 0) {
-      const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
       --steps;
       if (COUNT) ++cn.nodes;
-      const float tb = fmaf(tcut + errmax, 1.f + 2.f * kTieRel, pad);
-      float a0, a1;
-      const bool h0 = slab_test(sl, k0, tb, a0), h1 = slab_test(sl, k1, tb, a1);
-      const int c0 = (int)k0.w, c1 = (int)k1.w;
-      if (h0 && h1) {
-        const bool first0 = a0 <= a1;
-        node = first0 ? c0 : c1;
+      const Children ch = node_test<WIDE>(fa, sl, node, fmaf(tcut + errmax, 1.f + 2.f * kTieRel, pad));
+      if (ch.h0 && ch.h1) {
+        const bool first0 = ch.a0 <= ch.a1;
+        node = first0 ? ch.c0 : ch.c1;
         if (sp < kStack)
-          stack[sp++] = first0 ? c1 : c0;
+          stack[sp++] = first0 ? ch.c1 : ch.c0;
         else
           w.ok = false;
-      } else if (h0 || h1) {
-        node = h0 ? c0 : c1;
+      } else if (ch.h0 || ch.h1) {
+        node = ch.h0 ? ch.c0 : ch.c1;
       } else {
         node = sp ? stack[--sp] : kDone;
       }
@@ -604,6 +640,13 @@ __device__ __forceinline__ int walk_on(const FrameArgs& fa, RayMem<KMAX, kBlock>
   w.tcut = tcut;
   w.errmax = errmax;
   return steps;
+}
+template <int KMAX, bool COUNT>
+__device__ __forceinline__ int walk_on(const FrameArgs& fa, RayMem<KMAX, kBlock>& rm, Walk& w,
+                                       int* stack, int steps, Counts& cn) {
+  const Slabs sl = ray_slabs(fa, ray_o(rm, threadIdx.x), ray_d(rm, threadIdx.x));
+  return sl.wide ? walk_nodes<KMAX, COUNT, true>(fa, sl, rm, w, stack, steps, cn)
+                 : walk_nodes<KMAX, COUNT, false>(fa, sl, rm, w, stack, steps, cn);
 }
 
 // The K nearest hits of the warp's rays, one per live lane, without a stop.
@@ -889,39 +932,35 @@ __device__ __forceinline__ bool cross_leaf(const FrameArgs& fa, uint32_t id, con
 }
 
 // One node of a path: the next node, the other hit child on the stack.
+template <bool WIDE>
 __device__ __forceinline__ int path_node(const FrameArgs& fa, const Slabs& sl, int node, const float tmax,
                                          int* stack, int& sp, bool& ok) {
-  const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
-  float a0, a1;
-  const bool h0 = slab_test(sl, k0, tmax, a0), h1 = slab_test(sl, k1, tmax, a1);
-  const int c0 = (int)k0.w, c1 = (int)k1.w;
-  if (h0 && h1) {
+  const Children ch = node_test<WIDE>(fa, sl, node, tmax);
+  if (ch.h0 && ch.h1) {
     if (sp < kStack)
-      stack[sp++] = c1;
+      stack[sp++] = ch.c1;
     else
       ok = false;
-    return c0;
+    return ch.c0;
   }
-  if (h0 || h1) return h0 ? c0 : c1;
+  if (ch.h0 || ch.h1) return ch.h0 ? ch.c0 : ch.c1;
   return sp ? stack[--sp] : kDone;
 }
 
 // The light paths of a warp's lanes (lanes that are not live have none); with
 // WHOLE the whole warp calls it and leaves wait for one another as in walk_on,
 // without it each lane walks by itself.
-template <int PREC, bool COUNT, bool WHOLE>
-__device__ __forceinline__ void shadow_path(const FrameArgs& fa, bool live, const float3 x,
-                                            const float3 wi, const float tmax, const uint32_t self_mat,
-                                            float T[3], float& sg2, bool& ok, Counts& cn) {
-  LightPath lp{{1.f, 1.f, 1.f}, 0.f, false};
-  const Slabs sl = ray_slabs(fa, x, wi);
+template <int PREC, bool COUNT, bool WHOLE, bool WIDE>
+__device__ __forceinline__ void path_walk(const FrameArgs& fa, const Slabs& sl, bool live, const float3 x,
+                                          const float3 wi, const float tmax, const uint32_t self_mat,
+                                          LightPath& lp, bool& ok, Counts& cn) {
   int stack[kStack];
   int sp = 0;
   int node = !live || fa.n_prims == 0 ? kDone : (fa.n_prims == 1 ? ~(int)__ldg(fa.leaf_id) : 0);
   for (;;) {
     if (node >= 0) {
       if (COUNT) ++cn.nodes;
-      node = path_node(fa, sl, node, tmax, stack, sp, ok);
+      node = path_node<WIDE>(fa, sl, node, tmax, stack, sp, ok);
     }
     if (WHOLE) {
       const unsigned inner = __ballot_sync(0xffffffffu, node >= 0);
@@ -937,6 +976,17 @@ __device__ __forceinline__ void shadow_path(const FrameArgs& fa, bool live, cons
                                                                                        : stack[--sp];
     }
   }
+}
+template <int PREC, bool COUNT, bool WHOLE>
+__device__ __forceinline__ void shadow_path(const FrameArgs& fa, bool live, const float3 x,
+                                            const float3 wi, const float tmax, const uint32_t self_mat,
+                                            float T[3], float& sg2, bool& ok, Counts& cn) {
+  LightPath lp{{1.f, 1.f, 1.f}, 0.f, false};
+  const Slabs sl = ray_slabs(fa, x, wi);
+  if (sl.wide)
+    path_walk<PREC, COUNT, WHOLE, true>(fa, sl, live, x, wi, tmax, self_mat, lp, ok, cn);
+  else
+    path_walk<PREC, COUNT, WHOLE, false>(fa, sl, live, x, wi, tmax, self_mat, lp, ok, cn);
   const float dF = lp.crossed ? kDF : 1.f;
   T[0] = lp.T[0] * dF;
   T[1] = lp.T[1] * dF;

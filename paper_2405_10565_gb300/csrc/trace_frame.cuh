@@ -292,12 +292,12 @@ __global__ void __launch_bounds__(kBlock, 6)
         bool h0 = false, h1 = false, swap = false;
         int c0 = 0, c1 = 0;
         if (node >= 0) {
-          const uint4 k0 = __ldg(fa.nodes + 2 * (size_t)node), k1 = __ldg(fa.nodes + 2 * (size_t)node + 1);
           const float tb = fmaf(tcut + errmax, 1.f + 2.f * tr::kTieRel, pad);
-          float a0, a1;
-          h0 = tr::slab_test(sl, k0, tb, a0), h1 = tr::slab_test(sl, k1, tb, a1);
-          swap = a1 < a0;
-          c0 = (int)k0.w, c1 = (int)k1.w;
+          const tr::Children ch =
+              sl.wide ? tr::node_test<true>(fa, sl, node, tb) : tr::node_test<false>(fa, sl, node, tb);
+          h0 = ch.h0, h1 = ch.h1;
+          swap = ch.a1 < ch.a0;
+          c0 = ch.c0, c1 = ch.c1;
         } else if (mine) {  // a leaf that was pending when the ray was put aside
           h0 = true;
           c0 = node;

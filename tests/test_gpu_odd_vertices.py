@@ -1,5 +1,8 @@
-"""Scenes with vertices that are not numbers: the segments that touch one are
-never hit, and every other segment is, as the oracle has it without them."""
+"""Scenes with odd vertices.  One that is not a number or infinite: the
+segments that touch it are never hit, and every other segment is, as the oracle
+has it without them.  One far away, or parts of very different scale, which the
+node boxes' grid does not resolve: as the oracle has the scene, and at the cost
+of the same scene without it."""
 import numpy as np
 import pytest
 
@@ -67,3 +70,74 @@ def test_a_vertex_that_is_not_a_number(ctx, n, S, vertex, axes, update):
         odd[s, vertex, list(axes)] = np.nan
         bad[s, vertex] = True
     _check(ctx, sc, odd, bad, update)
+
+
+@pytest.mark.parametrize("n,S", [(40, 8), (300, 8)])
+@pytest.mark.parametrize("vertex,value", [(0, np.inf), (8, -np.inf), (4, np.inf)])
+def test_an_infinite_vertex(ctx, n, S, vertex, value):
+    sc = _scene(n, S)
+    odd, bad = np.array(sc.verts), np.zeros((n, S + 1), bool)
+    odd[n // 2, vertex, 1] = value
+    bad[n // 2, vertex] = True
+    _check(ctx, sc, odd, bad, False)
+
+
+def _far(sc, distance, vertex=-1):
+    odd = np.array(sc.verts)
+    odd[odd.shape[0] // 2, vertex, :3] += np.asarray([1.0, 0.3, -1.0], np.float32) * distance
+    return odd
+
+
+@pytest.mark.parametrize("n,S", [(40, 8), (300, 8)])
+@pytest.mark.parametrize("distance", [30.0, 1e3, 1e5, 1e9])  # the grid resolves the first alone
+def test_a_vertex_far_away(ctx, n, S, distance):
+    sc = _scene(n, S)
+    _check(ctx, sc, _far(sc, distance), np.zeros((n, S + 1), bool), False)
+
+
+@pytest.mark.parametrize("parts,ratio", [(2, 1e4), (3, 100.0)])
+def test_parts_of_very_different_scale_or_far_apart(ctx, parts, ratio):
+    """Two heads 10,000 heads apart; three of scales 1, 1 / 100 and 1 / 10,000
+    side by side.  The camera sees the first."""
+    sc = _scene(300, 8)
+    n = sc.n_strands
+    odd = np.array(sc.verts)
+    for p in range(1, parts):
+        part = slice(p * n // parts, (p + 1) * n // parts)
+        if parts == 2:
+            odd[part, :, :3] += np.asarray([0.0, 0.0, ratio], np.float32)
+        else:
+            odd[part, :, :3] = odd[part, :, :3] * ratio ** -p + np.asarray([1.5 * p, 0.0, 0.0], np.float32)
+            odd[part, :, 3] *= ratio ** -p
+    _check(ctx, sc, odd, np.zeros((n, 9), bool), False)
+
+
+@pytest.mark.parametrize("settled", ["built", "refit"])
+@pytest.mark.parametrize("distance", [1e3, 1e5])
+def test_a_far_vertex_costs_little(ctx, distance, settled):
+    """Node visits of a counting frame of 3,000 strands (clustered, so that the
+    list of leaves is in order): without the far vertex 1, with it below 2."""
+    w = scenegen.clustered(n=3000, S=16, res=96, spp=2, lod_setting="strands", n_clusters=60)
+    sc = w.scene
+    img = np.zeros((96, 96, 3), np.float32)
+    visits = []
+    for verts in (sc.verts, _far(sc, distance)):
+        a = hr.hr_asset_create(ctx, sc.verts, sc.mat, sc.shape)
+        hr.hr_build_clusters(ctx, a, w.n_clusters)
+        C, L, _ = hr.hr_hierarchy_info(ctx, a)
+        lod = scenegen.lod_preset("strands", C, L)
+        if settled == "refit":
+            hr.hr_build_bvh(ctx, a, lod)
+        hr.hr_asset_update(ctx, a, verts)
+        flags = hr.HR_FLAG_COUNT
+        if settled == "built":
+            hr.hr_build_bvh(ctx, a, lod)
+            st = hr.hr_render(ctx, a, hr.render_desc(w.camera.pack(), w.lights, 2, 4, 7, 0, flags), img, stats=True)
+        else:
+            flags |= hr.HR_FLAG_REFIT | hr.HR_FLAG_KEEP_HIERARCHY
+            d = hr.render_desc(w.camera.pack(), w.lights, 2, 4, 7, 0, flags)
+            st = hr.hr_render_frame(ctx, a, 0, 0.0, 0, d, img, stats=True)
+        visits.append(st.node_visits / max(1, st.traced_samples))
+        hr.hr_asset_destroy(ctx, a)
+    print(settled, distance, visits)
+    assert 0 < visits[1] < 2 * visits[0]
