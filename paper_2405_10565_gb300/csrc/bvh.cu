@@ -791,6 +791,17 @@ __global__ void k_bytes_differ(const uint8_t* __restrict__ x, const uint8_t* __r
   if (i < n && x[i] != y[i]) *diff = 1u;
 }
 
+// Nodes that span blocks of 256 leaves, at most: each holds both leaves at some
+// boundary of two blocks, so it lies on the path from the root to their split,
+// along which the common prefix grows from one node to the next: by a bit of
+// the codes or, between equal codes, of the index.  (A slot for six leaves at
+// 5M leaves, where one for each would be 52 bytes a leaf.)
+size_t max_span_nodes(size_t n) {
+  size_t bits = kMortonBits;
+  while ((1ull << (bits - kMortonBits)) < n) ++bits;
+  return std::min(n - 1, ((n + 255) / 256 - 1) * bits);
+}
+
 // Every node's record over the topology in bv and the primitives `ids` in leaf
 // order, after scene_grid on the same stream.
 hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, cudaStream_t st) {
@@ -799,9 +810,10 @@ hr_status gather_refit(hr_ctx* ctx, hr_asset* a, Bvh& bv, const uint32_t* ids, c
   int *starts = nullptr, *span_node = nullptr;
   uint32_t* span = nullptr;
   HR_TRY(scratch(ctx, 39, 16, (void**)&counts));
-  HR_TRY(scratch(ctx, 46, (size_t)n * 13 * 4, (void**)&span));
+  const size_t slots = max_span_nodes(n);
+  HR_TRY(scratch(ctx, 46, slots * 13 * 4, (void**)&span));
   HR_TRY(scratch(ctx, 48, (size_t)n * 2 * 4, (void**)&starts));  // one per leaf and per node at most
-  span_node = reinterpret_cast<int*>(span + 12 * (size_t)n);
+  span_node = reinterpret_cast<int*>(span + 12 * slots);
   k_gather_refit<256><<<(n + 255) / 256, 256, 0, st>>>(bv.child, bv.par_int, bv.par_leaf,
                                                        a->prim_box, bv.frame, ids, (int)n, bv.nodes,
                                                        bv.leaf_id, counts, starts, span_node, span);
