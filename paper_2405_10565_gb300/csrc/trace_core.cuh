@@ -323,9 +323,15 @@ static __device__ __noinline__ bool refine(const FrameArgs& fa, const RayKey& rk
 // The K nearest hits: depth and entry word.  The entry word holds the
 // global primitive id (which also addresses the primitive's records; a thick
 // hair's chord is recomputed from them when it is shaded) and two flags:
-// kExact when the depth was decided precisely (t + tr is then a normalised
-// double-word depth) and kOpaque for a strand hit.  An FP32 entry has tr = 0.
-// Entries order by (t, tr, id).
+// kExact when the depth was decided precisely and kOpaque for a strand hit.
+// The depth is t + tr, with tr = 0 until it is decided precisely; entries order
+// by (depth, id).  Shading takes t.  So that t does not depend on the order of the
+// tests (frames repeat bit for bit whichever kernel finishes a ray), it is the
+// precise depth only where the hit needs one for its own sake, whatever else the
+// ray hits; where only the order against another hit did, t stays the FP32
+// depth and tr takes the rest.  (A light path starts at t + tr: it can cross a
+// hair or miss it by less than FP32's rounding, and frames with shadow rays put
+// no ray aside.)
 constexpr uint32_t kIdMask = 0x3fffffffu, kOpaque = 0x40000000u, kExact = 0x80000000u;
 constexpr uint32_t kNoEntry = kIdMask;  // an empty slot (t = inf)
 // The ray and its hits live in shared memory, a column per thread (no bank
@@ -374,7 +380,9 @@ __device__ __forceinline__ float3 ray_d(const RayMem<KMAX, COLS>& rm, uint32_t c
 
 __device__ __forceinline__ bool key_less(float t, float tr, uint32_t id, float t2, float tr2,
                                          uint32_t id2) {
-  return t < t2 || (t == t2 && (tr < tr2 || (tr == tr2 && (id & kIdMask) < (id2 & kIdMask))));
+  // t - t2 is exact where tr can matter; both infinite: no less
+  const float d = __fadd_rn(__fsub_rn(t, t2), __fsub_rn(tr, tr2));
+  return d < 0.f || (d == 0.f && (id & kIdMask) < (id2 & kIdMask));
 }
 
 // The entry (t, tr, id) into the sorted places 0 .. j, the last one's old
@@ -411,7 +419,7 @@ struct Counts {
 // (strand) hit.  An FP32 hit is kept as it is when its depth bound terr is
 // narrow, it is not near the outline or an end, and neither the cut nor any
 // entry lies within terr + errmax of it, errmax being the widest bound of the
-// FP32 entries kept so far: the FP32 entries are then pairwise further apart
+// entries whose t is an FP32 depth: these are then pairwise further apart
 // than the sum of their bounds, so their FP32 order is their true order.
 // Otherwise the hit is decided precisely, and so is every FP32 entry within
 // errmax of its precise depth (the only entries whose order against it the
@@ -423,33 +431,33 @@ __device__ __forceinline__ void keep_hit(const FrameArgs& fa, RayMem<KMAX, COLS>
   const uint32_t k = kbuf_depth<KMAX>(fa);
   const float slack = terr + errmax;
   const float s_off = rm.s_off[c];
-  bool need = r == kBorder || terr > kTieRel * (s_off + th) || th >= tcut - slack;
+  const bool own = r == kBorder || terr > kTieRel * (s_off + th);  // whatever else the ray hits
+  bool need = own || th >= tcut - slack;
   for (uint32_t j = 0; j < k; ++j) need |= fabsf(th - rm.t[j][c]) <= slack;
   uint32_t word = id | (id < fa.N * fa.S ? kOpaque : 0u);  // strand ids come first
   float tr = 0.f;
   if (need) {
     const RayKey rk{rm.sid[0][c] | (uint64_t)rm.sid[1][c] << 32, s_off};
     if (COUNT) ++cn.precise_tests;
-    float tl;
-    if (!refine(fa, rk, id, th, th, tl)) return;
-    tr = tl;
+    float h, l;
+    if (!refine(fa, rk, id, th, h, l)) {
+      if (own) return;
+      h = th, l = 0.f;  // not expected inside the FP32 bounds
+    }
+    const float depth = h;
+    if (own)
+      th = h, tr = l;
+    else
+      tr = __fadd_rn(__fsub_rn(h, th), l);
     word |= kExact;
     bool moved = false;
 #pragma unroll 1
     for (uint32_t j = 0; j < k; ++j) {
       const float t = rm.t[j][c];
-      if (t < kInf && !(rm.id[j][c] & kExact) && fabsf(th - t) <= errmax) {
-        float h, l;
+      if (t < kInf && !(rm.id[j][c] & kExact) && fabsf(depth - t) <= errmax) {
         if (COUNT) ++cn.precise_entries;
-        if (refine(fa, rk, rm.id[j][c] & kIdMask, t, h, l)) {
-          rm.t[j][c] = h;
-          rm.tr[j][c] = l;
-          rm.id[j][c] |= kExact;
-        } else {  // not expected for an FP32 hit inside its bounds; dropped if it happens
-          rm.t[j][c] = kInf;
-          rm.tr[j][c] = 0.f;
-          rm.id[j][c] = kNoEntry;
-        }
+        if (refine(fa, rk, rm.id[j][c] & kIdMask, t, h, l)) rm.tr[j][c] = __fadd_rn(__fsub_rn(h, t), l);
+        rm.id[j][c] |= kExact;
         moved = true;
       }
     }
@@ -457,9 +465,8 @@ __device__ __forceinline__ void keep_hit(const FrameArgs& fa, RayMem<KMAX, COLS>
 #pragma unroll 1
       for (uint32_t i = 1; i < k; ++i) kbuf_place(rm, c, (int)i, rm.t[i][c], rm.tr[i][c], rm.id[i][c]);
     }
-  } else {
-    errmax = fmaxf(errmax, terr);
   }
+  if (!own) errmax = fmaxf(errmax, terr);
   if (key_less(th, tr, word, rm.t[k - 1][c], rm.tr[k - 1][c], rm.id[k - 1][c]))
     kbuf_place(rm, c, (int)k - 1, th, tr, word);
   tcut = kbuf_cut(rm, c, k);
@@ -1094,16 +1101,17 @@ __device__ __forceinline__ void shade_hit(const FrameArgs& fa, uint32_t id, floa
 }
 
 // Shading and front-to-back compositing of a sample's hits (entry j's depth at
-// t[j * stride], its word at id[j * stride], nearest first).
+// t[j * stride], with SHADOW its low part at tr[j * stride], its word at
+// id[j * stride], nearest first).
 template <int PREC, bool COUNT, bool SHADOW>
-__device__ __forceinline__ void shade_hits(const FrameArgs& fa, const float* t, const uint32_t* id,
-                                           uint32_t stride, uint32_t k, const float3 o, const float3 d,
+__device__ __forceinline__ void shade_hits(const FrameArgs& fa, const float* t, const float* tr,
+                                           const uint32_t* id, uint32_t stride, uint32_t k, const float3 o, const float3 d,
                                            float out[3], Counts& cn) {
   out[0] = out[1] = out[2] = 0.f;
   float T = 1.f;
 #pragma unroll 1
   for (uint32_t j = 0; j < k; ++j) {
-    const float tj = t[j * stride];
+    const float tj = SHADOW ? __fadd_rn(t[j * stride], tr[j * stride]) : t[j * stride];
     if (!(tj < kInf && T > 0.f)) break;  // sorted by depth
     float rgb[3], a;
     shade_hit<PREC, COUNT, SHADOW>(fa, id[j * stride] & kIdMask, tj, o, d, rgb, a, cn);
@@ -1135,7 +1143,7 @@ __device__ __forceinline__ void render_sample(const FrameArgs& fa, RayMem<KMAX, 
   ok = traverse<KMAX, COUNT>(fa, rm, live, cn);
   out[0] = out[1] = out[2] = 0.f;
   if (live)
-    shade_hits<PREC, COUNT, SHADOW>(fa, &rm.t[0][c], &rm.id[0][c], kBlock, kbuf_depth<KMAX>(fa),
+    shade_hits<PREC, COUNT, SHADOW>(fa, &rm.t[0][c], &rm.tr[0][c], &rm.id[0][c], kBlock, kbuf_depth<KMAX>(fa),
                                     ray_o(rm, c), ray_d(rm, c), out, cn);
 }
 
@@ -1356,7 +1364,7 @@ __device__ __forceinline__ void render_warp_tile(const FrameArgs& fa, RayMem<KMA
     }
     float v[3] = {0.f, 0.f, 0.f};
     if (live && !((aside >> lane) & 1u))
-      shade_hits<PREC, COUNT, SHADOW>(fa, &rm.t[0][c], &rm.id[0][c], kBlock, kbuf_depth<KMAX>(fa),
+      shade_hits<PREC, COUNT, SHADOW>(fa, &rm.t[0][c], &rm.tr[0][c], &rm.id[0][c], kBlock, kbuf_depth<KMAX>(fa),
                                       ray_o(rm, c), ray_d(rm, c), v, cn);
     if (COUNT && live) ++cn.rays;
     overflow |= !w.ok;

@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kBlock, 6)
       tr::RayKey rk;
       float3 ro, rd;
       tr::primary_ray(fa, tl.pixel * fa.spp + (lane & (fa.grp - 1)), ro, rd, rk);
-      tr::shade_hits<PREC, false, false>(fa, t, id, 1u, k, ro, rd, acc, cn);
+      tr::shade_hits<PREC, false, false>(fa, t, nullptr, id, 1u, k, ro, rd, acc, cn);
     }
     tr::tile_write(fa, tl, acc, rgb);
   }

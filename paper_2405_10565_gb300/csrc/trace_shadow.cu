@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kBlock, tr::kTraceBlocks)
     reinterpret_cast<uint8_t*>(sw.tiles[rec].cnt)[lane] = (uint8_t)cnt;
     const uint32_t h0 = base + incl - cnt;
     for (uint32_t j = 0; j < cnt; ++j) {
-      const float t = rm.t[j][threadIdx.x];
+      const float t = __fadd_rn(rm.t[j][threadIdx.x], rm.tr[j][threadIdx.x]);
       const float3 x3 = tr::hit_point(tr::ray_o(rm, threadIdx.x), tr::ray_d(rm, threadIdx.x), t);
       sw.hit[h0 + j] = make_float4(x3.x, x3.y, x3.z, __uint_as_float(rm.id[j][threadIdx.x]));
       sw.depth[h0 + j] = t;
