@@ -644,8 +644,13 @@ struct Offs {
 // k through it in double-word FP32, whose weights differ from FP64 ones by
 // less than their final FP32 rounding.  Neighbouring threads read and write
 // neighbouring vertices.  255 us for 100k strands x 65 and 22k thick hairs;
-// FP64 prisms per point took 1.51 and 0.81 ms.
+// FP64 prisms per point took 1.51 and 0.81 ms.  A cluster's points are shared
+// out to gridDim.y blocks: few guides make few and large clusters (a build of
+// 100k strands with 3, 8 and 32 guides 134, 24.5 and 7.1 ms with a block a
+// cluster, 97, 20.2 and 6.2 shared out; 2.88 both ways with 256).
 constexpr uint32_t kWeightBlock = 256;
+constexpr uint32_t kWeightMembers = 64;   // strands a block takes, on average
+constexpr uint32_t kWeightBlocks = 1216;  // eight an SM
 __global__ void __launch_bounds__(kWeightBlock)
     k_prism_weights(const float4* __restrict__ verts, uint32_t S1,
                     const uint32_t* __restrict__ order, const uint32_t* __restrict__ cl_first,
@@ -653,16 +658,18 @@ __global__ void __launch_bounds__(kWeightBlock)
                     const float4* __restrict__ xsec, Offs lv, float4* w_strand, float4* w_eth) {
   const uint32_t c = blockIdx.x;
   const uint32_t lanes = max(1u, kWeightBlock / S1);  // points taken side by side
+  const uint32_t step = lanes * gridDim.y;
   uint32_t ga, gb, gc;
   tri_of(cl_tri[c], ga, gb, gc);
   const size_t r0 = (size_t)guides[ga] * S1, r1 = (size_t)guides[gb] * S1,
                r2 = (size_t)guides[gc] * S1;
   const uint32_t m0 = cl_first[c], m1 = cl_first[c + 1];
   for (uint32_t t = threadIdx.x; t < lanes * S1; t += kWeightBlock) {
-    const uint32_t k = t % S1, side = t / S1;
+    const uint32_t k = t % S1, side = t / S1 + lanes * blockIdx.y;
+    if (m0 + side >= m1 && (lv.n_levels == 0 || side >> (2 * (lv.n_levels - 1)))) continue;  // none left
     const Prism pr = make_prism(__ldg(verts + r0 + k), __ldg(verts + r1 + k), __ldg(verts + r2 + k));
     const float3 g0 = pr.g0;
-    for (uint32_t m = m0 + side; m < m1; m += lanes) {
+    for (uint32_t m = m0 + side; m < m1; m += step) {
       const size_t idx = (size_t)__ldg(order + m) * S1 + k;
       const float4 p = __ldg(verts + idx);
       const df q[3] = {df_diff(p.x, g0.x), df_diff(p.y, g0.y), df_diff(p.z, g0.z)};
@@ -670,7 +677,7 @@ __global__ void __launch_bounds__(kWeightBlock)
     }
     for (uint32_t l = 0; l < lv.n_levels; ++l) {
       const uint32_t sub = 1u << (2 * l), e0 = lv.off[l] + c * sub;
-      for (uint32_t j = side; j < sub; j += lanes) {
+      for (uint32_t j = side; j < sub; j += step) {
         const size_t idx = (size_t)(e0 + j) * S1 + k;
         const float4 x = xsec[idx * 3], y = xsec[idx * 3 + 1], z = xsec[idx * 3 + 2];
         float4* o = w_eth + idx * 5;
@@ -889,8 +896,11 @@ hr_status guided_build(hr_ctx* ctx, hr_asset* a, uint32_t G, uint32_t iters, uin
   Offs lv{};
   lv.n_levels = a->n_levels;
   for (uint32_t k = 0; k <= a->n_levels && k < 16; ++k) lv.off[k] = a->eth_offset[k];
-  k_prism_weights<<<C, kWeightBlock, 0, st>>>(a->verts, S1, a->order, a->cl_first, a->cl_tri, guides,
-                                              a->xsec, lv, a->w_strand, a->w_eth);
+  const uint32_t parts = std::min(
+      65535u, std::max(blocks_for(N / C, kWeightMembers), blocks_for(kWeightBlocks, C)));
+  k_prism_weights<<<dim3(C, parts), kWeightBlock, 0, st>>>(a->verts, S1, a->order, a->cl_first,
+                                                           a->cl_tri, guides, a->xsec, lv,
+                                                           a->w_strand, a->w_eth);
   HR_LAUNCHED(ctx);
   return HR_OK;
 }
