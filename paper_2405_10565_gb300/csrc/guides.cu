@@ -346,7 +346,8 @@ __global__ void __launch_bounds__(256)
 // Members that can be the medoid.  u = 2^-24; T and W are within (S1 3 / 32 +
 // 16) u of exact (the lanes' chains, their tree, the mean's two words), the
 // FP32 sums within (m + S1 + 8) u, each with a tenth on top; squares that
-// underflow add at most m S1 3 2^-148.  A mean off by delta moves s_i by at
+// underflow add at most m S1 3 2^-147.  Where the least sum may overflow (the
+// medoid is then the lowest id) every member stays a candidate.  A mean off by delta moves s_i by at
 // most 2 m |delta| sqrt(T); the sums of 64 ranks are within 2^-36 of their
 // terms' magnitudes (Sum2), so |delta| is below 2^-35 of the largest norm.
 __global__ void k_medoid_candidates(const uint32_t* __restrict__ key, uint32_t N, uint32_t S1,
@@ -361,8 +362,8 @@ __global__ void k_medoid_candidates(const uint32_t* __restrict__ key, uint32_t N
                       sqrt((double)__uint_as_float(mw.vmax[g]));
   const double lower = (m * t + W) * (1.0 - tau) * (1.0 - eps);
   const double upper = (m * tmin + W) * (1.0 + tau) * (1.0 + eps) + move +
-                       m * S1 * 3.0 * 2.802596928649634e-45;
-  if (lower > upper && eps < 0.5) return;  // NaN compares false: stays
+                       m * S1 * 3.0 * 5.605193857299268e-45;
+  if (lower > upper && upper < 3.4028234e38 && eps < 0.5) return;  // NaN compares false: stays
   mw.cand[atomicAdd(mw.n_cand, 1u)] = r;
 }
 
