@@ -84,7 +84,7 @@ uint32_t* ctx_overflow(hr_ctx* ctx) { return ctx->d_overflow; }
 // Gives back the scratch that frames can do without (the rays put aside, the
 // light paths of a shadow frame), so that it never stands in the way of
 // another allocation; false when there was none.
-static bool drop_optional_scratch(hr_ctx* ctx) {
+bool drop_optional_scratch(hr_ctx* ctx) {
   bool any = false;
   for (int slot : {kScratchPaths, kScratchLong}) {
     Scratch& s = ctx->scratch[slot];

@@ -127,6 +127,8 @@ void dfree(hr_ctx* ctx, void* p, size_t bytes);
 // frames can do without and are given back when an allocation needs the room
 constexpr int kScratchPaths = 17, kScratchLong = 18;
 hr_status scratch(hr_ctx* ctx, int slot, size_t bytes, void** p);
+// Gives these two back (holding the API lock); false when there was nothing to give.
+bool drop_optional_scratch(hr_ctx* ctx);
 
 #define HR_CUDA(ctx, call)                                                              \
   do {                                                                                  \

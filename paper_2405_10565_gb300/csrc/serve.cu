@@ -340,9 +340,11 @@ void loop(Server* s) {
         return need <= fr;
       };
       if (!fits()) {
-        // reclaim unreferenced resident BVHs and idle slots' buffers, retry
+        // reclaim what frames can do without, unreferenced resident BVHs and
+        // idle slots' buffers, retry
         std::lock_guard<std::recursive_mutex> g(ctx_mutex(ctx));
         cudaStreamSynchronize(s->stream);
+        drop_optional_scratch(ctx);
         evict(s, 0);
         for (size_t i = 0; i < s->slots.size(); ++i) {
           Slot& sl = s->slots[i];
