@@ -135,7 +135,8 @@ hr_status scratch(hr_ctx* ctx, int slot, size_t bytes, void** p) {
       s.p = nullptr;
       s.bytes = 0;
     }
-    size_t want = bytes + bytes / 4 + 256;
+    // room to grow, but for the light paths' slot, whose size has a bound of its own
+    const size_t want = slot == kScratchPaths ? bytes : bytes + bytes / 4 + 256;
     HR_TRY(dalloc(ctx, &s.p, want, "scratch"));
     s.bytes = want;
   }

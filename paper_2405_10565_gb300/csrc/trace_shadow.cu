@@ -12,8 +12,8 @@
 // neighbouring hits toward one light per warp, they fill the GPU: 4.5 ms, and
 // 4.1 with leaves waiting for one another as in the primary rays' walk.
 //
-// The hits of a round go to a buffer of at most kPathBudget light paths; the
-// primary kernel stops taking tiles once it is full and the next round goes on
+// The hits of a round and their paths go to buffers of kPathBytes at most; the
+// primary kernel stops taking tiles once they are full and the next round goes on
 // from there.  The host does not know how many rounds a frame needs without
 // waiting for it, so it launches up to kMaxRounds and, when the worst case
 // would need more, the one-kernel form for whatever tiles are left.
@@ -24,7 +24,7 @@
 namespace hr {
 namespace {
 
-constexpr uint64_t kPathBudget = 1ull << 24;  // 256 MB of path records
+constexpr uint64_t kPathBytes = 448ull << 20;  // 2.5M hits of 8 lights, 13M of one, beside those at work
 constexpr uint32_t kMaxRounds = 3;
 // A round costs about 25 us more than the one-kernel form where little is
 // walked (four launches in a row for one); that form walks a hit's paths one
@@ -47,7 +47,7 @@ struct ShadowWork {
   uint32_t* ctr;      // [0] hits, [1] tiles with hits (of the round)
   float4* hit;        // [cap] hit position and entry word (id, flags)
   float* depth;       // [cap] depth past the re-based origin
-  ShadowTile* tiles;  // [cap]
+  ShadowTile* tiles;  // [the frame's warp tiles, cap at most]
   float4* path;       // [lights][cap] (T rgb, spread variance)
   uint32_t stop;      // no further tile is taken at this many hits
   uint32_t cap;       // stop plus what the warps at work can still add
@@ -249,12 +249,18 @@ hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, 
       (uint64_t)fa.cam.W * fa.cam.H * fa.spp <= kOneKernelSamples)
     return HR_OK;
   const uint64_t worst = (uint64_t)fa.cam.W * fa.cam.H * fa.spp * fa.k;
-  const uint64_t stop = std::min<uint64_t>(worst, kPathBudget / L);
+  const uint64_t per_hit = sizeof(float4) + sizeof(float) + L * sizeof(float4);
+  const uint64_t cap = std::min<uint64_t>(worst, kPathBytes / per_hit);
   // every launched warp can be at a tile of 32 lanes and k hits when the round
   // fills up; nothing is added past the worst case
   const int g_hits = 4 * sm_count();
-  const uint64_t cap = std::min<uint64_t>(worst, stop + (uint64_t)g_hits * kBlock * fa.k);
-  const size_t bytes = 64 + cap * (sizeof(float4) + sizeof(ShadowTile) + sizeof(float) + L * sizeof(float4));
+  const uint64_t at_work = (uint64_t)g_hits * kBlock * fa.k;
+  if (cap < worst && cap <= at_work) return HR_OK;
+  const uint64_t stop = cap < worst ? cap - at_work : worst;
+  const WarpGrid all = warp_grid(make_float4(0.f, 0.f, (float)fa.cam.W, (float)fa.cam.H),
+                                 (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
+  const uint64_t tiles = std::min<uint64_t>(cap, all.n);
+  const size_t bytes = 64 + cap * per_hit + tiles * sizeof(ShadowTile);
   char* p = nullptr;
   if (scratch(ctx, kScratchPaths, bytes, (void**)&p) != HR_OK) {
     set_error(ctx, HR_OK, "");
@@ -264,7 +270,7 @@ hr_status launch_shadow_rounds(hr_ctx* ctx, const FrameArgs& fa, int precision, 
   sw.path = reinterpret_cast<float4*>(p);
   sw.hit = sw.path + L * cap;
   sw.tiles = reinterpret_cast<ShadowTile*>(sw.hit + cap);
-  sw.depth = reinterpret_cast<float*>(sw.tiles + cap);
+  sw.depth = reinterpret_cast<float*>(sw.tiles + tiles);
   sw.ctr = reinterpret_cast<uint32_t*>(sw.depth + cap);
   sw.stop = (uint32_t)stop;
   sw.cap = (uint32_t)cap;
