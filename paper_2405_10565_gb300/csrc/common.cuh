@@ -104,6 +104,7 @@ struct hr_asset {
   float4* w_eth = nullptr;        // [E * (S + 1) * 5] of thick-hair centres and corners
   uint32_t guided_C = 0, guided_E = 0;  // shape the weights were taken for
   bool radii_old = false;  // vertices (and radii) were given since the thick hairs took their radii
+  bool eth_bounds = false;  // d_bounds holds thick hairs' bounds
   // frame-kernel schedule carried between frames (TileSched)
   hr::TileSched* sched = nullptr;
 };
@@ -232,6 +233,8 @@ hr_status build_hierarchy_from(hr_ctx* ctx, hr_asset* a, uint32_t C, uint32_t ma
 // skin_strands on the same stream (their radii are taken again where
 // hr_asset_update has given vertices since they were; their materials stay).
 hr_status skin_strands(hr_ctx* ctx, hr_asset* a, const float4* gv);
+// No thick-hair bounds (kEthBounds), before records that widen them or for none.
+hr_status clear_eth_bounds(hr_ctx* ctx, hr_asset* a);
 hr_status moved_eth_records(hr_ctx* ctx, hr_asset* a);
 
 // The three guides (10 bits each) of a cluster.

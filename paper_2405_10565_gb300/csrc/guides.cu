@@ -940,6 +940,7 @@ hr_status skin_asset(hr_ctx* ctx, hr_asset* a, const float4* gv_dev) {
                                                                      a->cl_tri, a->w_strand, a->verts);
     HR_LAUNCHED(ctx);
     HR_TRY(refresh_strand_prims(ctx, a));
+    HR_TRY(clear_eth_bounds(ctx, a));
   }
   if (a->E) {
     Offs lv{};

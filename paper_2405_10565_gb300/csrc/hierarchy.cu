@@ -1063,8 +1063,7 @@ hr_status build_strand_prims(hr_ctx* ctx, hr_asset* a) {
   HR_TRY(dalloc(ctx, (void**)&a->prim_wa, n * 2 * sizeof(float4), "strand aux"));
   HR_TRY(dalloc(ctx, (void**)&a->d_bounds, kBoundWords * sizeof(uint32_t), "scene bounds"));
   a->bytes += n * 6 * sizeof(float4);
-  k_init_bounds<<<1, 32, 0, ctx_stream(ctx)>>>(a->d_bounds + kEthBounds);  // no thick hairs yet
-  HR_LAUNCHED(ctx);
+  HR_TRY(clear_eth_bounds(ctx, a));
   return refresh_strand_prims(ctx, a);
 }
 
@@ -1101,6 +1100,13 @@ hr_status skin_strands(hr_ctx* ctx, hr_asset* a, const float4* gv) {
   HR_LAUNCHED(ctx);
   return launch_strand_update(
       ctx, a, SkinnedVerts{gv, a->w_strand, a->verts, a->cluster_of, a->cl_tri, a->S + 1}, st);
+}
+
+hr_status clear_eth_bounds(hr_ctx* ctx, hr_asset* a) {
+  k_init_bounds<<<1, 32, 0, ctx_stream(ctx)>>>(a->d_bounds + kEthBounds);
+  HR_LAUNCHED(ctx);
+  a->eth_bounds = false;
+  return HR_OK;
 }
 
 hr_status refresh_strand_prims(hr_ctx* ctx, hr_asset* a) {
@@ -1227,6 +1233,7 @@ hr_status hierarchy_finish(hr_ctx* ctx, hr_asset* a, const LevelInfo& li, uint64
       HR_CUDA(ctx, cudaEventRecord(ctx_fit_event(ctx), sf));
       HR_CUDA(ctx, cudaStreamWaitEvent(st, ctx_fit_event(ctx), 0));
     }
+    if (a->eth_bounds) HR_TRY(clear_eth_bounds(ctx, a));  // an earlier hierarchy's
     return HR_OK;
   }
 
@@ -1253,6 +1260,7 @@ hr_status hierarchy_finish(hr_ctx* ctx, hr_asset* a, const LevelInfo& li, uint64
       a->d_bounds + kEthBounds);
   HR_LAUNCHED(ctx);
   a->radii_old = false;
+  a->eth_bounds = true;
   const uint64_t ne = E * S;
   k_eth_prims<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(a->xsec, N, S, (uint32_t)E,
                                                            a->cl_first, li, eth_r, a->prim_uv,
@@ -1325,6 +1333,7 @@ hr_status moved_eth_records(hr_ctx* ctx, hr_asset* a) {
     HR_LAUNCHED(ctx);
     a->radii_old = false;
   }
+  a->eth_bounds = true;
   k_eth_prims<<<(unsigned)(((uint64_t)E * S + 255) / 256), 256, 0, st>>>(
       a->xsec, a->N, S, E, a->cl_first, li, eth_r, a->prim_uv, a->prim_box, a->prim_wa,
       a->d_bounds + kEthBounds);
