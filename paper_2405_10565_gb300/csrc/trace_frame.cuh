@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(kRectThreads) k_scene_rect(const FrameArgs fa,
   if (fa.lw.words && threadIdx.x < 4) fa.lw.ctr[threadIdx.x] = 0u;
   TileSched* sc = fa.sched;
   if (!sc) return;
-  __shared__ uint32_t s_hist[256], s_cut, s_n;
+  __shared__ uint32_t s_hist[256], s_cut, s_n, s_kept;
   __shared__ uint32_t s_tile[kHeavyMax], s_steps[kHeavyMax];
   const uint32_t tid = threadIdx.x;
   const bool have = sc->prev_n > 0 && sc->prev_W == (uint32_t)fa.cam.W &&
@@ -80,18 +80,26 @@ __global__ void __launch_bounds__(kRectThreads) k_scene_rect(const FrameArgs fa,
     }
     __syncthreads();
   }
-  const uint32_t nh = min(s_n, kHeavyMax);
-  if (tid < nh) {  // heaviest first (ties by tile index): rank by counting
-    uint32_t r = 0;
-    for (uint32_t k = 0; k < nh; ++k)
-      r += s_steps[k] > s_steps[tid] || (s_steps[k] == s_steps[tid] && s_tile[k] < s_tile[tid]);
-    const WarpGrid pg = warp_grid(sc->prev_rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
-    const uint32_t t = s_tile[tid];
-    sc->heavy[r] = (pg.x0 + (t % pg.nx) * pg.wtw) | ((pg.y0 + (t / pg.nx) * pg.wth) << 16);
+  const uint32_t listed = min(s_n, kHeavyMax);
+  if (tid < 32) {
+    // a tile listed several times (by parts of it) stays with its heaviest part
+    bool stays = tid < listed;
+    const uint32_t t = stays ? s_tile[tid] : 0u, steps = stays ? s_steps[tid] : 0u;
+    for (uint32_t k = 0; k < listed; ++k)
+      if (s_tile[k] == t && (s_steps[k] > steps || (s_steps[k] == steps && k < tid))) stays = false;
+    const unsigned heavy = __ballot_sync(0xffffffffu, stays);
+    if (stays) {  // heaviest first (ties by tile index): rank by counting
+      uint32_t r = 0;
+      for (uint32_t k = 0; k < listed; ++k)
+        r += ((heavy >> k) & 1u) && (s_steps[k] > steps || (s_steps[k] == steps && s_tile[k] < t));
+      const WarpGrid pg = warp_grid(sc->prev_rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
+      sc->heavy[r] = (pg.x0 + (t % pg.nx) * pg.wtw) | ((pg.y0 + (t / pg.nx) * pg.wth) << 16);
+    }
+    if (tid == 0) s_kept = (uint32_t)__popc(heavy);
   }
   __syncthreads();  // the previous frame's candidates and grid are no longer read
   if (tid == 0) {
-    sc->n_heavy = nh;
+    sc->n_heavy = s_kept;
     sc->grp = fa.grp;
     sc->thresh = lo;
     sc->max_steps = 0u;
@@ -172,8 +180,8 @@ __global__ void __launch_bounds__(kBlock, SHADOW ? 1 : tr::kTraceBlocks)
       x0 = xy & 0xffffu, y0 = xy >> 16;
       const uint32_t gx = (x0 - g.x0) / g.wtw, gy = (y0 - g.y0) / g.wth;
       if (x0 < g.x0 || y0 < g.y0 || (x0 - g.x0) % g.wtw || (y0 - g.y0) % g.wth || gx >= g.nx ||
-          gy * g.nx + gx >= g.n || __any_sync(0xffffffffu, lane < t && sc->heavy[lane] == xy))
-        continue;  // (or, from two of its parts, listed twice)
+          gy * g.nx + gx >= g.n)
+        continue;
       t = gy * g.nx + gx;
     } else {
       t -= nh;
