@@ -69,15 +69,15 @@ constexpr size_t kFrameWords = 7;
 //    hairs' boxes: low corner (two steps below the bounds; its fourth word says
 //    whether the nodes are in FP32), step, 1 / step.
 //  * The centroid codes' low corner and 1 / extent.
-// A whole block of WARPS warps calls it.
+// The whole block calls it, R boxes of strand segments a thread (count in all).
 // The grid resolves a scene whose boxes are many steps long; one far vertex or
 // parts of very different scale make it so coarse that neighbouring boxes
-// become the same, and so does the codes' cell.  So the block looks at 1,024
-// strand segments, spread evenly (and not in step with the strands): where more than one in kCoarsePart is not
-// kFineSteps steps long in any axis, or the bounds are not finite, the nodes are
-// in FP32, and the codes spread over the bulk of the segments instead of the
-// bounds: of 32 groups of 32 the 25th least minimum and the 25th greatest
-// maximum (three groups in four may hold far ones) and half as much on each side.
+// become the same, and so does the codes' cell.  So where more than one of these
+// segments in kCoarsePart is not kFineSteps steps long in any axis, or the bounds
+// are not finite, the nodes are in FP32, and the codes spread over the bulk of the
+// segments instead of the bounds: from the 25th least minimum of the lanes' 32
+// groups to their 25th greatest maximum (three groups in four may hold far ones)
+// and half as much on each side.
 // BVH and image, us a frame of 100k strands, one vertex put ever farther away,
 // on the grid / in FP32 by the steps of the median segment: a close view at 202
 // steps 3,692 / 3,821, at 113 3,844 / 3,820, at 60 4,080 / 3,814, at 16 5,577 /
@@ -85,19 +85,12 @@ constexpr size_t kFrameWords = 7;
 // 1,626, at 16 1,709 / 1,631, at 1 4,979 / 1,623.
 constexpr float kFineSteps = 64.f;
 constexpr uint32_t kCoarsePart = 8;
-template <int WARPS>
-__device__ __forceinline__ void scene_grid(const uint32_t* __restrict__ bounds,
-                                           const float4* __restrict__ box, uint32_t n, float4* frame,
-                                           unsigned* counts) {
+template <int R>
+__device__ __forceinline__ void scene_grid(const uint32_t* __restrict__ bounds, const float4 (&l)[R],
+                                           const float4 (&h)[R], bool has, uint32_t count,
+                                           float4* frame, unsigned* counts) {
   __shared__ uint32_t s_coarse, s_lo[3][32], s_hi[3][32];
-  constexpr int R = 32 / WARPS;  // groups a warp takes
-  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float4 l[R], h[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const size_t at = __umulhi(((w * R + r) * 32 + lane) * 2654435769u, n);  // golden-ratio steps
-    l[r] = box[2 * at], h[r] = box[2 * at + 1];
-  }
+  const uint32_t lane = threadIdx.x & 31;
   if (threadIdx.x == 0) s_coarse = 0u;
   __syncthreads();
   float lo[3], hi[3], st[3], clo[3], cinv[3];
@@ -118,38 +111,40 @@ __device__ __forceinline__ void scene_grid(const uint32_t* __restrict__ bounds,
   for (int r = 0; r < R; ++r) {
     const bool fine = h[r].x - l[r].x >= kFineSteps * st[0] || h[r].y - l[r].y >= kFineSteps * st[1] ||
                       h[r].z - l[r].z >= kFineSteps * st[2];
-    coarse += __popc(__ballot_sync(0xffffffffu, !fine));
+    coarse += __popc(__ballot_sync(0xffffffffu, has && !fine));
   }
   if (lane == 0 && coarse) atomicAdd(&s_coarse, coarse);
   __syncthreads();
   const bool finite = fabsf(lo[0] + lo[1] + lo[2]) + st[0] + st[1] + st[2] < __int_as_float(0x7f800000);
-  const bool wide = s_coarse * kCoarsePart > 1024u || !finite;
+  const bool wide = s_coarse * kCoarsePart > count || !finite;
   if (wide) {
+    if (threadIdx.x < 32)
+      for (int i = 0; i < 3; ++i) s_lo[i][lane] = 0xffffffffu, s_hi[i][lane] = 0u;
+    __syncthreads();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const float c[3] = {0.5f * (l[r].x + h[r].x), 0.5f * (l[r].y + h[r].y), 0.5f * (l[r].z + h[r].z)};
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const uint32_t a = __reduce_min_sync(0xffffffffu, low_bits(c[i]));
-        const uint32_t b = __reduce_max_sync(0xffffffffu, high_bits(c[i]));
-        if (lane == 0) s_lo[i][w * R + r] = a, s_hi[i][w * R + r] = b;
+      for (int i = 0; has && i < 3; ++i) {
+        atomicMin(&s_lo[i][lane], low_bits(c[i]));
+        atomicMax(&s_hi[i][lane], high_bits(c[i]));
       }
     }
     __syncthreads();
+    const uint32_t groups = min(32u, count), rank = groups * 3 / 4;
     for (int i = 0; i < 3; ++i) {
-      uint32_t a = 0, b = 0;  // the group whose minimum, maximum is the 25th
-      for (uint32_t g = 0; g < 32; ++g) {
+      uint32_t a = 0, b = 0;
+      for (uint32_t g = 0; g < groups; ++g) {
         uint32_t ra = 0, rb = 0;
-        for (uint32_t q = 0; q < 32; ++q) {
+        for (uint32_t q = 0; q < groups; ++q) {
           ra += s_lo[i][q] < s_lo[i][g] || (s_lo[i][q] == s_lo[i][g] && q < g);
           rb += s_hi[i][q] > s_hi[i][g] || (s_hi[i][q] == s_hi[i][g] && q < g);
         }
-        if (ra == 24) a = g;
-        if (rb == 24) b = g;
+        if (ra == rank) a = g;
+        if (rb == rank) b = g;
       }
-      const float l = from_ordered(s_lo[i][a]), h = from_ordered(s_hi[i][b]), e = h - l;
+      const float l0 = from_ordered(s_lo[i][a]), h0 = from_ordered(s_hi[i][b]), e = h0 - l0;
       const bool some = e > 0.f && e < 1e38f;
-      clo[i] = some ? fmaf(-0.5f, e, l) : 0.f;
+      clo[i] = some ? fmaf(-0.5f, e, l0) : 0.f;
       cinv[i] = some ? 0.5f / e : 0.f;
     }
   }
@@ -164,10 +159,25 @@ __device__ __forceinline__ void scene_grid(const uint32_t* __restrict__ bounds,
   if (counts) counts[0] = counts[1] = 0u;
 }
 
-__global__ void __launch_bounds__(256)
+// The same from 1,024 of the n strand segments, spread evenly and not in step
+// with the strands, by a block of 256.
+constexpr uint32_t kGridBlock = 256;
+__device__ __forceinline__ void sample_grid(const uint32_t* __restrict__ bounds,
+                                            const float4* __restrict__ box, uint32_t n, float4* frame,
+                                            unsigned* counts) {
+  float4 l[4], h[4];
+#pragma unroll
+  for (uint32_t r = 0; r < 4; ++r) {
+    const size_t at = __umulhi((r * kGridBlock + threadIdx.x) * 2654435769u, n);  // golden-ratio steps
+    l[r] = box[2 * at], h[r] = box[2 * at + 1];
+  }
+  scene_grid<4>(bounds, l, h, true, 1024, frame, counts);
+}
+
+__global__ void __launch_bounds__(kGridBlock)
     k_scene_grid(const uint32_t* __restrict__ bounds, const float4* __restrict__ box, uint32_t n,
                  float4* frame, unsigned* counts) {
-  scene_grid<8>(bounds, box, n, frame, counts);
+  sample_grid(bounds, box, n, frame, counts);
 }
 
 __global__ void __launch_bounds__(256, 8) k_cluster_fill(const uint8_t* __restrict__ lod, const uint32_t* __restrict__ cl_first,
@@ -177,7 +187,7 @@ __global__ void __launch_bounds__(256, 8) k_cluster_fill(const uint8_t* __restri
                                const uint32_t* __restrict__ bounds, const float4* __restrict__ box,
                                float4* frame, unsigned* counts) {
   if (blockIdx.x == 0) {
-    scene_grid<8>(bounds, box, N * S, frame, counts);
+    sample_grid(bounds, box, N * S, frame, counts);
     return;
   }
   const uint32_t c = blockIdx.x - 1;
@@ -209,7 +219,7 @@ __global__ void __launch_bounds__(256, 8) k_cluster_fill(const uint8_t* __restri
 __global__ void __launch_bounds__(256, 8) k_iota(uint32_t* ids, uint32_t n, const uint32_t* __restrict__ bounds,
                        const float4* __restrict__ box, float4* frame, unsigned* counts) {
   if (blockIdx.x == 0) {
-    scene_grid<8>(bounds, box, n, frame, counts);
+    sample_grid(bounds, box, n, frame, counts);
     return;
   }
   const uint32_t i = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
@@ -702,17 +712,20 @@ struct SmallBvh {
   float4 frame[kFrameWords];
 };
 __global__ void __launch_bounds__(kSmallLeaves)
-    k_small_bvh(const float4* __restrict__ box, const uint32_t* __restrict__ ids, int n, uint32_t NS,
+    k_small_bvh(const float4* __restrict__ box, const uint32_t* __restrict__ ids, int n,
                 const uint32_t* __restrict__ bounds, float4* frame, int4* child, int* parent_int,
                 int* parent_leaf, uint32_t* leaf_id, uint4* nodes) {
   __shared__ SmallBvh sm;
   const int j = threadIdx.x, lane = j & 31, w = j >> 5;
   const uint32_t lt = (1u << lane) - 1u;
-  scene_grid<kSmallWarps>(bounds, box, NS, sm.frame, nullptr);
-  __syncthreads();
   const bool valid = j < n;
   uint32_t id = valid ? (ids ? ids[j] : (uint32_t)j) : 0u, key = 0u;
-  if (valid) key = prim_code(box[2 * (size_t)id], box[2 * (size_t)id + 1], sm.frame);
+  {
+    const float4 l[1] = {box[2 * (size_t)id]}, h[1] = {box[2 * (size_t)id + 1]};
+    scene_grid<1>(bounds, l, h, valid, (uint32_t)n, sm.frame, nullptr);
+    __syncthreads();
+    if (valid) key = prim_code(l[0], h[0], sm.frame);
+  }
   for (int shift = 0; shift < kMortonBits; shift += 8) {
     for (int i = j; i < kSmallWarps * 256; i += kSmallLeaves) (&sm.whist[0][0])[i] = 0;
     __syncthreads();
@@ -936,7 +949,7 @@ hr_status build_bvh(hr_ctx* ctx, hr_asset* a, const uint8_t* lod_dev, Bvh& bv, c
     return HR_OK;
   }
   if (small) {  // all in one block
-    k_small_bvh<<<1, kSmallLeaves, 0, st>>>(a->prim_box, ids, (int)n, N * S, a->d_bounds, bv.frame, bv.child,
+    k_small_bvh<<<1, kSmallLeaves, 0, st>>>(a->prim_box, ids, (int)n, a->d_bounds, bv.frame, bv.child,
                                             bv.par_int, bv.par_leaf, bv.leaf_id, bv.nodes);
     HR_LAUNCHED(ctx);
     bv.valid = 1;
