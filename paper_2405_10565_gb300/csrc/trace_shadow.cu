@@ -16,7 +16,10 @@
 // primary kernel stops taking tiles once they are full and the next round goes on
 // from there.  The host does not know how many rounds a frame needs without
 // waiting for it, so it launches up to kMaxRounds and, when the worst case
-// would need more, the one-kernel form for whatever tiles are left.
+// would need more, the one-kernel form for whatever tiles are left: a close view
+// of the same head (6.4M traced samples) does not fit in the rounds and takes 34
+// ms with 8 lights and 70 with 16, a middle view with 8 lights 12 (56, 118 and 21
+// with the paths walked in the shading loop throughout).
 #include <algorithm>
 
 #include "trace_frame.cuh"
