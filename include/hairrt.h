@@ -318,7 +318,8 @@ hr_status hr_guides_export(hr_ctx* ctx, hr_asset* asset, int32_t* guides_out,
  * [n_guides][n_segments + 1][4] floats (host or device; xyz of the guide
  * strand of every k-means cluster, w ignored, rows of empty clusters
  * unused) carry every strand vertex and every thick-hair cross-section
- * centre and corner by its weights (FP32; the radius is kept); a
+ * centre and corner by its weights (FP32; the strands' radii are kept, the
+ * thick hairs' are their members' mean, also after hr_asset_update); a
  * cross-section's a and e1 come from its skinned corners c +- a e1, b and e2
  * from c +- b e2; the strand and thick-hair records are rebuilt, the
  * clustering and the fits are not.  Render with HR_FLAG_KEEP_HIERARCHY.
