@@ -83,15 +83,21 @@ __global__ void __launch_bounds__(kRectThreads) k_scene_rect(const FrameArgs fa,
   const uint32_t listed = min(s_n, kHeavyMax);
   if (tid < 32) {
     // a tile listed several times (by parts of it) stays with its heaviest part
-    bool stays = tid < listed;
-    const uint32_t t = stays ? s_tile[tid] : 0u, steps = stays ? s_steps[tid] : 0u;
-    for (uint32_t k = 0; k < listed; ++k)
-      if (s_tile[k] == t && (s_steps[k] > steps || (s_steps[k] == steps && k < tid))) stays = false;
+    const bool mine_listed = tid < listed;
+    const uint32_t t = mine_listed ? s_tile[tid] : 0u, steps = mine_listed ? s_steps[tid] : 0u;
+    bool stays = mine_listed;
+    uint32_t kt[kHeavyMax], ks[kHeavyMax];
+#pragma unroll
+    for (uint32_t k = 0; k < kHeavyMax; ++k) {
+      kt[k] = __shfl_sync(0xffffffffu, t, k), ks[k] = __shfl_sync(0xffffffffu, steps, k);
+      if (k < listed && kt[k] == t && (ks[k] > steps || (ks[k] == steps && k < tid))) stays = false;
+    }
     const unsigned heavy = __ballot_sync(0xffffffffu, stays);
     if (stays) {  // heaviest first (ties by tile index): rank by counting
       uint32_t r = 0;
-      for (uint32_t k = 0; k < listed; ++k)
-        r += ((heavy >> k) & 1u) && (s_steps[k] > steps || (s_steps[k] == steps && s_tile[k] < t));
+#pragma unroll
+      for (uint32_t k = 0; k < kHeavyMax; ++k)
+        r += ((heavy >> k) & 1u) && (ks[k] > steps || (ks[k] == steps && kt[k] < t));
       const WarpGrid pg = warp_grid(sc->prev_rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
       sc->heavy[r] = (pg.x0 + (t % pg.nx) * pg.wtw) | ((pg.y0 + (t / pg.nx) * pg.wth) << 16);
     }
