@@ -86,18 +86,19 @@ __global__ void __launch_bounds__(kRectThreads) k_scene_rect(const FrameArgs fa,
     const bool mine_listed = tid < listed;
     const uint32_t t = mine_listed ? s_tile[tid] : 0u, steps = mine_listed ? s_steps[tid] : 0u;
     bool stays = mine_listed;
-    uint32_t kt[kHeavyMax], ks[kHeavyMax];
-#pragma unroll
+#pragma unroll 4
     for (uint32_t k = 0; k < kHeavyMax; ++k) {
-      kt[k] = __shfl_sync(0xffffffffu, t, k), ks[k] = __shfl_sync(0xffffffffu, steps, k);
-      if (k < listed && kt[k] == t && (ks[k] > steps || (ks[k] == steps && k < tid))) stays = false;
+      const uint32_t kt = __shfl_sync(0xffffffffu, t, k), ks = __shfl_sync(0xffffffffu, steps, k);
+      if (k < listed && kt == t && (ks > steps || (ks == steps && k < tid))) stays = false;
     }
     const unsigned heavy = __ballot_sync(0xffffffffu, stays);
-    if (stays) {  // heaviest first (ties by tile index): rank by counting
-      uint32_t r = 0;
-#pragma unroll
-      for (uint32_t k = 0; k < kHeavyMax; ++k)
-        r += ((heavy >> k) & 1u) && (ks[k] > steps || (ks[k] == steps && kt[k] < t));
+    uint32_t r = 0;  // heaviest first (ties by tile index): rank by counting
+#pragma unroll 4
+    for (uint32_t k = 0; k < kHeavyMax; ++k) {
+      const uint32_t kt = __shfl_sync(0xffffffffu, t, k), ks = __shfl_sync(0xffffffffu, steps, k);
+      r += ((heavy >> k) & 1u) && (ks > steps || (ks == steps && kt < t));
+    }
+    if (stays) {
       const WarpGrid pg = warp_grid(sc->prev_rect, (uint32_t)fa.cam.W, (uint32_t)fa.cam.H, fa.grp);
       sc->heavy[r] = (pg.x0 + (t % pg.nx) * pg.wtw) | ((pg.y0 + (t / pg.nx) * pg.wth) << 16);
     }
