@@ -341,20 +341,31 @@ void loop(Server* s) {
       };
       if (!fits()) {
         // reclaim what frames can do without, unreferenced resident BVHs and
-        // idle slots' buffers, retry
-        std::lock_guard<std::recursive_mutex> g(ctx_mutex(ctx));
-        cudaStreamSynchronize(s->stream);
-        drop_optional_scratch(ctx);
-        evict(s, 0);
-        for (size_t i = 0; i < s->slots.size(); ++i) {
-          Slot& sl = s->slots[i];
-          if (sl.busy || (int)i == slot) continue;
-          if (sl.lod) dfree(ctx, sl.lod, sl.lod_cap);
-          if (sl.out) dfree(ctx, sl.out, sl.out_cap);
-          sl.lod = nullptr;
-          sl.out = nullptr;
-          sl.lod_cap = 0;
-          sl.out_cap = 0;
+        // idle slots' buffers, retry.  API calls take the API lock first and the
+        // server's after it (serve_forget_asset): never the other way round.  The
+        // slots and the BVHs' references change on this thread alone, the list of
+        // BVHs under the API lock.
+        lk.unlock();
+        {
+          std::lock_guard<std::recursive_mutex> g(ctx_mutex(ctx));
+          cudaStreamSynchronize(s->stream);
+          drop_optional_scratch(ctx);
+          evict(s, 0);
+          for (size_t i = 0; i < s->slots.size(); ++i) {
+            Slot& sl = s->slots[i];
+            if (sl.busy || (int)i == slot) continue;
+            if (sl.lod) dfree(ctx, sl.lod, sl.lod_cap);
+            if (sl.out) dfree(ctx, sl.out, sl.out_cap);
+            sl.lod = nullptr;
+            sl.out = nullptr;
+            sl.lod_cap = 0;
+            sl.out_cap = 0;
+          }
+        }
+        lk.lock();
+        if (s->pending.empty() || s->pending.front() != r) {  // cancelled meanwhile
+          progressed = true;
+          continue;
         }
         need = estimate_bytes(r, s->slots[slot]);
       }
