@@ -41,6 +41,7 @@ struct hr_ctx {
   // the kind of the last API call, as set by it (0 any other, kFrameCall,
   // kUpdateCall a pipelined hr_asset_update) and as seen by the current call
   int call_kind = 0, prev_kind = 0;
+  uint64_t api_calls = 0;  // calls so far that may have left work on the stream
   // frame-time ring: per hr_render_frame, events around the fit and the frame
   static constexpr int kRing = 256;
   cudaEvent_t ring[kRing][4] = {};
@@ -74,6 +75,8 @@ double ctx_now_ms(hr_ctx* ctx) {
 }
 
 int ctx_device(hr_ctx* ctx) { return ctx->device; }
+
+uint64_t ctx_api_calls(hr_ctx* ctx) { return ctx->api_calls; }
 
 Server** ctx_server_slot(hr_ctx* ctx) { return &ctx->server; }
 
@@ -250,7 +253,8 @@ struct DeviceGuard {
   std::lock_guard<std::recursive_mutex> api_lock_((ctx)->api_mu);        \
   DeviceGuard dev_guard_((ctx)->device);                                 \
   (ctx)->prev_kind = (ctx)->call_kind;                                   \
-  (ctx)->call_kind = 0
+  (ctx)->call_kind = 0;                                                  \
+  ++(ctx)->api_calls
 
 }  // namespace
 

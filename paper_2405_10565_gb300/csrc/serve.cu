@@ -97,6 +97,8 @@ struct Server {
   uint32_t* d_work = nullptr;
   cudaEvent_t batch_ev[2] = {nullptr, nullptr};
   cudaEvent_t ref_ev = nullptr;
+  cudaEvent_t api_ev = nullptr;  // the API stream's work that an admission waits for
+  uint64_t api_seen = 0;         // API calls whose work the build stream has waited for
   double ref_ms = 0;
   int buf = 0;
   uint32_t max_items = 0;
@@ -189,6 +191,13 @@ hr_status admit(Server* s, Request* r) {
   cudaStream_t bs = s->build_stream;
   Slot& sl = s->slots[r->slot];
   hr_asset* a = r->req.asset;
+  // API calls may return before their work is done: the asset's records may
+  // still be written, and the scratch that a build uses be in use
+  if (s->api_seen != ctx_api_calls(ctx)) {
+    HR_CUDA(ctx, cudaEventRecord(s->api_ev, ctx_stream(ctx)));
+    HR_CUDA(ctx, cudaStreamWaitEvent(bs, s->api_ev, 0));
+    s->api_seen = ctx_api_calls(ctx);
+  }
   const uint8_t* lod = nullptr;
   std::vector<uint8_t> lod_h;
   if (a->n_levels > 0) {
@@ -538,6 +547,7 @@ hr_status hr_serve_start(hr_ctx* ctx, uint32_t max_slots, uint64_t max_batch_sam
   }
   ok = ok && dalloc(ctx, (void**)&s->d_work, 16, "serve work") == HR_OK;
   ok = ok && cudaEventCreate(&s->ref_ev) == cudaSuccess;
+  ok = ok && cudaEventCreateWithFlags(&s->api_ev, cudaEventDisableTiming) == cudaSuccess;
   if (ok) {
     cudaEventRecord(s->ref_ev, s->stream);
     cudaEventSynchronize(s->ref_ev);
@@ -590,6 +600,7 @@ hr_status hr_serve_stop(hr_ctx* ctx) {
   }
   if (s->d_work) dfree(ctx, s->d_work, 16);
   if (s->ref_ev) cudaEventDestroy(s->ref_ev);
+  if (s->api_ev) cudaEventDestroy(s->api_ev);
   if (s->stream) cudaStreamDestroy(s->stream);
   if (s->build_stream) cudaStreamDestroy(s->build_stream);
   delete s;

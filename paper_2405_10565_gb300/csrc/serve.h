@@ -12,6 +12,7 @@ struct Server;
 std::recursive_mutex& ctx_mutex(hr_ctx* ctx);
 double ctx_now_ms(hr_ctx* ctx);
 int ctx_device(hr_ctx* ctx);
+uint64_t ctx_api_calls(hr_ctx* ctx);
 uint32_t* ctx_overflow(hr_ctx* ctx);
 bool is_device_ptr(const void* p);
 hr_status check_desc(hr_ctx* ctx, const hr_render_desc* d);
